@@ -60,12 +60,9 @@ extern "C" {
  * evaluate the wall diagnostics (Eqs. 7, 8) with correctly rounded division and
  * square root, as the generic diagnostic kernel does, instead of the fast kernels'
  * hardware reciprocal square root and approximate division.  The leapfrog step has
- * no division or square root: with one step per pass (tblock = 1) the fields are
- * bit-identical with and without the flag (prs_step_measure's diagnostics then run as
- * a separate pass, which can change how later steps group into two-step passes).
+ * no division or square root: the fields are bit-identical with and without the flag.
  * Sec. III compares single precision with and without correctly rounded divide and
  * square root.
- * prs_step_measure then runs the diagnostics and the steps as separate passes.
  * Ensembles (prs_batch_create) reject it. */
 #define PRS_FP32_CR 2u
 /* Checks after every call that queues work (slower; for development):
@@ -188,11 +185,10 @@ int prs_measure(prs_sim* sim, double* area_per_volume, double* gamma_v, int64_t*
 /* As prs_measure, filling the whole record. */
 int prs_measure_ex(prs_sim* sim, prs_diag* out);
 
-/* prs_step(nsteps) fused with the diagnostics of the state at the start of the call
- * (Eq. 7, Eq. 8 on phi^n, dphi^{n-1/2}): for FP32 boxes of the fast path the first
- * step's pass computes both from one read of the state.  *out receives what
- * prs_measure_ex would have returned before the call (out->step = n).  nsteps = 0
- * only measures.  Synchronises at the end. */
+/* The diagnostics of the state at the start of the call (Eq. 7, Eq. 8 on phi^n,
+ * dphi^{n-1/2}) and prs_step(nsteps) queued behind them, without a host round trip in
+ * between.  *out receives what prs_measure_ex would have returned before the call
+ * (out->step = n).  nsteps = 0 only measures.  Synchronises at the end. */
 int prs_step_measure(prs_sim* sim, int64_t nsteps, prs_diag* out);
 
 /* Checkpoint: copy the current fields to host arrays (either may be NULL) and the

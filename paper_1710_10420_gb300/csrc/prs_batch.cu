@@ -576,17 +576,12 @@ static int solo_queue(prs_batch* b, const int64_t* nsteps, int64_t measure_every
         const int m_runs = (int)sims.size();
         int rc = PRS_OK;
         if (measure_every > 0) {
-            std::vector<int64_t> taken(m_runs, 0);
             for (int k = 0; k < S.runs[r0].nout && !rc; ++k) {
                 const int64_t left = nsteps[r0] - (int64_t)k * measure_every;
                 const int64_t m = left < measure_every ? left : measure_every;
-                std::vector<DiagAcc*> res(m_runs);
-                for (int q = 0; q < m_runs; ++q) res[q] = (DiagAcc*)((char*)b->work + S.res_off[grp[q]]) + k;
-                rc = step_measure_first_runs(sims.data(), m_runs, m, res.data(), taken.data());
-                bool same = true;
-                for (int q = 0; q < m_runs; ++q) same = same && taken[q] == taken[0];
-                if (!rc && same) rc = step_runs(sims.data(), m_runs, m - taken[0]);
-                for (int q = 0; q < m_runs && !rc && !same; ++q) rc = step_runs(&sims[q], 1, m - taken[q]);
+                for (int q = 0; q < m_runs && !rc; ++q)
+                    rc = queue_diagnostics(sims[q], (DiagAcc*)((char*)b->work + S.res_off[grp[q]]) + k);
+                if (!rc) rc = step_runs(sims.data(), m_runs, m);
             }
         } else {
             rc = step_runs(sims.data(), m_runs, nsteps[r0]);

@@ -1,18 +1,13 @@
-// prs_generic.cu -- initial conditions, the any-shape leapfrog step and the fused
-// wall diagnostics with their FP64 reduction.
+// prs_generic.cu -- initial conditions and the any-shape leapfrog step.
 //
 //   init     : SplitMix64 random field (Sec. III initial conditions), dphi = 0
 //   step     : Eqs. 3-5 with the damping of Eq. 6, one thread per site, any box
 //              side >= 3 (used for sides that are not a multiple of 4, for FP64 and
 //              for the ragged cases the fast kernels do not take)
-//   measure  : Eq. 7 (link sign-change area) and Eq. 8 (wall-weighted velocity)
-//              in one pass, warp-shuffle + block reduction into per-block FP64
-//              partials, then a fixed-order final reduction by the last block.
 #include <cuda_runtime.h>
 
 #include "prs_arith.cuh"
 #include "prs_internal.h"
-#include "prs_reduce.cuh"
 
 namespace prs {
 
@@ -176,159 +171,6 @@ cudaError_t launch_step_generic(const Geo& g, int precision, bool repro, const v
     if (precision == PRS_FP32) return step_generic_t<float, false>(g, in, out, dphi, dphi_out, c1, c2, cV, rcd, st);
     if (repro) return step_generic_t<double, true>(g, in, out, dphi, dphi_out, c1, c2, cV, rcd, st);
     return step_generic_t<double, false>(g, in, out, dphi, dphi_out, c1, c2, cV, rcd, st);
-}
-
-// ------------------------------------------------------------ diagnostics
-
-template <typename R>
-__device__ __forceinline__ R fetch(const R* __restrict__ phi, const Geo& g, int64_t x, int64_t y, int64_t z)
-{
-    x = x < 0 ? x + g.nx : (x >= g.nx ? x - g.nx : x);
-    y = y < 0 ? y + g.ny : (y >= g.ny ? y - g.ny : y);
-    z = z < 0 ? z + g.nz : (z >= g.nz ? z - g.nz : z);
-    return phi[x + (int64_t)g.nx * (y + (int64_t)g.ny * z)];
-}
-
-// Eq. 7 weight of the link from site (x,y,z) to its +1 neighbour along axis d:
-// |g| / sum_i |g_i|, with g_d the one-sided difference along the link and the
-// transverse components the centred differences averaged over the two ends.
-template <typename R, int D>
-__device__ R link_weight(const R* __restrict__ phi, const Geo& g, int64_t x, int64_t y, int64_t z, int d, R ps, R pt)
-{
-    using A = Arith<R, true>;
-    int64_t tx = x + (d == 0), ty = y + (d == 1), tz = z + (d == 2);
-    R num = (R)0, den = (R)0;
-#pragma unroll
-    for (int e = 0; e < D; ++e) {
-        R gg;
-        if (e == d) {
-            gg = A::sub(pt, ps);
-        } else {
-            int ex = (e == 0), ey = (e == 1), ez = (e == 2);
-            R gs = A::sub(fetch(phi, g, x + ex, y + ey, z + ez), fetch(phi, g, x - ex, y - ey, z - ez));
-            R gt = A::sub(fetch(phi, g, tx + ex, ty + ey, tz + ez), fetch(phi, g, tx - ex, ty - ey, tz - ez));
-            gg = A::mul((R)0.25, A::add(gs, gt));
-        }
-        num = A::add(num, A::mul(gg, gg));
-        den = A::add(den, fabs(gg));
-    }
-    // den > 0 (the link's own component is non-zero); if the squares underflow,
-    // rescale the components by den first
-    const R tiny = sizeof(R) == 4 ? (R)1e-30 : (R)1e-290;
-    if (!(num >= tiny)) {
-        R n2 = (R)0;
-#pragma unroll
-        for (int e = 0; e < D; ++e) {
-            R gg;
-            if (e == d) {
-                gg = A::sub(pt, ps);
-            } else {
-                int ex = (e == 0), ey = (e == 1), ez = (e == 2);
-                R gs = A::sub(fetch(phi, g, x + ex, y + ey, z + ez), fetch(phi, g, x - ex, y - ey, z - ez));
-                R gt = A::sub(fetch(phi, g, tx + ex, ty + ey, tz + ez), fetch(phi, g, tx - ex, ty - ey, tz - ez));
-                gg = A::mul((R)0.25, A::add(gs, gt));
-            }
-            const R r = A::div(gg, den);
-            n2 = A::add(n2, A::mul(r, r));
-        }
-        return A::sqrt(n2);
-    }
-    return A::div(A::sqrt(num), den);
-}
-
-template <typename R, int D>
-__global__ void __launch_bounds__(256) k_measure(const R* __restrict__ phi, const R* __restrict__ dphi, Geo g,
-                                                 RunConst<R> rc, DiagScratch scr)
-{
-    using A = Arith<R, true>;
-    DiagAcc a{0.0, 0.0, 0, 0, 0, 0};
-    const int64_t rows = (int64_t)g.ny * g.nz;
-    for (int64_t row = blockIdx.y; row < rows; row += gridDim.y) {
-        const int64_t y = row % g.ny, z = row / g.ny;  // once per row
-        for (int64_t x = blockIdx.x * blockDim.x + threadIdx.x; x < g.nx; x += gridDim.x * blockDim.x) {
-            const int64_t s = row * g.nx + x;
-            R ps = phi[s];
-            R vs = dphi[s];
-            bool neg = ps < (R)0;
-            if (!isfinite(ps) || !isfinite(vs)) a.n_nonfinite++;
-            bool wall = false;
-#pragma unroll
-            for (int d = 0; d < D; ++d) {
-                int ex = (d == 0), ey = (d == 1), ez = (d == 2);
-                R pt = fetch(phi, g, x + ex, y + ey, z + ez);
-                R pm = fetch(phi, g, x - ex, y - ey, z - ez);
-                if ((pt < (R)0) != neg) {
-                    a.n_links++;
-                    a.sum_w += (double)link_weight<R, D>(phi, g, x, y, z, d, ps, pt);
-                    wall = true;
-                }
-                if ((pm < (R)0) != neg) wall = true;
-            }
-            if (wall) {
-                a.n_wall++;
-                // u = phi^2/phi0^2 - 1.  FP64 keeps the order of Eq. 1; FP32 factors it as
-                // (phi - phi0)(phi + phi0)/phi0^2, equal in exact arithmetic and free of
-                // the cancellation of phi^2 - 1 next to the vacua.
-                R u;
-                if (sizeof(R) == 8)
-                    u = A::sub(A::mul(A::mul(ps, ps), rc.inv_phi0sq), (R)1);
-                else
-                    u = A::mul(A::mul(A::sub(ps, rc.phi0), A::add(ps, rc.phi0)), rc.inv_phi0sq);
-                R V = A::mul(A::mul(rc.V0, u), u);
-                if (V > (R)0)
-                    a.sum_ratio += (double)A::div(A::mul(vs, vs), V);
-                else
-                    a.n_vzero++;
-            }
-        }
-    }
-    block_reduce_and_finish(a, scr);
-}
-
-template <typename R>
-static cudaError_t measure_t(const Geo& g, const void* phi, const void* dphi, const double rcd[6],
-                             const DiagScratch& scr, cudaStream_t st)
-{
-    const dim3 grid = rows_grid(g, scr.max_blocks < 152 * 8 ? scr.max_blocks : 152 * 8);  // one partial per block
-    RunConst<R> rc = make_rc<R>(rcd);
-    if (g.dims == 3)
-        k_measure<R, 3><<<grid, 256, 0, st>>>((const R*)phi, (const R*)dphi, g, rc, scr);
-    else
-        k_measure<R, 2><<<grid, 256, 0, st>>>((const R*)phi, (const R*)dphi, g, rc, scr);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_measure(const Geo& g, int precision, const void* phi, const void* dphi, const double rcd[6],
-                           const DiagScratch& scr, cudaStream_t st)
-{
-    if (precision == PRS_FP32) return measure_t<float>(g, phi, dphi, rcd, scr, st);
-    return measure_t<double>(g, phi, dphi, rcd, scr, st);
-}
-
-}  // namespace prs
-
-namespace prs {
-
-// The same diagnostic kernel on a caller-chosen grid (one partial slot per block in scr).
-template <typename R>
-static cudaError_t measure_grid_t(const Geo& g, const void* phi, const void* dphi, const double rcd[6],
-                                  const DiagScratch& scr, int grid, cudaStream_t st)
-{
-    RunConst<R> rc = make_rc<R>(rcd);
-    const dim3 g2(1, (unsigned)grid, 1);  // grid blocks striding over the rows
-    if (g.dims == 3)
-        k_measure<R, 3><<<g2, 256, 0, st>>>((const R*)phi, (const R*)dphi, g, rc, scr);
-    else
-        k_measure<R, 2><<<g2, 256, 0, st>>>((const R*)phi, (const R*)dphi, g, rc, scr);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_measure_on_grid(const Geo& g, int precision, const void* phi, const void* dphi,
-                                   const double rcd[6], const DiagScratch& scr, int grid, cudaStream_t st)
-{
-    if (grid < 1 || grid > scr.max_blocks || grid > 65535) return cudaErrorInvalidValue;  // gridDim.y limit
-    if (precision == PRS_FP32) return measure_grid_t<float>(g, phi, dphi, rcd, scr, grid, st);
-    return measure_grid_t<double>(g, phi, dphi, rcd, scr, grid, st);
 }
 
 }  // namespace prs

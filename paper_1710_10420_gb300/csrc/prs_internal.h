@@ -79,20 +79,25 @@ struct DiagAcc {
     long long n_nonfinite;
 };
 
-// Device scratch of the diagnostics: per-block partials + a completion counter.
-struct DiagScratch {
-    DiagAcc* partials;     // [max_blocks]
-    DiagAcc* result;       // [1]
-    unsigned int* counter; // [1], zero between launches
-    int max_blocks;
-};
-
 // Device words the host reads back with the diagnostics: the result, the
 // completion counter and the sticky error code of bounded waits (0 = none).
 struct DevStatus {
     DiagAcc result;
     unsigned int counter;
     unsigned int error;
+};
+
+// Device scratch of the diagnostics: per-block partials + a completion counter.
+struct DiagScratch {
+    DiagAcc* partials;     // [max_blocks]
+    DiagAcc* result;       // [1]
+    unsigned int* counter; // [1], zero between launches
+    int max_blocks;
+    // Host memory (pinned, mapped) that the reduction also writes its result and *error to, or
+    // null.  The last block's stores take the place of a copy behind the kernel: a copy engine's
+    // turn between two kernels costs a small box 5 us.
+    DevStatus* host;
+    const unsigned int* error;
 };
 
 // PRS_DEBUG: guard bands around library-owned fields and the scan's results.
@@ -127,18 +132,13 @@ cudaError_t launch_step_io(const Geo& g, int precision, bool repro, const void* 
 int max_fused_steps(const Geo& g, int precision, bool repro);
 int default_fused_steps(const Geo& g, int precision, bool repro);
 
-cudaError_t launch_measure(const Geo& g, int precision, const void* phi, const void* dphi, const double run_const[6],
-                           const DiagScratch& scr, cudaStream_t st);
+// The wall diagnostics of (phi, dphi) (prs_measure.cu), any box.  fast (FP32): hardware
+// reciprocal square root and division, else IEEE operations.  err: the run's error word.
+cudaError_t launch_measure(const Geo& g, int precision, bool fast, const void* phi, const void* dphi,
+                           const double run_const[6], const DiagScratch& scr, unsigned int* err, cudaStream_t st);
 
 // Fast FP32 kernels (prs_fast.cu) for x sides that are multiples of 128.
 bool fast_step_ok(const Geo& g, int precision);
-cudaError_t launch_measure_fast(const Geo& g, const float* phi, const float* v, RunConst<float> rc,
-                                const DiagScratch& scr, unsigned int* err, cudaStream_t st);
-// One step (in -> out, v -> v_out) and the diagnostics of (in, v); cudaErrorNotSupported
-// when this box has no fused kernel.
-cudaError_t launch_step_measure_fast(const Geo& g, const float* in, float* out, const float* v, float* v_out,
-                                     KickF k, RunConst<float> rc, const DiagScratch& scr, unsigned int* err,
-                                     cudaStream_t st);
 
 // Two fused leapfrog steps per pass (prs_tblock.cu), FP32 3D and 2D; dphi out of place.
 bool tblock_ok(const Geo& g, int precision);
@@ -178,7 +178,7 @@ cudaError_t launch_step_t3(const Geo& g, const float* phi_in, float* phi_out, co
 // Store a message for prs_last_error() on this thread.
 void record_error(const char* msg);
 
-// The diagnostic kernel launched on exactly `grid` blocks (1 <= grid <= scr.max_blocks).
+// The diagnostic kernel (IEEE operations) on at most `grid` blocks (1 <= grid <= scr.max_blocks).
 cudaError_t launch_measure_on_grid(const Geo& g, int precision, const void* phi, const void* dphi,
                                    const double run_const[6], const DiagScratch& scr, int grid, cudaStream_t st);
 

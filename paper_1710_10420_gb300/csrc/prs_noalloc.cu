@@ -101,6 +101,8 @@ extern "C" int prs_measure_noalloc(const prs_params* p, const void* d_phi, const
     scr.result = (DiagAcc*)((char*)base + kResultOffset);
     scr.counter = (unsigned int*)((char*)base + kCounterOffset);
     scr.max_blocks = kNoAllocSlots;
+    scr.host = nullptr;
+    scr.error = nullptr;
 
     Geo g;
     g.dims = p->dims;

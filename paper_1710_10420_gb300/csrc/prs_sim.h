@@ -51,17 +51,9 @@ int cuda_fail(cudaError_t e, const char* what);
 int ensure_buffers(prs_sim* s);
 // After a synchronised read of s->h_status: PRS_ETIMEOUT (once) if a device wait gave up.
 int check_device_error(prs_sim* s);
-// Queue the first part of what prs_step_measure(nsteps) does, without waiting for it: the
-// Eq. 7/8 sums of the current state into *result (device memory), fused into the first step
-// where a fused kernel serves the box.  *taken: the steps queued (1 fused, else 0); the
-// caller steps the other nsteps - *taken as prs_step would, for the same fields.  A bounded
-// wait that gives up sets the run's device error word.
-int step_measure_first(prs_sim* s, int64_t nsteps, DiagAcc* result, int64_t* taken);
-// step_measure_first for several runs: one launch of the fused one-step pass over all of them
-// when they share a 2D box and stream (at most kT3MaxRuns; the fields are those of the runs'
-// own passes, the sums the same to FP64 rounding), else run by run.
-int step_measure_first_runs(prs_sim* const* runs, int nruns, int64_t nsteps, DiagAcc* const* results,
-                            int64_t* taken);
+// Queue the Eq. 7/8 sums of the run's current state into *result (device memory), without
+// waiting for them.
+int queue_diagnostics(prs_sim* s, DiagAcc* result);
 // Step each of several runs by nsteps as prs_step would step it alone (the same passes in the
 // same order, so the same fields), issuing each round of 2D three-step passes and of single
 // steps as one launch over all the runs when they share a box, stream and plan (at most

@@ -26,8 +26,8 @@ EncodeTiled tmap_encoder();
 bool tmap_encode(EncodeTiled f, CUtensorMap* m, const float* base, const Geo& g, unsigned bw, unsigned bh);
 
 // One tensor copy of the box at (x, y, z) of `map` into shared memory at `dst` (128-byte
-// aligned), counted on `bar` as transaction bytes.  x times 4 bytes must be a multiple of 16.
-__device__ __forceinline__ void tma_load3(float* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar)
+// aligned), counted on `bar` as transaction bytes.  x times the element size must be a multiple of 16.
+__device__ __forceinline__ void tma_load3(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar)
 {
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
