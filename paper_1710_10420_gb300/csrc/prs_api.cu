@@ -353,9 +353,7 @@ static int set_state_device(prs_sim* s, const void* d_phi, const void* d_dphi, i
     int rc = ensure_buffers(s);
     if (rc) return rc;
     size_t bytes = (size_t)s->g.S * s->elem;
-    if (d_phi != s->phi[s->cur])
-        PRS_CUDA(cudaMemcpyAsync(s->phi[s->cur], d_phi, bytes, cudaMemcpyDeviceToDevice, s->stream));
-    if (d_dphi != s->dphi) PRS_CUDA(cudaMemcpyAsync(s->dphi, d_dphi, bytes, cudaMemcpyDeviceToDevice, s->stream));
+    PRS_CUDA(launch_copy_state(d_phi, s->phi[s->cur], d_dphi, s->dphi, bytes, s->stream));
     ensure_dphi_alt(s);
     s->n = n;
     s->initialised = true;

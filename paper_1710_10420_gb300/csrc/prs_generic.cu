@@ -173,4 +173,47 @@ cudaError_t launch_step_generic(const Geo& g, int precision, bool repro, const v
     return step_generic_t<double, false>(g, in, out, dphi, dphi_out, c1, c2, cV, rcd, st);
 }
 
+// ---------------------------------------------------------- state copies
+
+// phi and dphi of a state in one launch, 64 bytes a thread and turn.  Bound by HBM for large boxes
+// (1024^3: what two device-to-device copies take); for small ones by the launch, of which this
+// saves one (256^2: 4 us of 81).
+__global__ void __launch_bounds__(256) k_copy_state(const float4* __restrict__ p, float4* __restrict__ po,
+                                                    const float4* __restrict__ v, float4* __restrict__ vo, int64_t n)
+{
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x * 4 + threadIdx.x; i < 2 * n; i += stride) {
+        float4 a[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t j = i + u * (int64_t)blockDim.x;
+            if (j < 2 * n) a[u] = j < n ? __ldcs(p + j) : __ldcs(v + (j - n));
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t j = i + u * (int64_t)blockDim.x;
+            if (j < n) po[j] = a[u];
+            else if (j < 2 * n) vo[j - n] = a[u];
+        }
+    }
+}
+
+cudaError_t launch_copy_state(const void* phi, void* phi_out, const void* dphi, void* dphi_out, size_t bytes,
+                              cudaStream_t st)
+{
+    const uintptr_t a = (uintptr_t)phi, b = (uintptr_t)phi_out, c = (uintptr_t)dphi, d = (uintptr_t)dphi_out;
+    auto apart = [&](uintptr_t s, uintptr_t t) { return s + bytes <= t || t + bytes <= s; };
+    if (((a | b | c | d | bytes) & 15u) || !apart(a, b) || !apart(a, d) || !apart(c, b) || !apart(c, d) ||
+        !apart(b, d)) {
+        cudaError_t e = cudaSuccess;  // one after the other
+        if (a != b) e = cudaMemcpyAsync(phi_out, phi, bytes, cudaMemcpyDeviceToDevice, st);
+        if (e == cudaSuccess && c != d) e = cudaMemcpyAsync(dphi_out, dphi, bytes, cudaMemcpyDeviceToDevice, st);
+        return e;
+    }
+    const int64_t n = (int64_t)(bytes / 16);
+    k_copy_state<<<grid_for(2 * n, 1024), 256, 0, st>>>((const float4*)phi, (float4*)phi_out, (const float4*)dphi,
+                                                        (float4*)dphi_out, n);
+    return cudaGetLastError();
+}
+
 }  // namespace prs

@@ -127,6 +127,10 @@ cudaError_t launch_step_io(const Geo& g, int precision, bool repro, const void* 
                            const void* dphi_in, void* dphi_out, const double* c1, const double* c2, const double* cV,
                            int nsteps_in_pass, const double run_const[6], unsigned int* err, cudaStream_t st);
 
+// Copy a state's fields (device to device, `bytes` each; a field that is its own source stays).
+cudaError_t launch_copy_state(const void* phi, void* phi_out, const void* dphi, void* dphi_out, size_t bytes,
+                              cudaStream_t st);
+
 // Largest number of steps one pass can fuse for this geometry/precision, and the
 // number used when params.tblock is 0.
 int max_fused_steps(const Geo& g, int precision, bool repro);
