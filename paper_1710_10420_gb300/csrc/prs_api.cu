@@ -11,7 +11,6 @@
 
 #include "prs.h"
 #include "prs_internal.h"
-#include "prs_runs.h"
 #include "prs_sim.h"
 
 using namespace prs;
@@ -154,6 +153,11 @@ extern "C" int prs_max_tblock(const prs_params* params)
 
 static const int kMeasureBlocks = 8192;  // partial slots: the fast kernels use one per tile
 
+// FP32 2D runs step by the register march (prs_march2d.cuh); without a tblock the march also plans
+// the steps of its passes.
+static bool march_run(const prs_sim* s) { return s->g.dims == 2 && s->p.precision == PRS_FP32; }
+static bool march_plans(const prs_sim* s) { return march_run(s) && s->p.tblock == 0; }
+
 extern "C" int prs_create(const prs_params* params, void* stream, prs_sim** out)
 {
     if (!out) return PRS_EINVAL;
@@ -173,6 +177,7 @@ extern "C" int prs_create(const prs_params* params, void* stream, prs_sim** out)
     s->rc[4] = potential_height(*params);
     s->rc[5] = params->phi0;
     s->scr.max_blocks = kMeasureBlocks;
+    if (march_run(s)) march_plan(g, 1, &s->march);
     void* blob = nullptr;
     size_t bytes = sizeof(DiagAcc) * kMeasureBlocks + sizeof(DevStatus);
     if (cudaMalloc(&blob, bytes) != cudaSuccess) {
@@ -288,7 +293,7 @@ static int run_tblock(const prs_sim* s)
 // steps one step per pass.
 static void ensure_dphi_alt(prs_sim* s)
 {
-    if (s->dphi_alt || run_tblock(s) < 2) return;
+    if (s->dphi_alt || (run_tblock(s) < 2 && !march_plans(s))) return;
     if (cudaMalloc(&s->dphi_alt, (size_t)s->g.S * s->elem) != cudaSuccess) {
         cudaGetLastError();
         s->dphi_alt = nullptr;
@@ -444,26 +449,34 @@ bool prs::cfl_ok_over(const prs_params& p, int64_t n, int64_t nsteps)
     return cfl_ok(p, n) && cfl_ok(p, n + nsteps - 1);
 }
 
-// The passes of a call of nsteps (>= 1): n3 of three steps, n2 of two, then n1 single steps.
-static void step_plan(const prs_sim* s, int64_t nsteps, int64_t& n3, int64_t& n2, int64_t& n1)
+// The passes of a call of nsteps (>= 1): cnt[t] of t steps, the longest first.
+static void step_plan(const prs_sim* s, const MarchPlan* march, int64_t nsteps, int64_t cnt[kMarchMaxT + 1])
 {
     const bool repro = (s->p.flags & PRS_REPRO) != 0;
     const int tb = run_tblock(s);
-    // Multi-step passes (two or three steps) read dphi across sites, so they write it to a
-    // second buffer.  A call runs n3 passes of three steps, n2 of two, then n1 single steps:
-    // with T = tblock = 3, nsteps / 3 triples and a pair or a single step for the remainder;
-    // with T = 2, pairs, and for an odd count a single step, or, when the library chooses the
-    // steps per pass (tblock = 0) and the box takes three-step passes, one triple instead of a
-    // pair and a single step.  After an odd number of multi-step passes dphi sits in the
-    // second buffer.  A run whose buffers the library owns (no PRS_DEBUG guard bands) then
-    // swaps the roles of its two dphi buffers.  A run with bound buffers keeps dphi in the
-    // bound buffer at the end of every call: the first single step after an odd number of
-    // multi-step passes reads dphi in the second buffer and writes the bound one; with no
-    // single step to do it, the triple of an odd T = 2 count runs as a pair and a single
-    // step, else the last pair as two single steps, else the last triple as a pair and a
-    // single step.  Single steps otherwise update dphi in place.
+    // Multi-step passes read dphi across sites, so they write it to a second buffer.  A call runs its
+    // passes the longest first, single steps last: with T = tblock = 3, nsteps / 3 triples and a pair
+    // or a single step for the remainder; with T = 2, pairs, and for an odd count a single step, or,
+    // when the library chooses the steps per pass (tblock = 0) and the box takes three-step passes,
+    // one triple instead of a pair and a single step; in FP32 2D without a tblock what march_counts
+    // plans.  After an odd number of multi-step passes dphi sits in the second buffer.  A run whose
+    // buffers the library owns (no PRS_DEBUG guard bands) then swaps the roles of its two dphi
+    // buffers.  A run with bound buffers keeps dphi in the bound buffer at the end of every call: the
+    // first single step after an odd number of multi-step passes reads dphi in the second buffer and
+    // writes the bound one; with no single step to do it, the triple of an odd T = 2 count runs as a
+    // pair and a single step, else the last pair as two single steps, else the last triple as a pair
+    // and a single step.  Single steps otherwise update dphi in place.
     const bool swap_ok = s->owned && (s->p.flags & PRS_DEBUG) == 0;
-    n3 = 0, n2 = 0, n1 = nsteps;
+    for (int t = 0; t <= kMarchMaxT; ++t) cnt[t] = 0;
+    if (!s->dphi_alt) {  // no second buffer (no room at prs_init)
+        cnt[1] = nsteps;
+        return;
+    }
+    if (march_plans(s)) {
+        march_counts(*march, nsteps, !swap_ok, cnt);
+        return;
+    }
+    int64_t n3 = 0, n2 = 0, n1 = nsteps;
     if (tb == 3) {
         n3 = nsteps / 3;
         n2 = nsteps - 3 * n3 == 2 ? 1 : 0;
@@ -474,12 +487,52 @@ static void step_plan(const prs_sim* s, int64_t nsteps, int64_t& n3, int64_t& n2
         if (n1 == 1 && n2 >= 1 && s->p.tblock == 0 && max_fused_steps(s->g, s->p.precision, repro) >= 3)
             n3 = 1, n2 -= 1, n1 = 0;
     }
-    if (!s->dphi_alt) n3 = n2 = 0, n1 = nsteps;  // no second buffer (no room at prs_init)
     if (((n3 + n2) & 1) && n1 == 0 && !swap_ok) {
         if (tb == 2 && n3 == 1) n3 = 0, n2 += 1, n1 = 1;
         else if (n2 > 0) n2 -= 1, n1 += 2;
         else n3 -= 1, n2 += 1, n1 += 1;
     }
+    cnt[3] = n3, cnt[2] = n2, cnt[1] = n1;
+}
+
+// Queue one pass of t steps from step n: phi[cur] -> phi[1 - cur], dphi from v_in to v_out (equal only
+// for t = 1).  Flips cur.
+static cudaError_t queue_pass(prs_sim* s, int t, int64_t n, const void* v_in, void* v_out)
+{
+    const bool repro = (s->p.flags & PRS_REPRO) != 0;
+    unsigned int* err = &s->d_status->error;
+    const void* in = s->phi[s->cur];
+    void* out = s->phi[1 - s->cur];
+    double c[kMarchMaxT][5];
+    for (int l = 0; l < t; ++l) step_coefficients(s->p, n + l, c[l]);
+    cudaError_t e;
+    if (march_run(s)) {
+        MarchRun r{in, out, v_in, v_out, {}, s->rc};
+        for (int l = 0; l < t; ++l)
+            for (int q = 0; q < 3; ++q) r.coef[l][q] = c[l][q];
+        e = launch_march2d(s->g, t, s->march.shape[t], 1, &r, s->stream);
+    } else if (t == 1) {
+        e = launch_step_io(s->g, s->p.precision, repro, in, out, v_in, v_out, &c[0][0], &c[0][1], &c[0][2], 1, s->rc,
+                           err, s->stream);
+    } else {
+        const RunConst<float> rcf{(float)s->rc[0], (float)s->rc[1], (float)s->rc[2],
+                                  (float)s->rc[3], (float)s->rc[4], (float)s->rc[5]};
+        const KickF k0 = kick_f32(c[0], s->rc), k1 = kick_f32(c[1], s->rc);
+        e = t == 3 ? launch_step_t3_tma(s->g, (const float*)in, (float*)out, (const float*)v_in, (float*)v_out, k0, k1,
+                                        kick_f32(c[2], s->rc), rcf, err, s->stream)
+                   : launch_step_t2(s->g, (const float*)in, (float*)out, (const float*)v_in, (float*)v_out, k0, k1,
+                                    rcf, err, s->stream);
+        if (t == 3 && e == cudaErrorNotSupported) {  // no tensor-map encoder: a pair, then a single step in place
+            e = launch_step_t2(s->g, (const float*)in, (float*)out, (const float*)v_in, (float*)v_out, k0, k1, rcf, err,
+                               s->stream);
+            if (e == cudaSuccess)
+                e = launch_step_io(s->g, s->p.precision, repro, out, s->phi[s->cur], v_out, v_out, &c[2][0], &c[2][1],
+                                   &c[2][2], 1, s->rc, err, s->stream);
+            s->cur = 1 - s->cur;  // phi ends where it started; the flip below undoes this
+        }
+    }
+    s->cur = 1 - s->cur;
+    return e;
 }
 
 static int prs_step_impl(prs_sim* s, int64_t nsteps)
@@ -488,55 +541,19 @@ static int prs_step_impl(prs_sim* s, int64_t nsteps)
     if (!s->initialised) return PRS_ESTATE;
     if (nsteps == 0) return PRS_OK;
     if (!cfl_ok_over(s->p, s->n, nsteps)) return PRS_EINVAL;
-    const bool repro = (s->p.flags & PRS_REPRO) != 0;
-    int64_t n3, n2, n1;
-    step_plan(s, nsteps, n3, n2, n1);
-    unsigned int* err = &s->d_status->error;
-    const RunConst<float> rcf{(float)s->rc[0], (float)s->rc[1], (float)s->rc[2],
-                              (float)s->rc[3], (float)s->rc[4], (float)s->rc[5]};
+    if (march_run(s) && s->march.nruns != 1) march_plan(s->g, 1, &s->march);
+    int64_t cnt[kMarchMaxT + 1];
+    step_plan(s, &s->march, nsteps, cnt);
     void* vbuf[2] = {s->dphi, s->dphi_alt};
     int vi = 0;  // vbuf[vi] holds dphi
     int64_t n = s->n;
-    for (int64_t k = 0; k < n3 + n2; ++k) {
-        const int t = k < n3 ? 3 : 2;
-        double a[5], b[5], c[5];
-        step_coefficients(s->p, n, a);
-        step_coefficients(s->p, n + 1, b);
-        cudaError_t e;
-        if (t == 3) {
-            step_coefficients(s->p, n + 2, c);
-            e = launch_step_t3(s->g, (const float*)s->phi[s->cur], (float*)s->phi[1 - s->cur],
-                               (const float*)vbuf[vi], (float*)vbuf[1 - vi], kick_f32(a, s->rc), kick_f32(b, s->rc),
-                               kick_f32(c, s->rc), rcf, err, s->stream);
-            if (e == cudaErrorNotSupported) {  // no tensor-map encoder: a pair, then a single step in place
-                e = launch_step_t2(s->g, (const float*)s->phi[s->cur], (float*)s->phi[1 - s->cur],
-                                   (const float*)vbuf[vi], (float*)vbuf[1 - vi], kick_f32(a, s->rc),
-                                   kick_f32(b, s->rc), rcf, err, s->stream);
-                if (e == cudaSuccess)
-                    e = launch_step_io(s->g, s->p.precision, repro, s->phi[1 - s->cur], s->phi[s->cur],
-                                       vbuf[1 - vi], vbuf[1 - vi], &c[0], &c[1], &c[2], 1, s->rc, err, s->stream);
-                s->cur = 1 - s->cur;  // phi ends where it started; the common flip below undoes this
-            }
-        } else {
-            e = launch_step_t2(s->g, (const float*)s->phi[s->cur], (float*)s->phi[1 - s->cur],
-                               (const float*)vbuf[vi], (float*)vbuf[1 - vi], kick_f32(a, s->rc),
-                               kick_f32(b, s->rc), rcf, err, s->stream);
+    for (int t = kMarchMaxT; t >= 1; --t)
+        for (int64_t k = 0; k < cnt[t]; ++k, n += t) {
+            // the first single step brings dphi home
+            const cudaError_t e = queue_pass(s, t, n, vbuf[vi], t > 1 ? vbuf[1 - vi] : s->dphi);
+            if (e != cudaSuccess) return cuda_fail(e, "prs_step launch");
+            vi = t > 1 ? 1 - vi : 0;
         }
-        if (e != cudaSuccess) return cuda_fail(e, "prs_step launch");
-        s->cur = 1 - s->cur;
-        vi = 1 - vi;
-        n += t;
-    }
-    for (int64_t k = 0; k < n1; ++k) {
-        double c[5];
-        step_coefficients(s->p, n + k, c);
-        const void* v_in = vbuf[vi];  // the first single step brings dphi home
-        cudaError_t e = launch_step_io(s->g, s->p.precision, repro, s->phi[s->cur], s->phi[1 - s->cur], v_in,
-                                       s->dphi, &c[0], &c[1], &c[2], 1, s->rc, err, s->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "prs_step launch");
-        s->cur = 1 - s->cur;
-        vi = 0;
-    }
     if (vi) {  // dphi now sits in the second buffer, which becomes the run's own (only when swap_ok)
         void* t = s->dphi;
         s->dphi = s->dphi_alt;
@@ -623,117 +640,57 @@ int prs::step_runs(prs_sim* const* runs, int nruns, int64_t nsteps)
 {
     if (nruns < 0 || nsteps < 0) return PRS_EINVAL;
     if (nruns == 0 || nsteps == 0) return PRS_OK;
-    // the runs qualify when they share their box, stream and plan and the plan's triples are
-    // 2D three-step passes; else each runs alone
-    int64_t n3 = 0, n2 = 0, n1 = 0;
-    bool together = nruns > 1 && nruns <= kT3MaxRuns;
-    for (int r = 0; r < nruns && together; ++r) {
+    bool together = nruns > 1 && nruns <= kMarchMaxRuns;
+    for (int r = 0; r < nruns; ++r) {
         const prs_sim* s = runs[r];
         if (!s) return PRS_EINVAL;
         if (!s->initialised) return PRS_ESTATE;
         if (!cfl_ok_over(s->p, s->n, nsteps)) return PRS_EINVAL;
-        int64_t a3, a2, a1;
-        step_plan(s, nsteps, a3, a2, a1);
-        const Geo& g = s->g;
-        const Geo& g0 = runs[0]->g;
-        together = g.dims == 2 && g.nx == g0.nx && g.ny == g0.ny && s->stream == runs[0]->stream &&
-                   s->p.precision == PRS_FP32 && (s->p.flags & PRS_REPRO) == 0 && run_tblock(s) == 3 &&
-                   t3_2d_ok(g) && s->dphi_alt && (r == 0 || (a3 == n3 && a2 == n2 && a1 == n1));
-        if (r == 0) n3 = a3, n2 = a2, n1 = a1;
+        const Geo &g = s->g, &g0 = runs[0]->g;
+        together = together && march_plans(s) && g.nx == g0.nx && g.ny == g0.ny && g.nx % 128 == 0 &&
+                   g.nx <= 4096 && s->stream == runs[0]->stream && s->dphi_alt && s->owned == runs[0]->owned &&
+                   (s->p.flags & PRS_DEBUG) == 0;
     }
-    if (!together || n3 == 0) {
+    if (!together) {
         for (int r = 0; r < nruns; ++r) {
             const int rc = prs_step_impl(runs[r], nsteps);
             if (rc) return rc;
         }
         return PRS_OK;
     }
-    // the passes of prs_step_impl, pass by pass across the runs: the triples as one launch
-    std::vector<int> vi(nruns, 0);  // per run: its vbuf index that holds dphi
-    std::vector<const float*> pin(nruns), vin(nruns);
-    std::vector<float*> pout(nruns), vout(nruns);
-    std::vector<KickF> kk(3 * (size_t)nruns);
-    std::vector<RunConst<float>> rcs(nruns);
-    for (int r = 0; r < nruns; ++r) {
-        const prs_sim* s = runs[r];
-        rcs[r] = RunConst<float>{(float)s->rc[0], (float)s->rc[1], (float)s->rc[2],
-                                 (float)s->rc[3], (float)s->rc[4], (float)s->rc[5]};
-    }
-    auto vbuf = [&](int r, int i) { return i == 0 ? runs[r]->dphi : runs[r]->dphi_alt; };
-    int64_t done = 0;
-    for (int64_t k = 0; k < n3; ++k, done += 3) {
-        for (int r = 0; r < nruns; ++r) {
-            prs_sim* s = runs[r];
-            for (int l = 0; l < 3; ++l) {
-                double c[5];
-                step_coefficients(s->p, s->n + done + l, c);
-                kk[3 * (size_t)r + l] = kick_f32(c, s->rc);
-            }
-            pin[r] = (const float*)s->phi[s->cur];
-            pout[r] = (float*)s->phi[1 - s->cur];
-            vin[r] = (const float*)vbuf(r, vi[r]);
-            vout[r] = (float*)vbuf(r, 1 - vi[r]);
-        }
-        const cudaError_t e = launch_step_t3_2d_runs(runs[0]->g, nruns, pin.data(), pout.data(), vin.data(),
-                                                     vout.data(), kk.data(), rcs.data(),
-                                                     &runs[0]->d_status->error, runs[0]->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "step_runs launch");
-        for (int r = 0; r < nruns; ++r) runs[r]->cur = 1 - runs[r]->cur, vi[r] = 1 - vi[r];
-    }
-    for (int r = 0; r < nruns; ++r) {  // pairs, run by run
-        prs_sim* s = runs[r];
-        unsigned int* err = &s->d_status->error;
-        int64_t n = s->n + done;
-        for (int64_t k = 0; k < n2; ++k, n += 2) {
-            double a[5], b[5];
-            step_coefficients(s->p, n, a);
-            step_coefficients(s->p, n + 1, b);
-            const cudaError_t e =
-                launch_step_t2(s->g, (const float*)s->phi[s->cur], (float*)s->phi[1 - s->cur],
-                               (const float*)vbuf(r, vi[r]), (float*)vbuf(r, 1 - vi[r]), kick_f32(a, s->rc),
-                               kick_f32(b, s->rc), rcs[r], err, s->stream);
-            if (e != cudaSuccess) return cuda_fail(e, "step_runs launch");
-            s->cur = 1 - s->cur;
-            vi[r] = 1 - vi[r];
-        }
-    }
-    done += 2 * n2;
-    // single steps, each one launch over the runs (the first reads dphi where the multi-step
-    // passes left it and writes the run's own buffer)
-    std::vector<KickF> k1(nruns);
-    for (int64_t k = 0; k < n1; ++k, ++done) {
-        for (int r = 0; r < nruns; ++r) {
-            prs_sim* s = runs[r];
-            double c[5];
-            step_coefficients(s->p, s->n + done, c);
-            k1[r] = kick_f32(c, s->rc);
-            pin[r] = (const float*)s->phi[s->cur];
-            pout[r] = (float*)s->phi[1 - s->cur];
-            vin[r] = (const float*)vbuf(r, vi[r]);
-            vout[r] = (float*)s->dphi;
-        }
-        cudaError_t e = launch_step2d_runs(runs[0]->g, nruns, pin.data(), pout.data(), vin.data(), vout.data(),
-                                           k1.data(), rcs.data(), &runs[0]->d_status->error,
-                                           runs[0]->stream);
-        if (e == cudaErrorNotSupported) {  // no fast one-step pass for this box: run by run
-            e = cudaSuccess;
-            for (int r = 0; r < nruns && e == cudaSuccess; ++r) {
+    MarchPlan& plan = runs[0]->march;
+    if (plan.nruns != nruns) march_plan(runs[0]->g, nruns, &plan);
+    int64_t cnt[kMarchMaxT + 1], done = 0;
+    step_plan(runs[0], &plan, nsteps, cnt);
+    MarchRun q[kMarchMaxRuns];
+    int vi = 0;  // which of each run's dphi and dphi_alt holds dphi
+    for (int t = kMarchMaxT; t >= 1; --t)
+        for (int64_t k = 0; k < cnt[t]; ++k, done += t) {
+            for (int r = 0; r < nruns; ++r) {
                 prs_sim* s = runs[r];
-                double c[5];
-                step_coefficients(s->p, s->n + done, c);
-                e = launch_step_io(s->g, s->p.precision, false, s->phi[s->cur], s->phi[1 - s->cur], vbuf(r, vi[r]),
-                                   s->dphi, &c[0], &c[1], &c[2], 1, s->rc, &s->d_status->error, s->stream);
+                void* vbuf[2] = {s->dphi, s->dphi_alt};
+                q[r].phi_in = s->phi[s->cur];
+                q[r].phi_out = s->phi[1 - s->cur];
+                q[r].v_in = vbuf[vi];
+                q[r].v_out = t > 1 ? vbuf[1 - vi] : s->dphi;
+                q[r].run_const = s->rc;
+                for (int l = 0; l < t; ++l) {
+                    double c[5];
+                    step_coefficients(s->p, s->n + done + l, c);
+                    for (int u = 0; u < 3; ++u) q[r].coef[l][u] = c[u];
+                }
             }
+            const cudaError_t e = launch_march2d(runs[0]->g, t, plan.shape[t], nruns, q, runs[0]->stream);
+            if (e != cudaSuccess) return cuda_fail(e, "step_runs launch");
+            for (int r = 0; r < nruns; ++r) runs[r]->cur = 1 - runs[r]->cur;
+            vi = t > 1 ? 1 - vi : 0;
         }
-        if (e != cudaSuccess) return cuda_fail(e, "step_runs launch");
-        for (int r = 0; r < nruns; ++r) runs[r]->cur = 1 - runs[r]->cur, vi[r] = 0;
-    }
     for (int r = 0; r < nruns; ++r) {
         prs_sim* s = runs[r];
-        if (vi[r]) {  // as prs_step_impl: only where the run may swap its dphi buffers
-            void* t = s->dphi;
+        if (vi) {  // as prs_step_impl: only where the run may swap its dphi buffers
+            void* v = s->dphi;
             s->dphi = s->dphi_alt;
-            s->dphi_alt = t;
+            s->dphi_alt = v;
         }
         s->n += nsteps;
     }

@@ -51,7 +51,6 @@
 
 #include "prs.h"
 #include "prs_internal.h"
-#include "prs_runs.h"
 #include "prs_reduce.cuh"
 #include "prs_sim.h"
 #include "prs_tile.cuh"
@@ -547,7 +546,7 @@ static int solo_make(prs_batch* b, int r)
 }
 
 // Queue the runs stepped alone, after the persistent launch, in groups of runs of one box
-// at the same step with the same step count (at most kT3MaxRuns a group, which step_runs
+// at the same step with the same step count (at most kMarchMaxRuns a group, which step_runs
 // advances together, pass by pass): with outputs, per output the diagnostics of each run's
 // state (into its result slot) fused into its first step, one launch for the group
 // (step_measure_first_runs), then the steps up to the next output; else the steps.  Each run
@@ -562,7 +561,7 @@ static int solo_queue(prs_batch* b, const int64_t* nsteps, int64_t measure_every
         if (!b->solo[r0] || queued[r0]) continue;
         std::vector<int> grp;
         const Geo& a = b->g[r0];
-        for (int r = r0; r < R && (int)grp.size() < kT3MaxRuns; ++r) {
+        for (int r = r0; r < R && (int)grp.size() < kMarchMaxRuns; ++r) {
             const Geo& g = b->g[r];
             if (b->solo[r] && !queued[r] && g.dims == a.dims && g.nx == a.nx && g.ny == a.ny && g.nz == a.nz &&
                 b->n[r] == b->n[r0] && nsteps[r] == nsteps[r0])

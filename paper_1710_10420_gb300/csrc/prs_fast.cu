@@ -27,18 +27,6 @@ __global__ void __launch_bounds__(kFastThreads, 2)
     tile3d<ITEMS, true, false>(T, k, rc, smem_raw, nullptr, a, err);
 }
 
-template <int ITEMS>
-__global__ void __launch_bounds__(kFastThreads, 2)
-    k_step2d_f32(const float* __restrict__ phi_in, float* __restrict__ phi_out, const float* v, float* v_out, int nx,
-                 int ny, int rb, int cy, KickF k, RunConst<float> rc, unsigned int* err)
-{
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    Tile2D T{phi_in, phi_out, v, v_out, nx, ny, rb, (int)blockIdx.x * cy, 0};
-    T.yn = min(cy, ny - T.y0);
-    SiteAcc a{};
-    tile2d<ITEMS, true, false>(T, k, rc, smem_raw, nullptr, a, err);
-}
-
 // ------------------------------------------------------------------ dispatch
 
 static constexpr int kItems = 4;  // float4 per thread per plane: 4096 sites per plane tile
@@ -57,14 +45,13 @@ bool fast_step_ok(const Geo& g, int precision)
     return (g.dims == 3 ? smem3d(g.nx, t) : smem2d(g.nx, t)) <= kFastSmemMax;
 }
 
-// Shortest chunks the planner considers: 4 planes (3D), one band (2D).  A small box must be
+// Shortest chunks the planner considers: 4 planes.  A small box must be
 // cut into enough chunks to occupy the GPU, or each pass is bound by the latency of a few CTAs
-// marching long chunks (one step per pass, minimum 16 planes and 4 bands before: 128^3 22.1
-// against 8.2 us per step, 256^2 8.2 against 4.2, 1024^2 8.2 against 6.2; large boxes pick
-// long chunks either way).
-constexpr int kMinPlanes = 4, kMinBands = 1;
+// marching long chunks (128^3 22.1 us per step with at least 16 planes a chunk against 8.2; large
+// boxes pick long chunks either way).
+constexpr int kMinPlanes = 4;
 
-// Number of z-chunks (3D) or row chunks (2D): balance whole waves of resident
+// Number of z-chunks: balance whole waves of resident
 // CTAs against the two halo planes each chunk re-reads.
 static int pick_chunks(int tiles, int len, int min_len, int slots)
 {
@@ -90,7 +77,7 @@ static int pick_chunks(int tiles, int len, int min_len, int slots)
 cudaError_t launch_step_fast(const Geo& g, const float* in, float* out, const float* v, float* v_out,
                              KickF k, RunConst<float> rc, unsigned int* err, cudaStream_t st)
 {
-    static std::atomic<unsigned long long> attr3{0}, attr2{0};
+    static std::atomic<unsigned long long> attr3{0};
     const int t = kItems * 1024 / g.nx;
     const int slots = 2 * sm_count_current();  // two resident CTAs per SM
     if (g.dims == 3) {
@@ -108,19 +95,7 @@ cudaError_t launch_step_fast(const Geo& g, const float* in, float* out, const fl
                                                                          k, rc, err);
         return cudaGetLastError();
     }
-    const size_t sm = smem2d(g.nx, t);
-    {
-        const cudaError_t e = smem_limit_once(attr2, (const void*)k_step2d_f32<kItems>, (int)kFastSmemMax);
-        if (e != cudaSuccess) return e;
-    }
-    if (sm > kFastSmemMax) return cudaErrorInvalidValue;
-    const int bands = g.ny / t;
-    int nchunks = pick_chunks(1, bands, kMinBands, slots);
-    const int bpc = (bands + nchunks - 1) / nchunks;
-    const int cy = bpc * t;
-    nchunks = (g.ny + cy - 1) / cy;
-    k_step2d_f32<kItems><<<nchunks, kFastThreads, sm, st>>>(in, out, v, v_out, g.nx, g.ny, t, cy, k, rc, err);
-    return cudaGetLastError();
+    return cudaErrorNotSupported;
 }
 
 }  // namespace prs

@@ -58,6 +58,12 @@ struct KickD {
     double c1, g, k1, k2;
 };
 
+inline KickD kick_f64(const double coef[3], const double run_const[6])
+{
+    const double g = coef[1] * run_const[1], h = coef[1] * coef[2];
+    return KickD{coef[0], g, h - run_const[3] * g, h * run_const[2]};
+}
+
 // Scalars fixed for the whole run, in working precision.
 template <typename R>
 struct RunConst {
@@ -116,13 +122,8 @@ KickF kick_f32(const double coef[3], const double run_const[6]);
 cudaError_t launch_init_random(const Geo& g, int precision, uint64_t seed, void* phi, void* dphi, bool zero_dphi,
                                cudaStream_t st);
 
-// One pass of `nsteps_in_pass` fused leapfrog steps from phi_in into phi_out,
-// dphi in place.  coef holds one entry per fused step (host memory, by value).
-cudaError_t launch_step(const Geo& g, int precision, bool repro, const void* phi_in, void* phi_out, void* dphi,
-                        const double* c1, const double* c2, const double* cV, int nsteps_in_pass,
-                        const double run_const[6], unsigned int* err, cudaStream_t st);
-
-// As launch_step with dphi read from dphi_in and written to dphi_out (may be equal).
+// One leapfrog step (nsteps_in_pass is 1) from phi_in into phi_out, dphi from dphi_in into dphi_out
+// (may be equal).
 cudaError_t launch_step_io(const Geo& g, int precision, bool repro, const void* phi_in, void* phi_out,
                            const void* dphi_in, void* dphi_out, const double* c1, const double* c2, const double* cV,
                            int nsteps_in_pass, const double run_const[6], unsigned int* err, cudaStream_t st);
@@ -144,12 +145,11 @@ cudaError_t launch_measure(const Geo& g, int precision, bool fast, const void* p
 // Fast FP32 kernels (prs_fast.cu) for x sides that are multiples of 128.
 bool fast_step_ok(const Geo& g, int precision);
 
-// Two fused leapfrog steps per pass (prs_tblock.cu), FP32 3D and 2D; dphi out of place.
+// Two fused leapfrog steps per pass (prs_tblock.cu), FP32 3D; dphi out of place.
 bool tblock_ok(const Geo& g, int precision);
 // Rows of y per tile of the 3D two-step pass (0 when it does not apply).
 int tblock3_rows(const Geo& g);
-// phi_mid, v_mid (3D only; both or neither): also store the state between the two
-// steps there (cudaErrorNotSupported in 2D).
+// phi_mid, v_mid (both or neither): also store the state between the two steps there.
 cudaError_t launch_step_t2(const Geo& g, const float* phi_in, float* phi_out, const float* v_in, float* v_out,
                            KickF k0, KickF k1, RunConst<float> rc, unsigned int* err, cudaStream_t st,
                            float* phi_mid = nullptr, float* v_mid = nullptr);
@@ -168,16 +168,6 @@ bool t3tma_ok(const Geo& g);
 cudaError_t launch_step_t3_tma(const Geo& g, const float* phi_in, float* phi_out, const float* v_in, float* v_out,
                                KickF k0, KickF k1, KickF k2, RunConst<float> rc, unsigned int* err, cudaStream_t st,
                                int width = 0);
-
-// Three fused leapfrog steps per pass on FP32 2D boxes (prs_t3_2d.cu): x sides that are
-// multiples of 128 up to 4096; dphi out of place.
-bool t3_2d_ok(const Geo& g);
-cudaError_t launch_step_t3_2d(const Geo& g, const float* phi_in, float* phi_out, const float* v_in, float* v_out,
-                              KickF k0, KickF k1, KickF k2, RunConst<float> rc, unsigned int* err, cudaStream_t st);
-
-// One three-step pass on whichever kernel takes the box (3D tensor-copy tiles or 2D rows).
-cudaError_t launch_step_t3(const Geo& g, const float* phi_in, float* phi_out, const float* v_in, float* v_out,
-                           KickF k0, KickF k1, KickF k2, RunConst<float> rc, unsigned int* err, cudaStream_t st);
 
 // Store a message for prs_last_error() on this thread.
 void record_error(const char* msg);

@@ -1,0 +1,46 @@
+// prs_march2d.h -- launching the 2D register march (prs_march2d.cuh).
+#pragma once
+
+#include "prs_internal.h"
+
+namespace prs {
+
+constexpr int kMarchMaxT = 6;      // steps per pass
+constexpr int kMarchMaxRuns = 16;  // runs of one box per launch
+
+// The state of one FP32 run and the steps of a pass over it: coefficients (c1, c2, cV) of each
+// step and the run's constants (the layout of RunConst).
+struct MarchRun {
+    const void* phi_in;
+    void* phi_out;
+    const void* v_in;
+    void* v_out;  // may be v_in when t == 1
+    double coef[kMarchMaxT][3];
+    const double* run_const;
+};
+
+// How a pass is cut: columns a lane owns (2 or 4) and rows a warp marches.
+struct MarchShape {
+    int cols, cy;
+};
+
+// Shapes and modelled times (us, with the launch) of the passes of 1 .. kMarchMaxT steps over nruns
+// runs of a box.
+struct MarchPlan {
+    int nruns;  // 0: not made yet
+    MarchShape shape[kMarchMaxT + 1];
+    double us[kMarchMaxT + 1];
+};
+void march_plan(const Geo& g, int nruns, MarchPlan* p);
+
+// The passes of a call of n steps (>= 1): cnt[t] of t steps each, the longest first.  home: dphi has
+// to end in the buffer it started in, so that the passes of two steps and more, which alternate
+// between two buffers, are even in number or leave a single step to bring it back.
+void march_counts(const MarchPlan& p, int64_t n, bool home, int64_t cnt[kMarchMaxT + 1]);
+
+// One pass of t steps (1 .. kMarchMaxT) over nruns (1 .. kMarchMaxRuns) runs of the 2D box g, any
+// sides (several runs: x sides that are multiples of 128).
+cudaError_t launch_march2d(const Geo& g, int t, const MarchShape& shape, int nruns, const MarchRun* runs,
+                           cudaStream_t st);
+
+}  // namespace prs

@@ -8,6 +8,7 @@
 
 #include "prs.h"
 #include "prs_internal.h"
+#include "prs_march2d.h"
 
 struct prs_sim {
     prs_params p;
@@ -23,6 +24,7 @@ struct prs_sim {
     int64_t n;           // step index of the state
     double rc[6];        // deta, 1/dx^2, 1/phi0^2, 2D, V0, phi0
     prs::DiagScratch scr;
+    prs::MarchPlan march;     // FP32 2D: the passes' shapes and times, for this run or a group it leads
     prs::DevStatus* d_status; // device: result, counter, error word
     prs::DevStatus* h_status; // pinned host copy
     void* dphi_alt;           // second dphi buffer for passes that read dphi across sites (library-owned)
@@ -54,10 +56,9 @@ int check_device_error(prs_sim* s);
 // Queue the Eq. 7/8 sums of the run's current state into *result (device memory), without
 // waiting for them.
 int queue_diagnostics(prs_sim* s, DiagAcc* result);
-// Step each of several runs by nsteps as prs_step would step it alone (the same passes in the
-// same order, so the same fields), issuing each round of 2D three-step passes and of single
-// steps as one launch over all the runs when they share a box, stream and plan (at most
-// kT3MaxRuns); else one run after another.
+// Step each of several runs by nsteps: FP32 2D runs that share a box and stream (x sides that are
+// multiples of 128, at most kMarchMaxRuns) pass by pass in one launch over all the runs, else one run
+// after another.  The fields do not depend on how steps group into passes.
 int step_runs(prs_sim* const* runs, int nruns, int64_t nsteps);
 // PRS_DEBUG: the checks after a call that returned rc (prs_debug.cu); scan_state adds
 // the non-finite scan of the state.  Returns rc when the run has no PRS_DEBUG.

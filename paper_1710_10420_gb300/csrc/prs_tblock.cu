@@ -1,4 +1,4 @@
-// prs_tblock.cu -- two leapfrog steps (Eqs. 3-5) per pass over HBM, FP32 3D and 2D.
+// prs_tblock.cu -- two leapfrog steps (Eqs. 3-5) per pass over HBM, FP32 3D.
 //
 // One pass reads phi^n, dphi^{n-1/2} once and writes phi^{n+2}, dphi^{n+3/2} once:
 // 16 bytes per two site-updates.
@@ -230,173 +230,6 @@ __global__ void __launch_bounds__(XW == 128 && TY == 8 ? 160 : kTbThreads, XW ==
     }
 }
 
-// 2D: a CTA owns the rows [y0, y0+yn) of a chunk and marches along y through the same
-// two levels on whole rows (x neighbours by shuffle, the periodic wrap by lanes 0/31):
-//   level 1 (step n)   on rows y0-1 .. y0+yn, from level-0 rows y0-2 .. y0+yn+1 that the
-//                       TMA engine stages in a ring of kR2Slots0 rows;
-//   level 2 (step n+1) on rows y0 .. y0+yn-1, from level-1 rows kept in a ring of
-//                       kR2Slots1 rows.
-// Iteration t runs level 1 on local rows 2t-1, 2t and level 2 on rows 2t-4, 2t-3, whose
-// level-1 rows (up to 2t-2) were written an iteration earlier: one barrier per two rows.
-// y is the marching direction, so the only recomputed level-1 rows are the two outside
-// the chunk.  As in 3D, dphi enters those rows from the neighbouring chunks, so it is read
-// from one buffer and written to another; the level-1 dphi stays in the registers of the
-// thread that owns its columns.
-constexpr int kTb2Threads = 512;
-constexpr int kR2Ahead = 1;                   // iterations of level-0 rows in flight
-constexpr int kR2Slots0 = 4 + 2 * kR2Ahead;  // level-0 ring rows
-constexpr int kR2Slots1 = 6;                 // level-1 ring rows
-
-static __device__ __noinline__ void drain_rows(uint64_t* bar, int from, int issued, unsigned int* err)
-{
-    for (int i = from; i <= issued; ++i) mbar_wait(&bar[i % kR2Slots0], (i / kR2Slots0) & 1, err);
-}
-
-// NX > 0: the row width as a compile-time constant (the 4096-wide production box).
-template <int ITEMS, int NX>
-__global__ void __launch_bounds__(kTb2Threads, 1)
-    k_step2d_t2(const float* __restrict__ phi_in, float* __restrict__ phi_out, const float* __restrict__ v_in,
-                  float* __restrict__ v_out, int nx_, int ny, int cy, KickP p0, KickP p1, unsigned int* err)
-{
-    const int nx = NX > 0 ? NX : nx_;
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
-    float* ring0 = reinterpret_cast<float*>(smem_raw + 128);
-    float* ring1 = ring0 + kR2Slots0 * nx;
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int y0 = blockIdx.x * cy;
-    const int yn = min(cy, ny - y0);
-    const int nq = nx >> 2;
-
-    if (tid == 0) {
-#pragma unroll
-        for (int i = 0; i < kR2Slots0; ++i) mbar_init(&bar[i], 1);
-        mbar_fence_init();
-    }
-    __syncthreads();
-
-    auto wy = [&](int y) {
-        while (y < 0) y += ny;
-        while (y >= ny) y -= ny;
-        return y;
-    };
-    const unsigned rowb = (unsigned)nx * 4u;
-    const int nload = yn + 4;  // level-0 local rows 0..yn+3 = global y0-2 .. y0+yn+1
-    auto issue = [&](int i) {  // level-0 local row i
-        uint64_t* b = &bar[i % kR2Slots0];
-        mbar_arrive_expect_tx(b, rowb);
-        bulk_g2s(ring0 + (i % kR2Slots0) * nx, phi_in + (size_t)wy(y0 - 2 + i) * nx, rowb, b);
-    };
-    // iteration t waits for rows 2t, 2t+1 and issues the two rows iteration t + kR2Ahead waits for;
-    // before the first iteration every slot of the ring is free, so the rows of the first
-    // iterations are all in flight at once instead of one iteration's latency apart
-    int issued = -1;
-    if (tid == 0)
-        for (int i = 0; i < kR2Slots0 && i < nload; ++i) issue(i), issued = i;
-
-    int col[ITEMS];
-    bool on[ITEMS];
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-        const int q = tid + kTb2Threads * j;
-        on[j] = q < nq;
-        col[j] = on[j] ? q : 0;
-    }
-    // dphi^{n-1/2} of level-1 rows 2t-1, 2t (a: now, b: loaded for the next iteration)
-    float4 va0[ITEMS], va1[ITEMS], vb0[ITEMS], vb1[ITEMS];
-    // level-1 dphi^{n+1/2}: even rows for two iterations, odd rows for one
-    float4 e0[ITEMS], e1[ITEMS], o0[ITEMS];
-    auto load_v = [&](int jl, float4* dst) {
-        if (jl < 1 || jl > yn + 2) return;
-        const float* vp = v_in + (size_t)wy(y0 - 2 + jl) * nx;
-#pragma unroll
-        for (int j = 0; j < ITEMS; ++j)
-            if (on[j]) dst[j] = ldg_stream4(vp + 4 * col[j]);
-    };
-
-    // ring slots by rotation: level-0 row r sits in slot r mod kR2Slots0, level-1 row r in slot
-    // r mod kR2Slots1; an iteration advances every row index by two
-    auto level1 = [&](int jr, int sm, const float4* vin, float4* vout) {  // sm = (jr - 1) mod kR2Slots0
-        if (jr < 1 || jr > yn + 2) return;
-        const int sc = sm + 1 == kR2Slots0 ? 0 : sm + 1, sp = sc + 1 == kR2Slots0 ? 0 : sc + 1;
-        const float* pm = ring0 + sm * nx;
-        const float* pc = ring0 + sc * nx;
-        const float* pp = ring0 + sp * nx;
-        float* l1 = ring1 + (jr % kR2Slots1) * nx;
-#pragma unroll
-        for (int j = 0; j < ITEMS; ++j) {
-            if (!on[j]) continue;
-            const float4 c = lds4(pc + 4 * col[j]);
-            float left, right;
-            x_halo(pc, col[j], nq, nx, lane, c, left, right);
-            const float4 ym = lds4(pm + 4 * col[j]);
-            float4 pn;
-            float4 vv = vin[j];
-            update4p<false>(c, left, right, lds4(pp + 4 * col[j]), ym, ym, ym, vv, pn, p0);
-            *reinterpret_cast<float4*>(l1 + 4 * col[j]) = pn;
-            vout[j] = vv;
-        }
-    };
-    auto level2 = [&](int kr, const float4* vin) {
-        if (kr < 2 || kr > yn + 1) return;
-        const int sc = kr % kR2Slots1, sm = sc == 0 ? kR2Slots1 - 1 : sc - 1, sp = sc + 1 == kR2Slots1 ? 0 : sc + 1;
-        const float* pm = ring1 + sm * nx;
-        const float* pc = ring1 + sc * nx;
-        const float* pp = ring1 + sp * nx;
-        const size_t ro = (size_t)(y0 - 2 + kr) * nx;
-#pragma unroll
-        for (int j = 0; j < ITEMS; ++j) {
-            if (!on[j]) continue;
-            const float4 c = lds4(pc + 4 * col[j]);
-            float left, right;
-            x_halo(pc, col[j], nq, nx, lane, c, left, right);
-            const float4 ym = lds4(pm + 4 * col[j]);
-            float4 pn;
-            float4 vv = vin[j];
-            update4p<false>(c, left, right, lds4(pp + 4 * col[j]), ym, ym, ym, vv, pn, p1);
-            stg4(phi_out + ro + 4 * col[j], pn);
-            stg4(v_out + ro + 4 * col[j], vv);
-        }
-    };
-
-    const int tmax = (yn + 5) / 2;  // last iteration: level-2 row 2t-3 or 2t-4 reaches yn+1
-    int s0 = kR2Slots0 - 2;         // (2t - 2) mod kR2Slots0: slot of level-1 row 2t-1's row below
-    for (int t = 0; t <= tmax; ++t) {
-        bool ok = true;
-        for (int i = 2 * t; i <= 2 * t + 1; ++i)  // rows 2t, 2t+1 (rows below were waited earlier)
-            if (i < nload) ok = ok && mbar_wait(&bar[i % kR2Slots0], (i / kR2Slots0) & 1, err);
-        if (__syncthreads_or(!ok)) {
-            if (tid == 0) drain_rows(bar, 2 * t, issued, err);
-            return;
-        }
-        // rows 2(t+kR2Ahead) and the next, into the slots of rows 2t-4 and 2t-3 (last read by
-        // level 1 at iteration t-1; level 1 now reads rows 2t-2 .. 2t+1)
-        if (tid == 0)
-            for (int i = max(issued + 1, 2 * (t + kR2Ahead)); i <= 2 * (t + kR2Ahead) + 1 && i < nload; ++i)
-                issue(i), issued = i;
-#pragma unroll
-        for (int j = 0; j < ITEMS; ++j) va0[j] = vb0[j], va1[j] = vb1[j];
-        load_v(2 * t + 1, vb0);  // for iteration t+1: rows 2t+1, 2t+2
-        load_v(2 * t + 2, vb1);
-        float4 no[ITEMS], ne[ITEMS];
-        const int s1 = s0 + 1 == kR2Slots0 ? 0 : s0 + 1;  // (2t - 1) mod kR2Slots0
-        level1(2 * t - 1, s0, va0, no);
-        level1(2 * t, s1, va1, ne);
-        level2(2 * t - 4, e0);
-        level2(2 * t - 3, o0);
-#pragma unroll
-        for (int j = 0; j < ITEMS; ++j) {
-            e0[j] = e1[j];
-            e1[j] = ne[j];
-            o0[j] = no[j];
-        }
-        s0 += 2;
-        if (s0 >= kR2Slots0) s0 -= kR2Slots0;
-    }
-}
-
-size_t smem2d_t2(int nx) { return 128 + (kR2Slots0 + kR2Slots1) * (size_t)nx * sizeof(float); }
-
 constexpr size_t kTbSmemMax = 160 * 1024;
 
 // Tile of a 3D two-step pass: xw columns (128 for x sides up to 256, four CTAs per SM;
@@ -489,7 +322,7 @@ cudaError_t launch3(const Geo& g, const float* phi_in, float* phi_out, const flo
 bool tblock_ok(const Geo& g, int precision)
 {
     if (precision != PRS_FP32 || g.nx % 128 != 0) return false;
-    if (g.dims == 2) return g.nx <= 2 * kTb2Threads * 4;  // at most two float4 per thread of a row
+    if (g.dims == 2) return g.nx <= 4096;
     Tile3 t;
     return plan3(g, &t);
 }
@@ -504,36 +337,7 @@ cudaError_t launch_step_t2(const Geo& g, const float* phi_in, float* phi_out, co
                            KickF k0, KickF k1, RunConst<float> rc, unsigned int* err, cudaStream_t st,
                            float* phi_mid, float* v_mid)
 {
-    if (g.dims == 2) {
-        if (phi_mid || v_mid) return cudaErrorNotSupported;
-        const KickP p0 = kick_packed(k0, rc.deta), p1 = kick_packed(k1, rc.deta);
-        static std::atomic<unsigned long long> attr1{0}, attr2{0};
-        const size_t sm = smem2d_t2(g.nx);
-        const int sms = sm_count_current();
-        const int cy = (g.ny + sms - 1) / sms;
-        const int blocks = (g.ny + cy - 1) / cy;
-        if (g.nx / 4 > kTb2Threads) {
-            const cudaError_t e =
-                smem_limit_once(attr2, (const void*)k_step2d_t2<2, 0>, (int)smem2d_t2(8 * kTb2Threads));
-            if (e != cudaSuccess) return e;
-            static std::atomic<unsigned long long> attr4{0};
-            const cudaError_t e4 = smem_limit_once(attr4, (const void*)k_step2d_t2<2, 4096>, (int)smem2d_t2(4096));
-            if (e4 != cudaSuccess) return e4;
-            if (g.nx == 4096)
-                k_step2d_t2<2, 4096>
-                    <<<blocks, kTb2Threads, sm, st>>>(phi_in, phi_out, v_in, v_out, g.nx, g.ny, cy, p0, p1, err);
-            else
-                k_step2d_t2<2, 0>
-                    <<<blocks, kTb2Threads, sm, st>>>(phi_in, phi_out, v_in, v_out, g.nx, g.ny, cy, p0, p1, err);
-        } else {
-            const cudaError_t e =
-                smem_limit_once(attr1, (const void*)k_step2d_t2<1, 0>, (int)smem2d_t2(4 * kTb2Threads));
-            if (e != cudaSuccess) return e;
-            k_step2d_t2<1, 0>
-                <<<blocks, kTb2Threads, sm, st>>>(phi_in, phi_out, v_in, v_out, g.nx, g.ny, cy, p0, p1, err);
-        }
-        return cudaGetLastError();
-    }
+    if (g.dims != 3) return cudaErrorNotSupported;
     if ((phi_mid == nullptr) != (v_mid == nullptr)) return cudaErrorInvalidValue;
     if (t2tma_ok(g)) {  // the production tile: planes staged by tensor copies
         const cudaError_t e = launch_step_t2_tma(g, phi_in, phi_out, v_in, v_out, k0, k1, rc, err, st, phi_mid, v_mid);
