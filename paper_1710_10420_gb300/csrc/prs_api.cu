@@ -11,6 +11,7 @@
 
 #include "prs.h"
 #include "prs_internal.h"
+#include "prs_march3d.h"
 #include "prs_sim.h"
 
 using namespace prs;
@@ -153,10 +154,16 @@ extern "C" int prs_max_tblock(const prs_params* params)
 
 static const int kMeasureBlocks = 8192;  // partial slots: the fast kernels use one per tile
 
-// FP32 2D runs step by the register march (prs_march2d.cuh); without a tblock the march also plans
-// the steps of its passes.
-static bool march_run(const prs_sim* s) { return s->g.dims == 2 && s->p.precision == PRS_FP32; }
+// FP32 runs step by the register marches (prs_march2d.cuh, prs_march3d.cuh; in 3D beside the staged
+// passes); without a tblock their plan also sets the steps of the passes.
+static bool march_run(const prs_sim* s) { return s->p.precision == PRS_FP32; }
 static bool march_plans(const prs_sim* s) { return march_run(s) && s->p.tblock == 0; }
+static void make_plan(prs_sim* s, int nruns)
+{
+    if (s->march.nruns == nruns) return;
+    if (s->g.dims == 2) march_plan(s->g, nruns, &s->march);
+    else march_plan_3d(s->g, nruns, &s->march);
+}
 
 extern "C" int prs_create(const prs_params* params, void* stream, prs_sim** out)
 {
@@ -177,7 +184,7 @@ extern "C" int prs_create(const prs_params* params, void* stream, prs_sim** out)
     s->rc[4] = potential_height(*params);
     s->rc[5] = params->phi0;
     s->scr.max_blocks = kMeasureBlocks;
-    if (march_run(s)) march_plan(g, 1, &s->march);
+    if (march_run(s)) make_plan(s, 1);
     void* blob = nullptr;
     size_t bytes = sizeof(DiagAcc) * kMeasureBlocks + sizeof(DevStatus);
     if (cudaMalloc(&blob, bytes) != cudaSuccess) {
@@ -452,28 +459,26 @@ bool prs::cfl_ok_over(const prs_params& p, int64_t n, int64_t nsteps)
 // The passes of a call of nsteps (>= 1): cnt[t] of t steps, the longest first.
 static void step_plan(const prs_sim* s, const MarchPlan* march, int64_t nsteps, int64_t cnt[kMarchMaxT + 1])
 {
-    const bool repro = (s->p.flags & PRS_REPRO) != 0;
     const int tb = run_tblock(s);
     // Multi-step passes read dphi across sites, so they write it to a second buffer.  A call runs its
-    // passes the longest first, single steps last: with T = tblock = 3, nsteps / 3 triples and a pair
-    // or a single step for the remainder; with T = 2, pairs, and for an odd count a single step, or,
-    // when the library chooses the steps per pass (tblock = 0) and the box takes three-step passes,
-    // one triple instead of a pair and a single step; in FP32 2D without a tblock what march_counts
-    // plans.  After an odd number of multi-step passes dphi sits in the second buffer.  A run whose
+    // passes the longest first, single steps last: FP32 without a tblock what march_counts plans; else
+    // with T = tblock = 3, nsteps / 3 triples and a pair or a single step for the remainder; with T = 2,
+    // pairs, and for an odd count a single step.  After an odd number of multi-step passes dphi sits in the second buffer.  A run whose
     // buffers the library owns (no PRS_DEBUG guard bands) then swaps the roles of its two dphi
     // buffers.  A run with bound buffers keeps dphi in the bound buffer at the end of every call: the
     // first single step after an odd number of multi-step passes reads dphi in the second buffer and
-    // writes the bound one; with no single step to do it, the triple of an odd T = 2 count runs as a
-    // pair and a single step, else the last pair as two single steps, else the last triple as a pair
-    // and a single step.  Single steps otherwise update dphi in place.
+    // writes the bound one; with no single step to do it, the last pair runs as two single steps, else
+    // the last triple as a pair and a single step.  Single steps otherwise update dphi in place.
     const bool swap_ok = s->owned && (s->p.flags & PRS_DEBUG) == 0;
     for (int t = 0; t <= kMarchMaxT; ++t) cnt[t] = 0;
-    if (!s->dphi_alt) {  // no second buffer (no room at prs_init)
+    // no second buffer (no room at prs_init), or planes beyond the march's offsets
+    if (!s->dphi_alt || (s->g.dims == 3 && !march3d_ok(s->g))) {
         cnt[1] = nsteps;
         return;
     }
     if (march_plans(s)) {
-        march_counts(*march, nsteps, !swap_ok, cnt);
+        if (s->g.dims == 2) march_counts(*march, nsteps, !swap_ok, cnt);
+        else march_counts_3d(*march, nsteps, !swap_ok, cnt);
         return;
     }
     int64_t n3 = 0, n2 = 0, n1 = nsteps;
@@ -484,12 +489,9 @@ static void step_plan(const prs_sim* s, const MarchPlan* march, int64_t nsteps, 
     } else if (tb == 2) {
         n2 = nsteps / 2;
         n1 = nsteps - 2 * n2;
-        if (n1 == 1 && n2 >= 1 && s->p.tblock == 0 && max_fused_steps(s->g, s->p.precision, repro) >= 3)
-            n3 = 1, n2 -= 1, n1 = 0;
     }
     if (((n3 + n2) & 1) && n1 == 0 && !swap_ok) {
-        if (tb == 2 && n3 == 1) n3 = 0, n2 += 1, n1 = 1;
-        else if (n2 > 0) n2 -= 1, n1 += 2;
+        if (n2 > 0) n2 -= 1, n1 += 2;
         else n3 -= 1, n2 += 1, n1 += 1;
     }
     cnt[3] = n3, cnt[2] = n2, cnt[1] = n1;
@@ -505,31 +507,22 @@ static cudaError_t queue_pass(prs_sim* s, int t, int64_t n, const void* v_in, vo
     void* out = s->phi[1 - s->cur];
     double c[kMarchMaxT][5];
     for (int l = 0; l < t; ++l) step_coefficients(s->p, n + l, c[l]);
-    cudaError_t e;
-    if (march_run(s)) {
+    cudaError_t e = cudaErrorNotSupported;
+    if (t == 2 && s->g.dims == 3 && (s->march.shape[2].cols == 0 || !march3d_ok(s->g))) {
+        const RunConst<float> rcf{(float)s->rc[0], (float)s->rc[1], (float)s->rc[2],
+                                  (float)s->rc[3], (float)s->rc[4], (float)s->rc[5]};
+        e = launch_step_t2(s->g, (const float*)in, (float*)out, (const float*)v_in, (float*)v_out,
+                           kick_f32(c[0], s->rc), kick_f32(c[1], s->rc), rcf, err, s->stream);
+    }
+    if (e == cudaErrorNotSupported && march_run(s) && (t > 1 || s->march.shape[1].cols)) {
         MarchRun r{in, out, v_in, v_out, {}, s->rc};
         for (int l = 0; l < t; ++l)
             for (int q = 0; q < 3; ++q) r.coef[l][q] = c[l][q];
-        e = launch_march2d(s->g, t, s->march.shape[t], 1, &r, s->stream);
-    } else if (t == 1) {
+        e = s->g.dims == 2 ? launch_march2d(s->g, t, s->march.shape[t], 1, &r, s->stream)
+                           : launch_march3d(s->g, t, s->march.shape[t].cy, 1, &r, s->stream);
+    } else if (e == cudaErrorNotSupported) {
         e = launch_step_io(s->g, s->p.precision, repro, in, out, v_in, v_out, &c[0][0], &c[0][1], &c[0][2], 1, s->rc,
                            err, s->stream);
-    } else {
-        const RunConst<float> rcf{(float)s->rc[0], (float)s->rc[1], (float)s->rc[2],
-                                  (float)s->rc[3], (float)s->rc[4], (float)s->rc[5]};
-        const KickF k0 = kick_f32(c[0], s->rc), k1 = kick_f32(c[1], s->rc);
-        e = t == 3 ? launch_step_t3_tma(s->g, (const float*)in, (float*)out, (const float*)v_in, (float*)v_out, k0, k1,
-                                        kick_f32(c[2], s->rc), rcf, err, s->stream)
-                   : launch_step_t2(s->g, (const float*)in, (float*)out, (const float*)v_in, (float*)v_out, k0, k1,
-                                    rcf, err, s->stream);
-        if (t == 3 && e == cudaErrorNotSupported) {  // no tensor-map encoder: a pair, then a single step in place
-            e = launch_step_t2(s->g, (const float*)in, (float*)out, (const float*)v_in, (float*)v_out, k0, k1, rcf, err,
-                               s->stream);
-            if (e == cudaSuccess)
-                e = launch_step_io(s->g, s->p.precision, repro, out, s->phi[s->cur], v_out, v_out, &c[2][0], &c[2][1],
-                                   &c[2][2], 1, s->rc, err, s->stream);
-            s->cur = 1 - s->cur;  // phi ends where it started; the flip below undoes this
-        }
     }
     s->cur = 1 - s->cur;
     return e;
@@ -541,7 +534,7 @@ static int prs_step_impl(prs_sim* s, int64_t nsteps)
     if (!s->initialised) return PRS_ESTATE;
     if (nsteps == 0) return PRS_OK;
     if (!cfl_ok_over(s->p, s->n, nsteps)) return PRS_EINVAL;
-    if (march_run(s) && s->march.nruns != 1) march_plan(s->g, 1, &s->march);
+    if (march_run(s)) make_plan(s, 1);
     int64_t cnt[kMarchMaxT + 1];
     step_plan(s, &s->march, nsteps, cnt);
     void* vbuf[2] = {s->dphi, s->dphi_alt};
@@ -647,8 +640,8 @@ int prs::step_runs(prs_sim* const* runs, int nruns, int64_t nsteps)
         if (!s->initialised) return PRS_ESTATE;
         if (!cfl_ok_over(s->p, s->n, nsteps)) return PRS_EINVAL;
         const Geo &g = s->g, &g0 = runs[0]->g;
-        together = together && march_plans(s) && g.nx == g0.nx && g.ny == g0.ny && g.nx % 128 == 0 &&
-                   g.nx <= 4096 && s->stream == runs[0]->stream && s->dphi_alt && s->owned == runs[0]->owned &&
+        together = together && march_plans(s) && g.dims == g0.dims && g.nx == g0.nx && g.ny == g0.ny &&
+                   g.nz == g0.nz && g.nx % 128 == 0 && (g.dims == 2 ? g.nx <= 4096 : march3d_ok(g)) && s->stream == runs[0]->stream && s->dphi_alt && s->owned == runs[0]->owned &&
                    (s->p.flags & PRS_DEBUG) == 0;
     }
     if (!together) {
@@ -658,8 +651,8 @@ int prs::step_runs(prs_sim* const* runs, int nruns, int64_t nsteps)
         }
         return PRS_OK;
     }
-    MarchPlan& plan = runs[0]->march;
-    if (plan.nruns != nruns) march_plan(runs[0]->g, nruns, &plan);
+    make_plan(runs[0], nruns);
+    const MarchPlan& plan = runs[0]->march;
     int64_t cnt[kMarchMaxT + 1], done = 0;
     step_plan(runs[0], &plan, nsteps, cnt);
     MarchRun q[kMarchMaxRuns];
@@ -680,7 +673,9 @@ int prs::step_runs(prs_sim* const* runs, int nruns, int64_t nsteps)
                     for (int u = 0; u < 3; ++u) q[r].coef[l][u] = c[u];
                 }
             }
-            const cudaError_t e = launch_march2d(runs[0]->g, t, plan.shape[t], nruns, q, runs[0]->stream);
+            const cudaError_t e =
+                runs[0]->g.dims == 2 ? launch_march2d(runs[0]->g, t, plan.shape[t], nruns, q, runs[0]->stream)
+                                     : launch_march3d(runs[0]->g, t, plan.shape[t].cy, nruns, q, runs[0]->stream);
             if (e != cudaSuccess) return cuda_fail(e, "step_runs launch");
             for (int r = 0; r < nruns; ++r) runs[r]->cur = 1 - runs[r]->cur;
             vi = t > 1 ? 1 - vi : 0;

@@ -56,12 +56,15 @@ struct Fold32 {
     };
     static __device__ __forceinline__ P pair(float a, float b) { return P{pk2(a, b)}; }
     static __device__ __forceinline__ void split(P p, float& a, float& b) { upk2(p.r, a, b); }
-    static __device__ __forceinline__ P update(P m, P c, P p, float left, float right, P& v, const K& k, f2 dt,
-                                                const RunConst<float>&)
+    // D = 3: zp, zm are the neighbours along z
+    template <int D>
+    static __device__ __forceinline__ P update(P m, P c, P p, P zm, P zp, float left, float right, P& v, const K& k,
+                                                f2 dt, const RunConst<float>&)
     {
         float x, y;
         upk2(c.r, x, y);
-        const f2 s = add2(pk2(__fadd_rn(y, left), __fadd_rn(right, x)), add2(p.r, m.r));
+        f2 s = add2(pk2(__fadd_rn(y, left), __fadd_rn(right, x)), add2(p.r, m.r));
+        if (D == 3) s = add2(s, add2(zp.r, zm.r));
         const f2 u = mul2(c.r, fma2(f2{k.nk2}, mul2(c.r, c.r), f2{k.k1}));
         v.r = fma2(f2{k.c1}, v.r, fma2(f2{k.g}, s, u));
         return P{fma2(dt, v.r, c.r)};
@@ -78,12 +81,13 @@ struct Plain32 {
     };
     static __device__ __forceinline__ P pair(float a, float b) { return P{a, b}; }
     static __device__ __forceinline__ void split(P p, float& a, float& b) { a = p.a, b = p.b; }
-    static __device__ __forceinline__ P update(P m, P c, P p, float left, float right, P& v, const K& k, f2,
-                                                const RunConst<float>& rc)
+    template <int D>
+    static __device__ __forceinline__ P update(P m, P c, P p, P zm, P zp, float left, float right, P& v, const K& k,
+                                                f2, const RunConst<float>& rc)
     {
         P n;
-        site_update<float, false, 2>(c.a, c.b, left, p.a, m.a, 0.f, 0.f, v.a, n.a, k, rc);
-        site_update<float, false, 2>(c.b, right, c.a, p.b, m.b, 0.f, 0.f, v.b, n.b, k, rc);
+        site_update<float, false, D>(c.a, c.b, left, p.a, m.a, zp.a, zm.a, v.a, n.a, k, rc);
+        site_update<float, false, D>(c.b, right, c.a, p.b, m.b, zp.b, zm.b, v.b, n.b, k, rc);
         return n;
     }
 };
@@ -234,8 +238,8 @@ __global__ void __launch_bounds__(kThreads, resident(T, COLS)) k_march2d(const _
             P n[NP];
 #pragma unroll
             for (int j = 0; j < NP; ++j) {
-                n[j] = M::update(m[l][j], c[l][j], p[j], j == 0 ? left : f[2 * j - 1], j == NP - 1 ? right : f[2 * j + 2],
-                                 v[j], k, dt, rc);
+                n[j] = M::template update<2>(m[l][j], c[l][j], p[j], p[j], p[j], j == 0 ? left : f[2 * j - 1],
+                                             j == NP - 1 ? right : f[2 * j + 2], v[j], k, dt, rc);
                 m[l][j] = c[l][j];
                 c[l][j] = p[j];
                 p[j] = n[j];

@@ -19,24 +19,27 @@ struct MarchRun {
     const double* run_const;
 };
 
-// How a pass is cut: columns a lane owns (2 or 4) and rows a warp marches.
+// How a pass is cut: columns a lane owns (2 or 4; 3D: 2) and rows (3D: planes) a warp marches.  cols
+// 0: the pass is not the march's (3D boxes of the staged passes).
 struct MarchShape {
     int cols, cy;
 };
 
-// Shapes and modelled times (us, with the launch) of the passes of 1 .. kMarchMaxT steps over nruns
-// runs of a box.
+// Shapes and modelled times (us, with the launch) of the passes of 1 .. kMarchMaxT (3D: kMarch3MaxT)
+// steps over nruns FP32 runs of a box.
 struct MarchPlan {
     int nruns;  // 0: not made yet
     MarchShape shape[kMarchMaxT + 1];
     double us[kMarchMaxT + 1];
 };
-void march_plan(const Geo& g, int nruns, MarchPlan* p);
+void march_plan(const Geo& g, int nruns, MarchPlan* p);     // 2D
+void march_plan_3d(const Geo& g, int nruns, MarchPlan* p);  // 3D
 
 // The passes of a call of n steps (>= 1): cnt[t] of t steps each, the longest first.  home: dphi has
 // to end in the buffer it started in, so that the passes of two steps and more, which alternate
 // between two buffers, are even in number or leave a single step to bring it back.
-void march_counts(const MarchPlan& p, int64_t n, bool home, int64_t cnt[kMarchMaxT + 1]);
+void march_counts(const MarchPlan& p, int64_t n, bool home, int64_t cnt[kMarchMaxT + 1]);     // 2D
+void march_counts_3d(const MarchPlan& p, int64_t n, bool home, int64_t cnt[kMarchMaxT + 1]);  // 3D
 
 // One pass of t steps (1 .. kMarchMaxT) over nruns (1 .. kMarchMaxRuns) runs of the 2D box g, any
 // sides (several runs: x sides that are multiples of 128).

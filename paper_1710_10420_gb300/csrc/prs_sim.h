@@ -24,7 +24,7 @@ struct prs_sim {
     int64_t n;           // step index of the state
     double rc[6];        // deta, 1/dx^2, 1/phi0^2, 2D, V0, phi0
     prs::DiagScratch scr;
-    prs::MarchPlan march;     // FP32 2D: the passes' shapes and times, for this run or a group it leads
+    prs::MarchPlan march;     // FP32: the passes' shapes and times, for this run or a group it leads
     prs::DevStatus* d_status; // device: result, counter, error word
     prs::DevStatus* h_status; // pinned host copy
     void* dphi_alt;           // second dphi buffer for passes that read dphi across sites (library-owned)
@@ -56,7 +56,7 @@ int check_device_error(prs_sim* s);
 // Queue the Eq. 7/8 sums of the run's current state into *result (device memory), without
 // waiting for them.
 int queue_diagnostics(prs_sim* s, DiagAcc* result);
-// Step each of several runs by nsteps: FP32 2D runs that share a box and stream (x sides that are
+// Step each of several runs by nsteps: FP32 runs that share a box and stream (x sides that are
 // multiples of 128, at most kMarchMaxRuns) pass by pass in one launch over all the runs, else one run
 // after another.  The fields do not depend on how steps group into passes.
 int step_runs(prs_sim* const* runs, int nruns, int64_t nsteps);

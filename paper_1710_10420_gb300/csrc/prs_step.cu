@@ -1,6 +1,6 @@
 // prs_step.cu -- chooses the kernel for one pass of fused leapfrog steps.
 #include "prs_internal.h"
-#include "prs_march2d.h"
+#include "prs_march3d.h"
 
 namespace prs {
 
@@ -20,13 +20,16 @@ KickF kick_f32(const double coef[3], const double run_const[6])
 // register march replaced; without a tblock the march takes any FP32 2D box, up to six steps a pass).
 static bool rows_ok(const Geo& g) { return g.dims == 2 && g.nx % 128 == 0 && g.nx <= 4096; }
 
+// The same for tblock = 3 on 3D boxes.
+static bool t3_ok(const Geo& g) { return g.nx % 128 == 0 && g.ny % 8 == 0 && g.ny >= 16 && g.nz >= 3; }
+
 // Steps one pass may fuse (params.tblock above this is clamped): three on the FP32 boxes the
 // three-step passes take, two on the other boxes of the two-step passes.
 int max_fused_steps(const Geo& g, int precision, bool repro)
 {
     (void)repro;
     if (!tblock_ok(g, precision)) return 1;
-    return (g.dims == 3 ? t3tma_ok(g) : rows_ok(g)) ? 3 : 2;
+    return (g.dims == 3 ? t3_ok(g) : rows_ok(g)) ? 3 : 2;
 }
 
 // The library's default number of steps per pass (us per step, one / two / three steps per
@@ -34,7 +37,7 @@ int max_fused_steps(const Geo& g, int precision, bool repro)
 // occupies the GPU best (128^3 8.3 / 15.4 / 11.0, 256^2 x 128 18.1 / 21.6 / 20.5); from 2^24 two
 // wherever the two-step pass gets tiles of at least 4 rows (256^3 46.7 / 32.8 / 34.3; 1024^3
 // 2.53 / 1.37 / 1.43 ms).  FP32 2D: nominal; the register march has a plan of its own
-// (march_counts).  FP64 and other boxes: one.
+// (march_counts), as has FP32 3D without a tblock (march_counts_3d).  FP64 and other boxes: one.
 int default_fused_steps(const Geo& g, int precision, bool repro)
 {
     (void)repro;
@@ -65,6 +68,10 @@ cudaError_t launch_step_io(const Geo& g, int precision, bool repro, const void* 
                            (float)run_const[4], (float)run_const[5]};
         return launch_step_fast(g, (const float*)phi_in, (float*)phi_out, (const float*)dphi_in, (float*)dphi_out, k,
                                 rc, err, st);
+    }
+    if (precision == PRS_FP32 && march3d_ok(g)) {
+        const MarchRun r{phi_in, phi_out, dphi_in, dphi_out, {{c1[0], c2[0], cV[0]}}, run_const};
+        return launch_march3d(g, 1, march3d_planes(g, 1, 1, nullptr), 1, &r, st);
     }
     return launch_step_generic(g, precision, repro, phi_in, phi_out, dphi_in, dphi_out, c1[0], c2[0], cV[0], run_const,
                                st);

@@ -343,8 +343,8 @@ cudaError_t launch_step_t2(const Geo& g, const float* phi_in, float* phi_out, co
         const cudaError_t e = launch_step_t2_tma(g, phi_in, phi_out, v_in, v_out, k0, k1, rc, err, st, phi_mid, v_mid);
         if (e != cudaErrorNotSupported) return e;
     }
-    if (phi_mid) return launch3<true>(g, phi_in, phi_out, v_in, v_out, phi_mid, v_mid, k0, k1, rc, err, st);
-    return launch3<false>(g, phi_in, phi_out, v_in, v_out, nullptr, nullptr, k0, k1, rc, err, st);
+    if (!phi_mid) return cudaErrorNotSupported;
+    return launch3<true>(g, phi_in, phi_out, v_in, v_out, phi_mid, v_mid, k0, k1, rc, err, st);
 }
 
 }  // namespace prs
