@@ -641,7 +641,7 @@ int prs::step_runs(prs_sim* const* runs, int nruns, int64_t nsteps)
         if (!cfl_ok_over(s->p, s->n, nsteps)) return PRS_EINVAL;
         const Geo &g = s->g, &g0 = runs[0]->g;
         together = together && march_plans(s) && g.dims == g0.dims && g.nx == g0.nx && g.ny == g0.ny &&
-                   g.nz == g0.nz && g.nx % 128 == 0 && (g.dims == 2 ? g.nx <= 4096 : march3d_ok(g)) && s->stream == runs[0]->stream && s->dphi_alt && s->owned == runs[0]->owned &&
+                   g.nz == g0.nz && march_packed(g) && (g.dims == 2 || march3d_ok(g)) && s->stream == runs[0]->stream && s->dphi_alt && s->owned == runs[0]->owned &&
                    (s->p.flags & PRS_DEBUG) == 0;
     }
     if (!together) {

@@ -6,7 +6,10 @@
 
 namespace prs {
 
-static bool packed(const Geo& g) { return fast_step_ok(g, PRS_FP32) || tblock_ok(g, PRS_FP32); }
+bool march_packed(const Geo& g)
+{
+    return fast_step_ok(g, PRS_FP32) || default_fused_steps(g, PRS_FP32, false) > 1;
+}
 
 // A warp's iteration takes the chain of its levels, or its scheduler's turns for all its warps,
 // whichever is longer; a pass takes its waves of iterations or its bytes, and a launch (2.3 us from
@@ -18,7 +21,7 @@ static bool packed(const Geo& g) { return fast_step_ok(g, PRS_FP32) || tblock_ok
 static double march_us(const Geo& g, int t, int nruns, MarchShape* best)
 {
     const int sms = sm_count_current();
-    const double plain = packed(g) ? 1.0 : 1.3;
+    const double plain = march_packed(g) ? 1.0 : 1.3;
     double least = 1e300;
     for (int cols = 2; cols <= 4; cols += 2) {
         const int u = march::width(t, cols);
@@ -69,8 +72,8 @@ cudaError_t launch_march2d(const Geo& g, int t, const MarchShape& shape, int nru
                            cudaStream_t st)
 {
     if (g.dims != 2 || nruns < 1 || nruns > kMarchMaxRuns) return cudaErrorInvalidValue;
-    if (nruns > 1 && !packed(g)) return cudaErrorNotSupported;
-    return packed(g) ? launch_march_fold32(g, t, shape, nruns, runs, st)
+    if (nruns > 1 && !march_packed(g)) return cudaErrorNotSupported;
+    return march_packed(g) ? launch_march_fold32(g, t, shape, nruns, runs, st)
                      : launch_march_plain32(g, t, shape, nruns, runs, st);
 }
 

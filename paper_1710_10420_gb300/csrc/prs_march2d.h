@@ -8,6 +8,10 @@ namespace prs {
 constexpr int kMarchMaxT = 6;      // steps per pass
 constexpr int kMarchMaxRuns = 16;  // runs of one box per launch
 
+// Whether an FP32 box steps by the folded kick of the staged passes (the boxes they take), else by the
+// generic step's arithmetic, whose rounding errors are a little smaller.
+bool march_packed(const Geo& g);
+
 // The state of one FP32 run and the steps of a pass over it: coefficients (c1, c2, cV) of each
 // step and the run's constants (the layout of RunConst).
 struct MarchRun {
@@ -42,7 +46,7 @@ void march_counts(const MarchPlan& p, int64_t n, bool home, int64_t cnt[kMarchMa
 void march_counts_3d(const MarchPlan& p, int64_t n, bool home, int64_t cnt[kMarchMaxT + 1]);  // 3D
 
 // One pass of t steps (1 .. kMarchMaxT) over nruns (1 .. kMarchMaxRuns) runs of the 2D box g, any
-// sides (several runs: x sides that are multiples of 128).
+// sides (several runs: march_packed boxes).
 cudaError_t launch_march2d(const Geo& g, int t, const MarchShape& shape, int nruns, const MarchRun* runs,
                            cudaStream_t st);
 

@@ -75,7 +75,7 @@ cudaError_t launch3(const Geo& g, int t, int nruns, const MarchRun* runs, cudaSt
 bool march3d_ok(const Geo& g) { return g.dims == 3 && (int64_t)g.nx * g.ny < ((int64_t)1 << 32); }
 
 // As march_us in 2D: a warp's iteration takes its instructions' latency or its scheduler's turns for
-// all its warps, a pass its iterations or its bytes (beyond L2 at 5 TB/s).  Waves of blocks count half
+// all its warps, a pass its iterations or its bytes (beyond L2 at 5.6 TB/s).  Waves of blocks count half
 // as whole and half as they fill, as measured from 67^3 to 1024^3: long chunks waste fewer of their
 // cz + 2t planes, short ones fill the GPU.
 int march3d_planes(const Geo& g, int t, int nruns, double* us)
@@ -87,28 +87,28 @@ int march3d_planes(const Geo& g, int t, int nruns, double* us)
     const double slots = (double)sms * march::resident3(t);
     double rows = 0.0;  // updates of an iteration, in rows
     for (int l = 1; l <= t; ++l) rows += march::kRows + 2 * (t - l);
-    const double turn = (fast_step_ok(g, PRS_FP32) || tblock_ok(g, PRS_FP32) ? 26.0 : 36.0) * rows + 30.0 * t + 70.0;
-    const double lone = 1.6 * turn + 300.0;
+    const double base = 380.0 + 36.0 * rows;  // cycles at 1.9 GHz
+    const double lone = (march_packed(g) ? 1.0 : 1.2) * base, turn = (march_packed(g) ? 0.72 : 0.95) * base;
     int best = 1;
     double least = 1e300;
     for (int nc = 1; nc <= g.nz && nc <= 4096; ++nc) {
         const int c = (g.nz + nc - 1) / nc, n = (g.nz + c - 1) / c;
         const double w = tiles * n / slots, at_once = w < 1.0 ? tiles * n : slots;
-        const double waves = w <= 1.0 ? 1.0 : 0.5 * (ceil(w) + w + 0.35);
-        const double cost = waves * (c + 2 * t) * std::max(lone, at_once / sms * turn);
+        const double waves = w <= 1.0 ? 1.1 - 0.1 * w : 0.5 * (ceil(w) + w + 0.35);
+        const double cost = waves * (c + 2 * t) * std::max(lone, ceil(at_once / sms) * turn);
         if (cost < least * 0.999) least = cost, best = c;
     }
     if (us) {
         const double bytes = 16.0 * (double)g.S * nruns;
-        *us = 2.3 + std::max(least / 1900.0, bytes > 1e8 ? bytes / 5.0e6 : bytes / 9.0e6);
+        *us = 3.5 + std::max(least / 1900.0, bytes / (bytes < 1e8 ? 9.0e6 : (t == 1 ? 6.2e6 : 5.6e6)));
     }
     return best;
 }
 
 // The staged passes stay where they are the faster: one step on the boxes they take (1024^3: 2.54 ms,
-// HBM; the march 2.8), two steps where the 256 x 8 tensor-copy tiles fit (us: 0.154 a MB of the state
-// crossing HBM twice and a start of up to 93, that is 2740 at 1024^3, 424 at 512^3 and 65 at 256^3;
-// the march 3370, 430 and 66).  Three steps are the march's: 3620, 510 and 80, which is the least
+// HBM; the march 2.8), two steps on large boxes where the 256 x 8 tensor-copy tiles fit (us: 0.154 a
+// MB of the state crossing HBM twice and a start of up to 93, that is 2740 at 1024^3, 424 at 512^3 and
+// 65 at 256^3; the march 3100, 395 and 60).  Three steps are the march's: 3620, 510 and 80, which is the least
 // time a step from 1024^3 down to 100^3.
 void march_plan_3d(const Geo& g, int nruns, MarchPlan* p)
 {
@@ -120,7 +120,7 @@ void march_plan_3d(const Geo& g, int nruns, MarchPlan* p)
     }
     if (nruns > 1) return;
     const double mb = 16e-6 * (double)g.S;
-    const double one = 2.3 + std::max(6.0, mb * 0.15), two = 2.3 + 0.154 * mb + std::min(93.0, 0.09 * mb);
+    const double one = 3.5 + std::max(6.5, mb * 0.15), two = 3.5 + 0.154 * mb + std::min(93.0, 0.09 * mb);
     if (fast_step_ok(g, PRS_FP32) || !march3d_ok(g)) p->shape[1].cols = 0, p->us[1] = one;
     if (t2tma_ok(g) && two < p->us[2]) p->shape[2].cols = 0, p->us[2] = two;
 }
@@ -150,7 +150,7 @@ void march_counts_3d(const MarchPlan& p, int64_t n, bool home, int64_t cnt[kMarc
 
 cudaError_t launch_march3d(const Geo& g, int t, int cz, int nruns, const MarchRun* runs, cudaStream_t st)
 {
-    const bool packed = fast_step_ok(g, PRS_FP32) || tblock_ok(g, PRS_FP32);
+    const bool packed = march_packed(g);
     if (!march3d_ok(g) || nruns < 1 || nruns > kMarchMaxRuns) return cudaErrorInvalidValue;
     if (nruns > 1 && !packed) return cudaErrorNotSupported;
     return packed ? march::launch3<march::Fold32>(g, t, nruns, runs, st, cz)

@@ -14,7 +14,7 @@ bool march3d_ok(const Geo& g);
 int march3d_planes(const Geo& g, int t, int nruns, double* us);
 
 // One pass of t steps (1 .. kMarch3MaxT) over nruns (1 .. kMarchMaxRuns) runs of the FP32 3D box g, any
-// sides (several runs: x sides that are multiples of 128); cz from march3d_planes.
+// sides (several runs: march_packed boxes); cz from march3d_planes.
 cudaError_t launch_march3d(const Geo& g, int t, int cz, int nruns, const MarchRun* runs, cudaStream_t st);
 
 }  // namespace prs
