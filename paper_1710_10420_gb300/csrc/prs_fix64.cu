@@ -1,0 +1,321 @@
+// prs_fix64.cu -- the FP64 leapfrog step (Eqs. 3-5, folded kick) with its force in 64-bit fixed point.
+//
+// What bounds the plain FP64 step: GB300 adds or multiplies two doubles a clock and SM, so its 11
+// (2D: 9) double operations a site take 350 us at 256^3, where HBM would allow 79 us.  An SM issues 64
+// integer instructions in the time of one double instruction of a warp.  So the force
+//   A = g (sum of the 2D neighbours) + phi (k1 - k2 phi^2)
+// is evaluated in integers, and only the kick c1 dphi + A and the drift phi + deta dphi' stay
+// double operations (one fused multiply-add each).
+//
+// With S the power of two at or above phi0, a value |phi| < 2 S becomes the integer phi/S 2^59,
+// whose neighbour sum is exact; three high-half products evaluate the cubic and one the
+// neighbour term, with the constants scaled so that A, times 2^(60 - ek) / S, fits 63 bits (ek: the
+// exponent that bounds the constants); A is then rounded to double once.  Its error is a few 2^-60 of
+// S 2^ek, where the double evaluation rounds each of its terms (6 g phi and its like) to 2^-54: the
+// step's error against 64-bit references is not larger (tests/test_gpu_fix64.py).  Products take the
+// magnitudes, so the step of a negated field is the negated step, bit for bit.
+//
+// The integers hold their precision absolutely, doubles relatively.  So each warp scales by an S of its
+// own, S 2^-down: it is lowered when the three planes of an iteration hold no value of a sixteenth of it
+// or more, and raised again when a plane needs it.  A warp that meets values at 2 phi0's S or beyond
+// (blow-ups) or not finite evaluates the double form.
+//
+// Measured (us a step; the double form): 256^3 163 (355), 512^3 1245 (2805), 128^3 29 (47), 2048^2 48
+// (74), 128^2 4.4 (4.2: the launch).  230 integer instructions a site at 0.6 of the issue slots now set
+// the pace.
+//
+// A warp owns 32 columns (30 outputs) of four rows (2D: one) and marches along z (2D: y): a value is
+// converted once where it enters, its z neighbours wait in registers, x neighbours come by shuffle.
+#include <cuda_runtime.h>
+#include <math.h>
+
+#include <algorithm>
+
+#include "prs_internal.h"
+#include "prs_site.cuh"
+
+namespace prs {
+
+namespace {
+
+typedef long long i64;
+typedef unsigned long long u64;
+
+constexpr int kFxThreads = 128, kFxWarps = kFxThreads / 32, kFxU = 30;
+constexpr int fx_blocks(int dims) { return dims == 3 ? 4 : 8; }  // CTAs an SM (registers)
+
+// The force's constants: k1, k2 S^2 and g scaled by 2^(62-ek), 2^(66-ek), 2^(65-ek); e_base: what a
+// value's exponent field is subtracted from for its shift; e_out: exponent field of an A of 2^63.
+struct Fix64 {
+    i64 k1;
+    u64 k2, g;
+    int e_base, e_out;
+};
+
+struct FixArgs {
+    const double* phi_in;
+    double* phi_out;
+    const double* v_in;
+    double* v_out;
+    Fix64 f;
+    KickD k;
+    double deta;
+    Geo g;
+    int nstrips, ygroups, cz;
+};
+
+// phi/S 2^59, rounded (halves away from zero); shift is 3 for S <= |phi| < 2 S and below 3 for larger
+// or non-finite values.
+__device__ __forceinline__ i64 to_fixed(double d, int e_base, int& shift)
+{
+    const int hi = __double2hiint(d);
+    const unsigned lo = (unsigned)__double2loint(d);
+    shift = e_base - ((hi >> 20) & 0x7ff);
+    const u64 m = ((u64)((hi & 0xfffff) | 0x100000) << 32 | lo) << 10;
+    const u64 a = shift > 63 ? 0ull : ((m >> ((shift - 1) & 63)) + 1) >> 1;
+    const i64 s = (i64)(hi >> 31);
+    return (i64)(a ^ (u64)s) - s;
+}
+
+// a times sign (0 or -1): its negation where sign is -1.
+__device__ __forceinline__ i64 with_sign(u64 a, i64 sign) { return (i64)(a ^ (u64)sign) - sign; }
+
+// a times 2^by, towards zero.
+__device__ __forceinline__ i64 rescaled(i64 a, int by)
+{
+    const i64 s = a >> 63;
+    const u64 m = (u64)with_sign((u64)a, s);
+    return with_sign(by >= 0 ? (by > 63 ? 0ull : m << by) : (by < -63 ? 0ull : m >> -by), s);
+}
+
+__device__ __forceinline__ double from_fixed(i64 a, int e_out)
+{
+    const i64 s = a >> 63;
+    const u64 m = (u64)with_sign((u64)a, s);
+    const int lz = __clzll((i64)m);
+    const u64 n = m << (lz & 63);
+    // 53 bits and the next as rounding, added onto the exponent: a carry bumps it
+    const u64 bits = (n >> 11) + ((n >> 10) & 1ull) + ((u64)(unsigned)(e_out - lz - 1) << 52);
+    const double r = __longlong_as_double((i64)(bits | ((u64)s & 0x8000000000000000ull)));
+    return m ? r : 0.0;
+}
+
+// A of one site: c its value, s2 the sum of its neighbours.
+// k2, e_out: f's for the warp's scale.
+__device__ __forceinline__ double force(i64 c, i64 s2, const Fix64& f, u64 k2, int e_out)
+{
+    const i64 sc = c >> 63, ss = s2 >> 63;
+    const u64 b = (u64)with_sign((u64)c, sc) << 3;              // |x| 2^62
+    const u64 t = __umul64hi(b, b);                             // x^2 2^60
+    const i64 k = f.k1 - (i64)__umul64hi(t, k2);                // (k1 - k2 phi^2) 2^(62-ek)
+    const i64 u = with_sign((u64)__mul64hi((i64)b, k), sc);     // x (k1 - k2 phi^2) 2^(60-ek)
+    const i64 l = with_sign(__umul64hi((u64)with_sign((u64)s2, ss), f.g), ss);
+    return from_fixed(u + l, e_out);
+}
+
+template <int D>
+__global__ void __launch_bounds__(kFxThreads, fx_blocks(D)) k_step_fix64(const __grid_constant__ FixArgs a)
+{
+    constexpr int R = D == 3 ? 4 : 1, N = D == 3 ? R + 2 : 1, H = D == 3 ? 1 : 0;  // output and stored rows; halo
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int nx = a.g.nx, ny = D == 3 ? a.g.ny : 1, nz = D == 3 ? a.g.nz : a.g.ny;
+    int x0, y0, z0;
+    if (D == 3) {
+        int b = blockIdx.x;
+        x0 = b % a.nstrips * kFxU;
+        b /= a.nstrips;
+        y0 = (b % a.ygroups * kFxWarps + wid) * R;
+        z0 = b / a.ygroups * a.cz;
+        if (y0 >= ny) return;
+    } else {
+        const int w = blockIdx.x * kFxWarps + wid;
+        x0 = w % a.nstrips * kFxU;
+        y0 = 0;
+        z0 = w / a.nstrips * a.cz;
+        if (z0 >= nz) return;
+    }
+    const int planes = min(a.cz, nz - z0), rows = min(R, ny - y0);
+    int x = (x0 - 1 + lane) % nx;
+    if (x < 0) x += nx;
+    const bool out = lane >= 1 && lane <= min(kFxU, nx - x0);
+    unsigned row[N];  // element offsets of the stored rows in a plane, periodic
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+        int y = (y0 - H + r) % ny;
+        if (y < 0) y += ny;
+        row[r] = (unsigned)y * (unsigned)nx + (unsigned)x;
+    }
+    const int64_t plane = (int64_t)nx * ny;
+    int z = z0 == 0 ? nz - 1 : z0 - 1;
+    const double* pin = a.phi_in + (int64_t)z * plane;
+    const double* vin = a.v_in + (int64_t)z0 * plane;
+    double* pout = a.phi_out + (int64_t)z0 * plane;
+    double* vout = a.v_out + (int64_t)z0 * plane;
+    double next[N], vnext[R];  // the plane on its way
+    auto fetch = [&] {
+#pragma unroll
+        for (int r = 0; r < N; ++r) next[r] = pin[row[r]];
+        ++z;
+        pin += z == nz ? plane * (1 - (int64_t)nz) : plane;
+        if (z == nz) z = 0;
+    };
+    // planes z-1 (output rows), z, z+1 as integers, plane z's values, the planes' smallest shifts
+    i64 m[R], c[N], p[N];
+    double d[R], v[R];
+    int sm = 4096, sc = 4096, sp, down = 0;
+    const int most = a.f.e_out - 192;  // exponents of A stay in range
+    u64 k2 = a.f.k2;
+    fetch();
+#pragma unroll
+    for (int r = 0; r < R; ++r) m[r] = 0, vnext[r] = 0.0, d[r] = 0.0;
+#pragma unroll
+    for (int r = 0; r < N; ++r) c[r] = 0;
+    for (int i = -1; i <= planes; ++i) {  // plane z0 + i arrives, plane z0 + i - 1 is updated
+        sp = 4096;
+        double dn[R];
+#pragma unroll
+        for (int r = 0; r < N; ++r) {
+            int s;
+            p[r] = to_fixed(next[r], a.f.e_base - down, s);
+            sp = min(sp, s);
+            if (r >= H && r < R + H) dn[r - H] = next[r];
+        }
+        sp = __reduce_min_sync(0xffffffffu, sp);
+        const int least = min(min(sm, sc), sp);  // the shift of the largest value
+        if ((least < 3 || least > 7) && least < 1100) {  // (planes of zeros keep the scale)
+            const int by = max(min(least - 3, most - down), -down);
+            if (by != 0) {
+                down += by;
+                k2 = down > 31 ? 0ull : a.f.k2 >> 2 * down;
+                sm -= by, sc -= by, sp -= by;
+#pragma unroll
+                for (int r = 0; r < R; ++r) m[r] = rescaled(m[r], by);
+#pragma unroll
+                for (int r = 0; r < N; ++r) {
+                    int s;
+                    c[r] = rescaled(c[r], by);
+                    p[r] = to_fixed(next[r], a.f.e_base - down, s);
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = vnext[r];
+        if (i < planes) fetch();
+        if (i >= 0 && i < planes) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) vnext[r] = r < rows ? vin[row[r + H]] : 0.0;
+            vin += plane;
+        }
+        if (i >= 1) {
+            const bool fixed = min(min(sm, sc), sp) >= 3;
+            double pn[R];
+            if (fixed) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const i64 cc = c[r + H];
+                    i64 s2 = (__shfl_up_sync(0xffffffffu, cc, 1) + __shfl_down_sync(0xffffffffu, cc, 1)) +
+                             (m[r] + p[r + H]);
+                    if (D == 3) s2 += c[r] + c[r + 2 * H];
+                    v[r] = fma(a.k.c1, v[r], force(cc, s2, a.f, k2, a.f.e_out - down));
+                    pn[r] = fma(a.deta, v[r], d[r]);
+                }
+            } else {
+                const int zc = z0 + i - 1, zm = zc == 0 ? nz - 1 : zc - 1, zp = zc + 1 == nz ? 0 : zc + 1;
+                const double* q = a.phi_in + (int64_t)zc * plane;
+                const double* qp = a.phi_in + (int64_t)zp * plane;
+                const double* qm = a.phi_in + (int64_t)zm * plane;
+#pragma unroll 1
+                for (int r = 0; r < rows; ++r) {
+                    const int y = y0 + r;
+                    const int64_t o = (int64_t)y * nx, up = (int64_t)(y + 1 == ny ? 0 : y + 1) * nx + x;
+                    const int64_t dn2 = (int64_t)(y == 0 ? ny - 1 : y - 1) * nx + x;
+                    const double xp = q[o + (x + 1 == nx ? 0 : x + 1)], xm = q[o + (x == 0 ? nx - 1 : x - 1)];
+                    const double cc = q[o + x], yp = D == 3 ? q[up] : qp[o + x], ym = D == 3 ? q[dn2] : qm[o + x];
+                    const double zpv = D == 3 ? qp[o + x] : 0.0, zmv = D == 3 ? qm[o + x] : 0.0;
+                    double vv, pp;
+#pragma unroll
+                    for (int u = 0; u < R; ++u) vv = u == r ? v[u] : vv;
+                    site_update_folded<D>(cc, xp, xm, yp, ym, zpv, zmv, vv, pp, a.k, a.deta);
+#pragma unroll
+                    for (int u = 0; u < R; ++u)
+                        if (u == r) v[u] = vv, pn[u] = pp;
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (out && r < rows) {
+                    pout[row[r + H]] = pn[r];
+                    vout[row[r + H]] = v[r];
+                }
+            pout += plane;
+            vout += plane;
+        }
+        sm = sc;
+        sc = sp;
+#pragma unroll
+        for (int r = 0; r < R; ++r) m[r] = c[r + H], d[r] = dn[r];
+#pragma unroll
+        for (int r = 0; r < N; ++r) c[r] = p[r];
+    }
+}
+
+}  // namespace
+
+// The constants of a step, or false where they do not fit (the double form everywhere then).
+static bool make_fix64(const KickD& k, double phi0, Fix64* f)
+{
+    int es;  // S = 2^es >= phi0
+    const double fr = frexp(phi0, &es);
+    if (fr == 0.5) --es;
+    const double k2s = ldexp(k.k2, 2 * es);
+    const double bound = fabs(k.k1) + 8.0 * fabs(k2s) + 4.0 * fabs(k.g);
+    if (!(bound > 0) || !isfinite(bound) || k2s < 0 || !(k.g > 0)) return false;
+    int ek;
+    frexp(bound, &ek);  // bound < 2^ek
+    if (ek < -400 || ek > 400 || es < -400 || es > 400) return false;
+    f->k1 = (i64)llrint(ldexp(k.k1, 62 - ek));
+    f->k2 = (u64)llrint(ldexp(k2s, 65 - ek)) << 1;
+    f->g = (u64)llrint(ldexp(k.g, 65 - ek));
+    f->e_base = 1026 + es;
+    f->e_out = 1023 + 63 + ek - 60 + es;
+    return true;
+}
+
+cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const double* v, double* v_out,
+                              const KickD& k, double deta, double phi0, cudaStream_t st)
+{
+    FixArgs a;
+    if (!make_fix64(k, phi0, &a.f)) return cudaErrorNotSupported;
+    if (g.dims == 3 && (int64_t)g.nx * g.ny >= ((int64_t)1 << 32)) return cudaErrorNotSupported;
+    a.phi_in = in;
+    a.phi_out = out;
+    a.v_in = v;
+    a.v_out = v_out;
+    a.k = k;
+    a.deta = deta;
+    a.g = g;
+    a.nstrips = (g.nx + kFxU - 1) / kFxU;
+    const int len = g.dims == 3 ? g.nz : g.ny;
+    a.ygroups = g.dims == 3 ? (g.ny + 4 * kFxWarps - 1) / (4 * kFxWarps) : 1;
+    // warps (2D) or blocks of them (3D) against the two planes a chunk re-reads and the iteration
+    // that fills it
+    const double tiles = (double)a.nstrips * a.ygroups / (g.dims == 3 ? 1 : kFxWarps);
+    const double slots = (double)fx_blocks(g.dims) * sm_count_current();
+    double least = 1e300;
+    a.cz = len;
+    for (int nc = 1; nc <= len && nc <= 4096; ++nc) {
+        const int c = (len + nc - 1) / nc, n = (len + c - 1) / c;
+        const double w = tiles * n / slots;
+        const double cost = (w <= 1.0 ? 0.7 + 0.3 * w : 0.5 * (ceil(w) + w + 0.35)) * (c + 2.0);
+        if (cost < least * 0.999) least = cost, a.cz = c;
+    }
+    const int64_t n = (len + a.cz - 1) / a.cz;
+    const int64_t blocks = g.dims == 3 ? (int64_t)a.nstrips * a.ygroups * n
+                                       : ((int64_t)a.nstrips * n + kFxWarps - 1) / kFxWarps;
+    if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
+    if (g.dims == 3) k_step_fix64<3><<<(unsigned)blocks, kFxThreads, 0, st>>>(a);
+    else k_step_fix64<2><<<(unsigned)blocks, kFxThreads, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace prs

@@ -138,6 +138,10 @@ cudaError_t launch_step_generic(const Geo& g, int precision, bool repro, const v
 {
     if (precision == PRS_FP32) return step_generic_t<float, false>(g, in, out, dphi, dphi_out, c1, c2, cV, rcd, st);
     if (repro) return step_generic_t<double, true>(g, in, out, dphi, dphi_out, c1, c2, cV, rcd, st);
+    const double coef[3] = {c1, c2, cV};
+    const cudaError_t e = launch_step_fix64(g, (const double*)in, (double*)out, (const double*)dphi, (double*)dphi_out,
+                                            kick_f64(coef, rcd), rcd[0], rcd[5], st);
+    if (e != cudaErrorNotSupported) return e;
     return step_generic_t<double, false>(g, in, out, dphi, dphi_out, c1, c2, cV, rcd, st);
 }
 

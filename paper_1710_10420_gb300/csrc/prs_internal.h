@@ -128,6 +128,11 @@ cudaError_t launch_step_io(const Geo& g, int precision, bool repro, const void* 
                            const void* dphi_in, void* dphi_out, const double* c1, const double* c2, const double* cV,
                            int nsteps_in_pass, const double run_const[6], unsigned int* err, cudaStream_t st);
 
+// The FP64 step (folded kick) with its force in 64-bit fixed point (prs_fix64.cu);
+// cudaErrorNotSupported where its constants or the box do not fit.
+cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const double* v, double* v_out,
+                              const KickD& k, double deta, double phi0, cudaStream_t st);
+
 // Copy a state's fields (device to device, `bytes` each; a field that is its own source stays).
 cudaError_t launch_copy_state(const void* phi, void* phi_out, const void* dphi, void* dphi_out, size_t bytes,
                               cudaStream_t st);
