@@ -196,7 +196,7 @@ extern "C" int prs_create(const prs_params* params, void* stream, prs_sim** out)
     s->d_status = (DevStatus*)(s->scr.partials + kMeasureBlocks);
     s->scr.result = &s->d_status->result;
     s->scr.counter = &s->d_status->counter;
-    if (cudaMemset(blob, 0, bytes) != cudaSuccess ||
+    if (cudaMemsetAsync(blob, 0, bytes, s->stream) != cudaSuccess ||
         cudaMallocHost((void**)&s->h_status, sizeof(DevStatus)) != cudaSuccess ||
         ((params->flags & PRS_DEBUG) && cudaMalloc((void**)&s->d_dbg, sizeof(DebugCheck)) != cudaSuccess)) {
         int r = cuda_fail(cudaGetLastError(), "prs_create");
@@ -580,7 +580,7 @@ static bool fast_diag_ok(const prs_sim* s)
 // Queue the diagnostics of the current state.
 static cudaError_t queue_measure(prs_sim* s, const DiagScratch& scr)
 {
-    return launch_measure(s->g, s->p.precision, fast_diag_ok(s), s->phi[s->cur], s->dphi, s->rc, scr,
+    return launch_measure(s->g, s->p.precision, fast_diag_ok(s), MeasureRun{s->phi[s->cur], s->dphi, s->rc, scr},
                           &s->d_status->error, s->stream);
 }
 
@@ -692,14 +692,28 @@ int prs::step_runs(prs_sim* const* runs, int nruns, int64_t nsteps)
     return PRS_OK;
 }
 
-int prs::queue_diagnostics(prs_sim* s, DiagAcc* result)
+int prs::queue_diagnostics(prs_sim* const* runs, int nruns, DiagAcc* const* results)
 {
-    if (!s || !result) return PRS_EINVAL;
-    if (!s->initialised) return PRS_ESTATE;
-    DiagScratch scr = s->scr;
-    scr.result = result;
-    const cudaError_t e = queue_measure(s, scr);
-    return e == cudaSuccess ? PRS_OK : cuda_fail(e, "measure launch");
+    for (int r0 = 0; r0 < nruns; r0 += kMeasureMaxRuns) {
+        const int n = nruns - r0 < kMeasureMaxRuns ? nruns - r0 : kMeasureMaxRuns;
+        MeasureRun q[kMeasureMaxRuns];
+        bool together = n > 1;
+        for (int r = 0; r < n; ++r) {
+            prs_sim* s = runs[r0 + r];
+            if (!s || !results[r0 + r]) return PRS_EINVAL;
+            if (!s->initialised) return PRS_ESTATE;
+            const Geo &g = s->g, &g0 = runs[r0]->g;
+            together = together && fast_diag_ok(s) && g.dims == g0.dims && g.nx == g0.nx && g.ny == g0.ny &&
+                       g.nz == g0.nz && s->stream == runs[r0]->stream;
+            q[r] = MeasureRun{s->phi[s->cur], s->dphi, s->rc, s->scr};
+            q[r].scr.result = results[r0 + r];
+        }
+        cudaError_t e = cudaSuccess;
+        if (together) e = launch_measure_runs(runs[r0]->g, n, q, runs[r0]->stream);
+        for (int r = 0; r < n && !together && e == cudaSuccess; ++r) e = queue_measure(runs[r0 + r], q[r].scr);
+        if (e != cudaSuccess) return cuda_fail(e, "measure launch");
+    }
+    return PRS_OK;
 }
 
 static int prs_measure_ex_impl(prs_sim* s, prs_diag* out)

@@ -23,8 +23,7 @@ __global__ void __launch_bounds__(kFastThreads, 2)
     Tile3D T{phi_in, phi_out, v, v_out, nx, ny, nz, ty, (int)(blockIdx.x % ytiles) * ty,
              (int)(blockIdx.x / ytiles) * cz, 0};
     T.zn = min(cz, nz - T.z0);
-    SiteAcc a{};
-    tile3d<ITEMS, true, false>(T, k, rc, smem_raw, nullptr, a, err);
+    tile3d<ITEMS>(T, k, rc, smem_raw, err);
 }
 
 // ------------------------------------------------------------------ dispatch

@@ -142,10 +142,21 @@ cudaError_t launch_copy_state(const void* phi, void* phi_out, const void* dphi, 
 int max_fused_steps(const Geo& g, int precision, bool repro);
 int default_fused_steps(const Geo& g, int precision, bool repro);
 
-// The wall diagnostics of (phi, dphi) (prs_measure.cu), any box.  fast (FP32): hardware
-// reciprocal square root and division, else IEEE operations.  err: the run's error word.
-cudaError_t launch_measure(const Geo& g, int precision, bool fast, const void* phi, const void* dphi,
-                           const double run_const[6], const DiagScratch& scr, unsigned int* err, cudaStream_t st);
+// The wall diagnostics (prs_measure.cu), any box: a state, the run's constants (the layout of
+// RunConst) and where the sums go.
+struct MeasureRun {
+    const void* phi;
+    const void* dphi;
+    const double* run_const;
+    DiagScratch scr;
+};
+// fast (FP32): hardware reciprocal square root and division, else IEEE operations.  err: the run's
+// error word.
+cudaError_t launch_measure(const Geo& g, int precision, bool fast, const MeasureRun& run, unsigned int* err,
+                           cudaStream_t st);
+// Up to kMeasureMaxRuns FP32 runs of one box in one launch, as launch_measure with fast.
+constexpr int kMeasureMaxRuns = 16;
+cudaError_t launch_measure_runs(const Geo& g, int nruns, const MeasureRun* runs, cudaStream_t st);
 
 // Fast FP32 kernels (prs_fast.cu) for x sides that are multiples of 128.
 bool fast_step_ok(const Geo& g, int precision);
@@ -170,8 +181,7 @@ cudaError_t launch_step_t2_tma(const Geo& g, const float* phi_in, float* phi_out
 void record_error(const char* msg);
 
 // The diagnostic kernel (IEEE operations) on at most `grid` blocks (1 <= grid <= scr.max_blocks).
-cudaError_t launch_measure_on_grid(const Geo& g, int precision, const void* phi, const void* dphi,
-                                   const double run_const[6], const DiagScratch& scr, int grid, cudaStream_t st);
+cudaError_t launch_measure_on_grid(const Geo& g, int precision, const MeasureRun& run, int grid, cudaStream_t st);
 
 // Host-side setup shared by the launchers.  Calls on different prs_sim handles may
 // run concurrently from several host threads, so neither keeps unsynchronised state.

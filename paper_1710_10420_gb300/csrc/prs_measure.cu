@@ -194,15 +194,28 @@ __device__ __forceinline__ int warp_prefix(int cnt, int lane, int& total)
     return incl - cnt;
 }
 
+// The runs of one launch: blocks (., r) take run r.
+template <typename R, int NR>
+struct MRuns {
+    const R* phi[NR];
+    const R* dphi[NR];
+    RunConst<R> rc[NR];
+    DiagScratch scr[NR];
+};
+
 // FAST: FP32 with the hardware reciprocal square root and division; else IEEE operations.
 // vec: rows may be staged 16 bytes at a time (row length and base address multiples of 16 bytes).
 // err: the run's error word when map describes phi in boxes of a tile with its halo (then one
 // tensor copy stages each tile whose rows do not wrap, the wrapped columns patched in), or null.
-template <typename R, int D, bool FAST>
+template <typename R, int D, bool FAST, int NR>
 __global__ void __launch_bounds__(kMThreads, D == 2 ? 4 : 3)
-    k_measure(const __grid_constant__ CUtensorMap map, const R* __restrict__ phi, const R* __restrict__ dphi, Geo g,
-              RunConst<R> rc, MTiling T, bool vec, unsigned int* err, DiagScratch scr)
+    k_measure(const __grid_constant__ CUtensorMap map, const __grid_constant__ MRuns<R, NR> runs, Geo g, MTiling T,
+              bool vec, unsigned int* err)
 {
+    const int run = NR > 1 ? blockIdx.y : 0;
+    const R* __restrict__ phi = runs.phi[run];
+    const R* __restrict__ dphi = runs.dphi[run];
+    const RunConst<R>& rc = runs.rc[run];
     using A = Arith<R, true>;
     constexpr int kOff = MRow<R>::kOff, kLd = MRow<R>::kLd;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -463,7 +476,8 @@ __global__ void __launch_bounds__(kMThreads, D == 2 ? 4 : 3)
         }
     }
     __syncthreads();  // the tile's memory is free
-    block_reduce_and_finish(DiagAcc{a.sw, a.sr, a.nl, a.nw, a.nv0, a.nnf}, scr, reinterpret_cast<double2*>(tile));
+    block_reduce_and_finish_at(DiagAcc{a.sw, a.sr, a.nl, a.nw, a.nv0, a.nnf}, runs.scr[run], blockIdx.x, gridDim.x,
+                               reinterpret_cast<double2*>(tile));
 }
 
 // Resident CTAs: four by registers (three in 3D), fewer where shared memory holds fewer.
@@ -491,8 +505,9 @@ MTiling tiling(const Geo& g, size_t elem, int sms)
             T.ntx = ((unsigned)g.nx + kMCols - 1) / kMCols;
             T.nty = ((unsigned)g.ny + (1u << ly) - 1) >> ly;
             T.ntiles = T.ntx * T.nty * (((unsigned)g.nz + (1u << lz) - 1) >> lz);
-            const double slots = (double)ctas_per_sm(g.dims, elem, T) * sms, waves = ceil(T.ntiles / slots);
-            const double fill = waves > 1 ? 1.0 : (T.ntiles > sms ? T.ntiles / slots : 1.0 / 3.0);
+            const double tiles = (double)T.ntiles, slots = (double)ctas_per_sm(g.dims, elem, T) * sms;
+            const double waves = ceil(tiles / slots);
+            const double fill = waves > 1 ? 1.0 : (tiles > sms ? tiles / slots : 1.0 / 3.0);
             const double cost = waves * (3.0 + fill * (0.03 * halo_rows(g.dims, T) + 0.11 * (1 << (ly + lz))));
             if (cost < best_cost) best_cost = cost, best = T;
         }
@@ -515,57 +530,70 @@ bool phi_map(CUtensorMap* m, const R* phi, const Geo& g, const MTiling& T)
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <typename R, int D, bool FAST>
-cudaError_t measure_t(const Geo& g, const void* phi, const void* dphi, const double rcd[6], const DiagScratch& scr,
-                      unsigned int* err, int grid, cudaStream_t st)
+template <typename R, int D, bool FAST, int NR>
+cudaError_t measure_t(const Geo& g, int nruns, const MeasureRun* q, unsigned int* err, int grid, cudaStream_t st)
 {
     static std::atomic<unsigned long long> attr{0};
     const int sms = sm_count_current();
+    // the tiling of a run alone: a tile's partial sums are FP32 (FAST), so the same tiles give the same
+    // sums to FP64 rounding
     const MTiling T = tiling(g, sizeof(R), sms);
     const MTiling most{D == 3 ? 3 : 6, D == 3 ? 3 : 0, 0, 0, 0};
-    cudaError_t e = smem_limit_once(attr, (const void*)k_measure<R, D, FAST>,
+    cudaError_t e = smem_limit_once(attr, (const void*)k_measure<R, D, FAST, NR>,
                                     (int)(sizeof(R) == 4 ? measure_smem(D, 4, most) : 100 * 1024));
     if (e != cudaSuccess) return e;
-    if (grid <= 0) {  // the resident CTAs, one partial slot each
-        const int most = ctas_per_sm(D, sizeof(R), T) * sms;
-        grid = T.ntiles < (unsigned)most ? (int)T.ntiles : most;
-        if (grid > scr.max_blocks) grid = scr.max_blocks;
+    if (grid <= 0) {  // the resident CTAs, shared by the runs; one partial slot each
+        const int all = ctas_per_sm(D, sizeof(R), T) * sms / nruns;
+        grid = T.ntiles < (unsigned)all ? (int)T.ntiles : (all > 0 ? all : 1);
+        if (grid > q[0].scr.max_blocks) grid = q[0].scr.max_blocks;
     }
-    const bool vec = g.nx % MRow<R>::kOff == 0 && (((uintptr_t)phi | (uintptr_t)dphi) & 15u) == 0;
-    const RunConst<R> rc{(R)rcd[0], (R)rcd[1], (R)rcd[2], (R)rcd[3], (R)rcd[4], (R)rcd[5]};
-    CUtensorMap map;
-    if (!vec || !phi_map(&map, (const R*)phi, g, T)) err = nullptr;
-    k_measure<R, D, FAST><<<grid, kMThreads, measure_smem(D, sizeof(R), T), st>>>(map, (const R*)phi, (const R*)dphi,
-                                                                                 g, rc, T, vec, err, scr);
+    MRuns<R, NR> runs;
+    uintptr_t bits = 0;
+    for (int r = 0; r < nruns; ++r) {
+        const double* c = q[r].run_const;
+        runs.phi[r] = (const R*)q[r].phi;
+        runs.dphi[r] = (const R*)q[r].dphi;
+        runs.rc[r] = RunConst<R>{(R)c[0], (R)c[1], (R)c[2], (R)c[3], (R)c[4], (R)c[5]};
+        runs.scr[r] = q[r].scr;
+        bits |= (uintptr_t)q[r].phi | (uintptr_t)q[r].dphi;
+    }
+    const bool vec = g.nx % MRow<R>::kOff == 0 && (bits & 15u) == 0;
+    CUtensorMap map{};
+    if (NR > 1 || !vec || !phi_map(&map, (const R*)q[0].phi, g, T)) err = nullptr;
+    k_measure<R, D, FAST, NR><<<dim3((unsigned)grid, (unsigned)nruns), kMThreads, measure_smem(D, sizeof(R), T), st>>>(
+        map, runs, g, T, vec, err);
     return cudaGetLastError();
 }
 
-template <typename R, bool FAST>
-cudaError_t measure_d(const Geo& g, const void* phi, const void* dphi, const double rcd[6], const DiagScratch& scr,
-                      unsigned int* err, int grid, cudaStream_t st)
+template <typename R, bool FAST, int NR>
+cudaError_t measure_d(const Geo& g, int nruns, const MeasureRun* q, unsigned int* err, int grid, cudaStream_t st)
 {
-    return g.dims == 3 ? measure_t<R, 3, FAST>(g, phi, dphi, rcd, scr, err, grid, st)
-                       : measure_t<R, 2, FAST>(g, phi, dphi, rcd, scr, err, grid, st);
+    return g.dims == 3 ? measure_t<R, 3, FAST, NR>(g, nruns, q, err, grid, st)
+                       : measure_t<R, 2, FAST, NR>(g, nruns, q, err, grid, st);
 }
 
 }  // namespace
 
-cudaError_t launch_measure(const Geo& g, int precision, bool fast, const void* phi, const void* dphi,
-                           const double rcd[6], const DiagScratch& scr, unsigned int* err, cudaStream_t st)
+cudaError_t launch_measure(const Geo& g, int precision, bool fast, const MeasureRun& run, unsigned int* err,
+                           cudaStream_t st)
 {
-    if (precision != PRS_FP32) return measure_d<double, false>(g, phi, dphi, rcd, scr, err, 0, st);
-    return fast ? measure_d<float, true>(g, phi, dphi, rcd, scr, err, 0, st)
-                : measure_d<float, false>(g, phi, dphi, rcd, scr, err, 0, st);
+    if (precision != PRS_FP32) return measure_d<double, false, 1>(g, 1, &run, err, 0, st);
+    return fast ? measure_d<float, true, 1>(g, 1, &run, err, 0, st) : measure_d<float, false, 1>(g, 1, &run, err, 0, st);
 }
 
-cudaError_t launch_measure_on_grid(const Geo& g, int precision, const void* phi, const void* dphi,
-                                   const double rcd[6], const DiagScratch& scr, int grid, cudaStream_t st)
+cudaError_t launch_measure_runs(const Geo& g, int nruns, const MeasureRun* runs, cudaStream_t st)
 {
-    if (grid < 1 || grid > scr.max_blocks) return cudaErrorInvalidValue;
+    if (nruns < 1 || nruns > kMeasureMaxRuns) return cudaErrorInvalidValue;
+    return measure_d<float, true, kMeasureMaxRuns>(g, nruns, runs, nullptr, 0, st);
+}
+
+cudaError_t launch_measure_on_grid(const Geo& g, int precision, const MeasureRun& run, int grid, cudaStream_t st)
+{
+    if (grid < 1 || grid > run.scr.max_blocks) return cudaErrorInvalidValue;
     const int most = 3 * sm_count_current();  // resident CTAs: more only add partials
     if (grid > most) grid = most;
-    if (precision == PRS_FP32) return measure_d<float, false>(g, phi, dphi, rcd, scr, nullptr, grid, st);
-    return measure_d<double, false>(g, phi, dphi, rcd, scr, nullptr, grid, st);
+    if (precision == PRS_FP32) return measure_d<float, false, 1>(g, 1, &run, nullptr, grid, st);
+    return measure_d<double, false, 1>(g, 1, &run, nullptr, grid, st);
 }
 
 }  // namespace prs

@@ -123,7 +123,7 @@ extern "C" int prs_measure_noalloc(const prs_params* p, const void* d_phi, const
     // the completion counter must start at zero; a previous call normally leaves it
     // there, but an interrupted one might not
     cudaError_t e = cudaMemsetAsync(scr.counter, 0, sizeof(unsigned int), st);
-    if (e == cudaSuccess) e = launch_measure_on_grid(g, p->precision, d_phi, d_dphi, rcd, scr, grid, st);
+    if (e == cudaSuccess) e = launch_measure_on_grid(g, p->precision, MeasureRun{d_phi, d_dphi, rcd, scr}, grid, st);
     DiagAcc a;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&a, scr.result, sizeof(DiagAcc), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -53,9 +53,9 @@ int cuda_fail(cudaError_t e, const char* what);
 int ensure_buffers(prs_sim* s);
 // After a synchronised read of s->h_status: PRS_ETIMEOUT (once) if a device wait gave up.
 int check_device_error(prs_sim* s);
-// Queue the Eq. 7/8 sums of the run's current state into *result (device memory), without
-// waiting for them.
-int queue_diagnostics(prs_sim* s, DiagAcc* result);
+// Queue the Eq. 7/8 sums of each run's current state into *results[r] (device memory), without waiting
+// for them: runs of one box and stream share launches.
+int queue_diagnostics(prs_sim* const* runs, int nruns, DiagAcc* const* results);
 // Step each of several runs by nsteps: FP32 runs that share a box and stream (x sides that are
 // multiples of 128, at most kMarchMaxRuns) pass by pass in one launch over all the runs, else one run
 // after another.  The fields do not depend on how steps group into passes.
