@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "prs_arith.cuh"
+#include "prs_chain.h"
 #include "prs_internal.h"
 #include "prs_ptx.cuh"
 #include "prs_tile.cuh"
@@ -19,6 +20,7 @@ __global__ void __launch_bounds__(kFastThreads, 2)
                  int ny, int nz, int ty, int cz, KickF k, RunConst<float> rc, unsigned int* err)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    chain_enter();
     const int ytiles = ny / ty;
     Tile3D T{phi_in, phi_out, v, v_out, nx, ny, nz, ty, (int)(blockIdx.x % ytiles) * ty,
              (int)(blockIdx.x / ytiles) * cz, 0};
@@ -90,9 +92,8 @@ cudaError_t launch_step_fast(const Geo& g, const float* in, float* out, const fl
         int nchunks = pick_chunks(ytiles, g.nz, kMinPlanes, slots);
         const int cz = (g.nz + nchunks - 1) / nchunks;
         nchunks = (g.nz + cz - 1) / cz;
-        k_step3d_f32<kItems><<<ytiles * nchunks, kFastThreads, sm, st>>>(in, out, v, v_out, g.nx, g.ny, g.nz, t, cz,
-                                                                         k, rc, err);
-        return cudaGetLastError();
+        return launch_chained(k_step3d_f32<kItems>, dim3((unsigned)(ytiles * nchunks)), kFastThreads, sm, st, in, out, v,
+                              v_out, g.nx, g.ny, g.nz, t, cz, k, rc, err);
     }
     return cudaErrorNotSupported;
 }

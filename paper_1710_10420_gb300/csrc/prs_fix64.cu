@@ -31,7 +31,9 @@
 
 #include <algorithm>
 
+#include "prs_chain.h"
 #include "prs_internal.h"
+#include "prs_ptx.cuh"
 #include "prs_site.cuh"
 
 namespace prs {
@@ -117,6 +119,7 @@ template <int D>
 __global__ void __launch_bounds__(kFxThreads, fx_blocks(D)) k_step_fix64(const __grid_constant__ FixArgs a)
 {
     constexpr int R = D == 3 ? 4 : 1, N = D == 3 ? R + 2 : 1, H = D == 3 ? 1 : 0;  // output and stored rows; halo
+    chain_enter();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nx = a.g.nx, ny = D == 3 ? a.g.ny : 1, nz = D == 3 ? a.g.nz : a.g.ny;
     int x0, y0, z0;
@@ -303,7 +306,7 @@ cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const
     const double slots = (double)fx_blocks(g.dims) * sm_count_current();
     double least = 1e300;
     a.cz = len;
-    for (int nc = 1; nc <= len && nc <= 4096; ++nc) {
+    for (int nc = 1; nc <= len && nc <= 4096; nc += nc < 32 ? 1 : nc / 16) {
         const int c = (len + nc - 1) / nc, n = (len + c - 1) / c;
         const double w = tiles * n / slots;
         const double cost = (w <= 1.0 ? 0.7 + 0.3 * w : 0.5 * (ceil(w) + w + 0.35)) * (c + 2.0);
@@ -313,9 +316,7 @@ cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const
     const int64_t blocks = g.dims == 3 ? (int64_t)a.nstrips * a.ygroups * n
                                        : ((int64_t)a.nstrips * n + kFxWarps - 1) / kFxWarps;
     if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
-    if (g.dims == 3) k_step_fix64<3><<<(unsigned)blocks, kFxThreads, 0, st>>>(a);
-    else k_step_fix64<2><<<(unsigned)blocks, kFxThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(g.dims == 3 ? k_step_fix64<3> : k_step_fix64<2>, dim3((unsigned)blocks), kFxThreads, 0, st, a);
 }
 
 }  // namespace prs

@@ -7,7 +7,9 @@
 #include <cuda_runtime.h>
 
 #include "prs_arith.cuh"
+#include "prs_chain.h"
 #include "prs_internal.h"
+#include "prs_ptx.cuh"
 #include "prs_site.cuh"
 
 namespace prs {
@@ -69,9 +71,10 @@ static dim3 rows_grid(const Geo& g, int cap)
 // --------------------------------------------------------- generic step
 
 template <typename R, bool REPRO, int D>
-__global__ void k_step_generic(const R* __restrict__ phi, R* __restrict__ phi_out, const R* dphi, R* dphi_out,
-                               Geo g, StepCoef<R> k, RunConst<R> rc, KickD kd)
+__global__ void k_step_generic(const R* phi, R* phi_out, const R* dphi, R* dphi_out, Geo g, StepCoef<R> k,
+                               RunConst<R> rc, KickD kd)
 {
+    chain_enter();
     const int64_t nx = g.nx, ny = g.ny, nz = g.nz;
     const int64_t plane = nx * ny;
     // rows of x: y blocks stride over the rows (y, z decoded once per row), x threads over a row
@@ -120,17 +123,12 @@ static cudaError_t step_generic_t(const Geo& g, const void* in, void* out, const
     RunConst<R> rc = make_rc<R>(rcd);
     const double coef[3] = {c1, c2, cV};
     const KickD kd = kick_f64(coef, rcd);
-    if constexpr (sizeof(R) == 4) {  // FP32 2D boxes take the register march
-        if (g.dims != 3) return cudaErrorNotSupported;
-        k_step_generic<R, REPRO, 3><<<grid, block, 0, st>>>((const R*)in, (R*)out, (const R*)dphi, (R*)dphi_out, g, k,
-                                                             rc, kd);
-    } else if (g.dims == 3)
-        k_step_generic<R, REPRO, 3><<<grid, block, 0, st>>>((const R*)in, (R*)out, (const R*)dphi, (R*)dphi_out, g, k,
-                                                             rc, kd);
-    else
-        k_step_generic<R, REPRO, 2><<<grid, block, 0, st>>>((const R*)in, (R*)out, (const R*)dphi, (R*)dphi_out, g, k,
-                                                             rc, kd);
-    return cudaGetLastError();
+    void (*kernel)(const R*, R*, const R*, R*, Geo, StepCoef<R>, RunConst<R>, KickD) = k_step_generic<R, REPRO, 3>;
+    if (g.dims == 2) {
+        if constexpr (sizeof(R) == 4) return cudaErrorNotSupported;  // FP32 2D boxes take the register march
+        else kernel = k_step_generic<R, REPRO, 2>;
+    }
+    return launch_chained(kernel, grid, block, 0, st, (const R*)in, (R*)out, (const R*)dphi, (R*)dphi_out, g, k, rc, kd);
 }
 
 cudaError_t launch_step_generic(const Geo& g, int precision, bool repro, const void* in, void* out, const void* dphi,
@@ -150,9 +148,9 @@ cudaError_t launch_step_generic(const Geo& g, int precision, bool repro, const v
 // phi and dphi of a state in one launch, 64 bytes a thread and turn.  Bound by HBM for large boxes
 // (1024^3: what two device-to-device copies take); for small ones by the launch, of which this
 // saves one (256^2: 4 us of 81).
-__global__ void __launch_bounds__(256) k_copy_state(const float4* __restrict__ p, float4* __restrict__ po,
-                                                    const float4* __restrict__ v, float4* __restrict__ vo, int64_t n)
+__global__ void __launch_bounds__(256) k_copy_state(const float4* p, float4* po, const float4* v, float4* vo, int64_t n)
 {
+    chain_enter();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x * 4 + threadIdx.x; i < 2 * n; i += stride) {
         float4 a[4];
@@ -183,9 +181,8 @@ cudaError_t launch_copy_state(const void* phi, void* phi_out, const void* dphi, 
         return e;
     }
     const int64_t n = (int64_t)(bytes / 16);
-    k_copy_state<<<grid_for(2 * n, 1024), 256, 0, st>>>((const float4*)phi, (float4*)phi_out, (const float4*)dphi,
-                                                        (float4*)dphi_out, n);
-    return cudaGetLastError();
+    return launch_chained(k_copy_state, dim3((unsigned)grid_for(2 * n, 1024)), 256, 0, st, (const float4*)phi,
+                          (float4*)phi_out, (const float4*)dphi, (float4*)dphi_out, n);
 }
 
 }  // namespace prs

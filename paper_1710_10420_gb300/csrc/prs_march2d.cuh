@@ -20,6 +20,7 @@
 #include "prs_f32x2.cuh"
 #include "prs_internal.h"
 #include "prs_march2d.h"
+#include "prs_ptx.cuh"
 #include "prs_site.cuh"
 
 namespace prs {
@@ -160,6 +161,7 @@ __global__ void __launch_bounds__(kThreads, resident(T, COLS)) k_march2d(const _
     constexpr int HX = halo(T, COLS), U = width(T, COLS), NP = COLS / 2, kRow = 32 * COLS;
     __shared__ __align__(16) float ring[kWarps][2 * kRing][kRow];  // phi rows, then dphi rows; a lane reads its own slots
     __shared__ K kicks[M::kShared ? kWarps : 1][T];
+    chain_enter();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nx = a.nx, ny = a.ny;
     int w = blockIdx.x * kWarps + wid, run = 0;
     if (NR > 1) {

@@ -2,6 +2,7 @@
 // compiled in a file of its own.
 #pragma once
 
+#include "prs_chain.h"
 #include "prs_march2d.cuh"
 
 namespace prs {
@@ -40,8 +41,7 @@ cudaError_t launch_one(const Geo& g, int cy, int nruns, const MarchRun* runs, cu
     }
     const int64_t warps = (int64_t)a.nstrips * a.nchunks * nruns, blocks = (warps + kWarps - 1) / kWarps;
     if (warps > 0x7fffffff) return cudaErrorInvalidValue;
-    k_march2d<M, T, COLS, VEC, NR><<<(unsigned)blocks, kThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_march2d<M, T, COLS, VEC, NR>, dim3((unsigned)blocks), kThreads, 0, st, a);
 }
 
 template <class M, int T, int COLS>

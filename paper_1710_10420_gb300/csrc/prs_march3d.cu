@@ -40,8 +40,7 @@ cudaError_t launch3_one(const Geo& g, int nruns, const MarchRun* runs, cudaStrea
     }
     const int64_t blocks = tiles * a.nchunks;
     if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
-    k_march3d<M, T, VEC, NR><<<(unsigned)blocks, kThreads, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_march3d<M, T, VEC, NR>, dim3((unsigned)blocks), kThreads, smem, st, a);
 }
 
 template <class M, int T>
@@ -91,7 +90,7 @@ int march3d_planes(const Geo& g, int t, int nruns, double* us)
     const double lone = (march_packed(g) ? 1.0 : 1.2) * base, turn = (march_packed(g) ? 0.72 : 0.95) * base;
     int best = 1;
     double least = 1e300;
-    for (int nc = 1; nc <= g.nz && nc <= 4096; ++nc) {
+    for (int nc = 1; nc <= g.nz && nc <= 4096; nc += nc < 32 ? 1 : nc / 16) {
         const int c = (g.nz + nc - 1) / nc, n = (g.nz + c - 1) / c;
         const double w = tiles * n / slots, at_once = w < 1.0 ? tiles * n : slots;
         const double waves = w <= 1.0 ? 1.1 - 0.1 * w : 0.5 * (ceil(w) + w + 0.35);

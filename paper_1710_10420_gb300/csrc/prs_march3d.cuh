@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(kThreads, resident3(T)) k_march3d(const __grid
     constexpr int N0 = kRows + 2 * T, N1 = N0 - 2;  // rows of level 0 and of level 1
     constexpr int kPlane = (N0 + N1) * kRow;        // floats of a ring slot: phi rows, then dphi rows
     extern __shared__ __align__(16) float ring3[];
+    chain_enter();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nx = a.nx, ny = a.ny, nz = a.nz;
     // blocks: x strips fastest, then groups of kWarps row tiles, then chunks, then runs
     int b = blockIdx.x;

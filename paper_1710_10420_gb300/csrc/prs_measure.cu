@@ -28,6 +28,7 @@
 #include <type_traits>
 
 #include "prs_arith.cuh"
+#include "prs_chain.h"
 #include "prs_internal.h"
 #include "prs_ptx.cuh"
 #include "prs_reduce.cuh"
@@ -213,8 +214,9 @@ __global__ void __launch_bounds__(kMThreads, D == 2 ? 4 : 3)
               bool vec, unsigned int* err)
 {
     const int run = NR > 1 ? blockIdx.y : 0;
-    const R* __restrict__ phi = runs.phi[run];
-    const R* __restrict__ dphi = runs.dphi[run];
+    const R* phi = runs.phi[run];
+    const R* dphi = runs.dphi[run];
+    chain_enter();
     const RunConst<R>& rc = runs.rc[run];
     using A = Arith<R, true>;
     constexpr int kOff = MRow<R>::kOff, kLd = MRow<R>::kLd;
@@ -560,9 +562,8 @@ cudaError_t measure_t(const Geo& g, int nruns, const MeasureRun* q, unsigned int
     const bool vec = g.nx % MRow<R>::kOff == 0 && (bits & 15u) == 0;
     CUtensorMap map{};
     if (NR > 1 || !vec || !phi_map(&map, (const R*)q[0].phi, g, T)) err = nullptr;
-    k_measure<R, D, FAST, NR><<<dim3((unsigned)grid, (unsigned)nruns), kMThreads, measure_smem(D, sizeof(R), T), st>>>(
-        map, runs, g, T, vec, err);
-    return cudaGetLastError();
+    return launch_chained(k_measure<R, D, FAST, NR>, dim3((unsigned)grid, (unsigned)nruns), kMThreads,
+                          measure_smem(D, sizeof(R), T), st, map, runs, g, T, vec, err);
 }
 
 template <typename R, bool FAST, int NR>

@@ -27,6 +27,10 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
+// A kernel launched by launch_chained may start while the kernel before it in the stream drains: it
+// touches memory only after this, which waits for that kernel's end.
+__device__ __forceinline__ void chain_enter() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
