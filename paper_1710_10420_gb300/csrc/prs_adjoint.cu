@@ -36,6 +36,7 @@
 #include <vector>
 
 #include "prs.h"
+#include "prs_adj_march.h"
 #include "prs_arith.cuh"
 #include "prs_internal.h"
 #include "prs_reduce.cuh"
@@ -651,6 +652,12 @@ cudaError_t launch_adjoint_step(const prs_sim* s, const void* phi, const void* v
         }
         k_adjoint2d_f32<kAdjItems><<<blocks, kFastThreads, sm, s->stream>>>(T, k, rc, last, scr, err);
         return cudaGetLastError();
+    }
+    if (s->p.precision == PRS_FP32 && g.dims == 3) {
+        const float k[5] = {(float)c.c1, (float)c.c2, (float)c.cV, (float)c.dc1, (float)c.dc2};
+        const cudaError_t e = launch_adj_march(g, (const float*)phi, (const float*)v, k, (const float*)lt_in,
+                                               (float*)lt_out, (float*)lphi, s->rc, last, scr, s->stream);
+        if (e != cudaErrorNotSupported) return e;
     }
     const dim3 grid = grid_for(g);
     if ((int)(grid.x * grid.y) > scr.max_blocks) return cudaErrorInvalidValue;
