@@ -2,9 +2,13 @@
 //
 //   init     : SplitMix64 random field (Sec. III initial conditions), dphi = 0
 //   step     : Eqs. 3-5 with the damping of Eq. 6, one thread per site, any box
-//              side >= 3 (used for sides that are not a multiple of 4, for FP64 and
-//              for the ragged cases the fast kernels do not take)
+//              side >= 3 (used for PRS_REPRO and for FP32 3D boxes whose planes hold
+//              2^32 sites or more)
+//   copy     : both fields of a state in one launch
+#include <cuda.h>
 #include <cuda_runtime.h>
+
+#include <atomic>
 
 #include "prs_arith.cuh"
 #include "prs_chain.h"
@@ -168,13 +172,44 @@ __global__ void __launch_bounds__(256) k_copy_state(const float4* p, float4* po,
     }
 }
 
+// Whether the kernel may read bytes at p: memory of the current device, in one allocation.  (A copy
+// by the driver finds out by itself and returns an error; a kernel would fault.)
+static bool on_device(const void* p, size_t bytes)
+{
+    using Range = decltype(&cuMemGetAddressRange);
+    static std::atomic<Range> fn{nullptr};
+    Range range = fn.load(std::memory_order_acquire);
+    if (!range) {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess || !f) {
+            cudaGetLastError();
+            return false;
+        }
+        range = reinterpret_cast<Range>(f);
+        fn.store(range, std::memory_order_release);
+    }
+    cudaPointerAttributes attr;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    return attr.type == cudaMemoryTypeDevice && attr.device == dev &&
+           range(&base, &size, (CUdeviceptr)p) == CUDA_SUCCESS && (CUdeviceptr)p - base <= size &&
+           bytes <= size - (size_t)((CUdeviceptr)p - base);
+}
+
 cudaError_t launch_copy_state(const void* phi, void* phi_out, const void* dphi, void* dphi_out, size_t bytes,
                               cudaStream_t st)
 {
     const uintptr_t a = (uintptr_t)phi, b = (uintptr_t)phi_out, c = (uintptr_t)dphi, d = (uintptr_t)dphi_out;
     auto apart = [&](uintptr_t s, uintptr_t t) { return s + bytes <= t || t + bytes <= s; };
     if (((a | b | c | d | bytes) & 15u) || !apart(a, b) || !apart(a, d) || !apart(c, b) || !apart(c, d) ||
-        !apart(b, d)) {
+        !apart(b, d) || !on_device(phi, bytes) || !on_device(dphi, bytes)) {
         cudaError_t e = cudaSuccess;  // one after the other
         if (a != b) e = cudaMemcpyAsync(phi_out, phi, bytes, cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess && c != d) e = cudaMemcpyAsync(dphi_out, dphi, bytes, cudaMemcpyDeviceToDevice, st);
