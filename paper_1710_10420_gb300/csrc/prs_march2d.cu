@@ -11,34 +11,37 @@ bool march_packed(const Geo& g)
     return fast_step_ok(g, PRS_FP32) || default_fused_steps(g, PRS_FP32, false) > 1;
 }
 
-// A warp's iteration takes the chain of its levels, or its scheduler's turns for all its warps,
-// whichever is longer; a pass takes its waves of iterations or its bytes, and a launch (2.3 us from
-// one kernel's end to the next's start).  Cycles at 1.9 GHz, measured per level and iteration (256^2
-// to 4096^2): a lone warp 100 (two columns a lane: 78), each warp of a busy scheduler 92 (60); a
-// third more with the unpacked arithmetic.  So small boxes take pairs and short chunks, which make
-// warps, and boxes of 512^2 and more take quads and chunks of 20 to 60 rows, which waste fewer of
-// their rows and columns (2048^2, T = 4: 16.5 us with quads, 20.6 with pairs).
+// Every scheduler holds as many warps as its SM holds blocks (b), so a pass takes the iterations of a chunk
+// times what an iteration takes among b warps, or its bytes, and a launch (1.7 us from one kernel's end
+// to the next's start).  Cycles of an iteration at 1.9 GHz, measured from 256^2 to 4096^2: a lone
+// warp with four columns a lane 185 + 43 T, b of them 0.76 b times that; with two columns 150 + 40 T,
+// b of them 0.3 + 0.51 b; a fifth more with the unpacked arithmetic.  The last block decides, so the rows
+// of a chunk are the fewest that fill every SM with b blocks and no SM with one more: 4096^2, T = 5, 128
+// rows and b = 2 46.4 us, 229 rows and 1.1 blocks an SM on average 78; 2048^2 15.3 and 23.4.  Small boxes
+// come out with pairs, which make warps, boxes of 512^2 and more with quads, which waste fewer of their
+// columns.
 static double march_us(const Geo& g, int t, int nruns, MarchShape* best)
 {
-    const int sms = sm_count_current();
-    const double plain = march_packed(g) ? 1.0 : 1.3;
+    const int64_t per_b = (int64_t)sm_count_current() * march::kWarps;  // warps of a block an SM
+    const double plain = march_packed(g) ? 1.0 : 1.2;
     double least = 1e300;
     for (int cols = 2; cols <= 4; cols += 2) {
-        const int u = march::width(t, cols);
+        const int u = march::width(t, cols), r = march::resident(t, cols);
         const int64_t strips = (int64_t)((g.nx + u - 1) / u) * nruns;
-        const int64_t slots = (int64_t)sms * march::resident(t, cols) * march::kWarps;
-        const double chain = plain * (cols == 4 ? 100.0 : 78.0) * t, turn = plain * (cols == 4 ? 92.0 : 60.0) * t;
-        for (int cy = 1;; cy += cy < 16 ? 1 : cy / 8) {
-            if (cy > g.ny) cy = g.ny;
-            const int64_t warps = strips * ((g.ny + cy - 1) / cy), waves = (warps + slots - 1) / slots;
-            const double most = (double)(waves > 1 ? slots : warps);  // warps at once
-            const double cost = (double)waves * (cy + 2 * t) * std::max(chain, most / (4.0 * sms) * turn);
+        const double lone = plain * (cols == 4 ? 185.0 + 43.0 * t : 150.0 + 40.0 * t);
+        const auto among = [&](int64_t b) { return std::max(1.0, cols == 4 ? 0.76 * b : 0.3 + 0.51 * b); };
+        for (int64_t b = 1; b <= 4 * r || least == 1e300; b += b < 4 * r ? 1 : b) {
+            const int64_t most = std::min<int64_t>(b * per_b / strips, g.ny);  // chunks
+            if (most < 1) continue;
+            const int cy = (int)((g.ny + most - 1) / most);
+            const double waves = (double)(b / r) * among(r) + (b % r ? among(b % r) : 0.0);
+            const double cost = waves * lone * (cy + 2 * t);
             if (cost < least * 0.999) least = cost, *best = MarchShape{cols, cy};
-            if (cy == g.ny) break;
+            if (most == g.ny) break;
         }
     }
-    const double bytes = 16.0 * (double)g.S * nruns;  // beyond L2: 5.4 TB/s
-    return 2.3 + std::max(least / 1900.0, bytes > 1e8 ? bytes / 5.4e6 : bytes / 1.2e7);
+    const double bytes = 16.0 * (double)g.S * nruns;  // beyond L2: 6.1 TB/s
+    return 1.7 + std::max(least / 1900.0, bytes > 1e8 ? bytes / 6.1e6 : bytes / 1.2e7);
 }
 
 void march_plan(const Geo& g, int nruns, MarchPlan* p)

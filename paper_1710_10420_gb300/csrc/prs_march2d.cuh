@@ -13,6 +13,10 @@
 // when each level's rows pass through shared memory) and, on boxes larger than L2, HBM at 16 B per
 // T site-updates.  Both sides of a row are recomputed instead of exchanged, which is what lets warps
 // run without waiting for one another.  phi and dphi are read across sites, so both go out of place.
+//
+// Measured (an output interval of 10 steps and the diagnostics, us; with the one- to three-step passes
+// over rows in shared memory, or one thread a site on ragged boxes, that this replaced): 256^2 42 (82),
+// 2048^2 87 (158), 4096^2 215 (375), 2500 x 1701 94 (328).
 #pragma once
 
 #include <cuda_runtime.h>
