@@ -1,9 +1,9 @@
 """Benchmark of the PRS hot path on GB300: site-updates/s and the HBM roofline fraction.
 
-One benchmark step = one output interval of the paper's runs: ``--interval`` (20)
-leapfrog steps (Eqs. 3-6), the first of them fused with the wall diagnostics (Eq. 7,
-Eq. 8) of the state it reads, reduced in FP64 and read back on the host.  Default workload: 3D 1024^3 FP32, PRS (alpha=3,
-beta=0), radiation era, deta=0.1, seeded uniform(-1,1) initial field.
+One benchmark step = one output interval of the paper's runs: the wall diagnostics (Eq. 7,
+Eq. 8) of the current state, reduced in FP64 and read back on the host, and ``--interval`` (20)
+leapfrog steps (Eqs. 3-6).  Default workload: 3D 1024^3 FP32, PRS (alpha=3, beta=0), radiation
+era, deta=0.1, seeded uniform(-1,1) initial field.
 
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--workload 3d1024|2d4096|3d512]
        python bench.py --impl reference ...   (the FP64 oracle on the host cores)
@@ -29,7 +29,7 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 WORKLOADS = {
-    # name: (shape, fused-steps-per-pass default, description)
+    # name: (shape, description)
     "3d1024": ((1024, 1024, 1024), "3D 1024^3 FP32 PRS step (7-point), radiation era, deta=0.1, "
                                    "20 steps + FP64 wall diagnostics per output"),
     "3d512": ((512, 512, 512), "3D 512^3 FP32 PRS step, radiation era, 20 steps + FP64 wall diagnostics"),
@@ -51,7 +51,7 @@ def parse():
     ap.add_argument("--impl", default="gb300", choices=["gb300", "reference"])
     ap.add_argument("--workload", default="3d1024", choices=sorted(WORKLOADS))
     ap.add_argument("--interval", type=int, default=20, help="leapfrog steps per diagnostic output")
-    ap.add_argument("--tblock", type=int, default=0, help="fused steps per HBM pass (0: library default)")
+    ap.add_argument("--tblock", type=int, default=0, help="fused steps per HBM pass (0: library's plan)")
     ap.add_argument("--e2e-steps", type=int, default=40)
     ap.add_argument("--no-cpu", action="store_true", help="skip the oracle CPU baseline")
     ap.add_argument("--no-batch", action="store_true", help="skip the ensemble (batched vs one-at-a-time) figure")
@@ -264,15 +264,14 @@ def peaks():
 
 # the sources that define the FP32 step kernels (device code and the structs they take),
 # by steps per pass
-STEP_KERNEL_SOURCES = {1: ("prs_fast.cu", "prs_tile.cuh", "prs_ptx.cuh", "prs_internal.h", "prs_reduce.cuh",
-                           "prs_f32x2.cuh"),
+STEP_KERNEL_SOURCES = {1: ("prs_fast.cu", "prs_tile.cuh", "prs_ptx.cuh", "prs_internal.h", "prs_f32x2.cuh"),
                        2: ("prs_t2tma.cu", "prs_tile.cuh", "prs_ptx.cuh", "prs_internal.h", "prs_f32x2.cuh",
                            "prs_tmap.h"),
-                       3: ("prs_t3tma.cu", "prs_tile.cuh", "prs_ptx.cuh", "prs_internal.h", "prs_f32x2.cuh",
-                           "prs_tmap.h")}
+                       3: ("prs_march3d.cuh", "prs_march3d.cu", "prs_march2d.cuh", "prs_march2d.h", "prs_tile.cuh",
+                           "prs_ptx.cuh", "prs_internal.h", "prs_f32x2.cuh")}
 STEP_KERNELS_3D = {1: "k_step3d_f32, one leapfrog step per pass",
                    2: "k_step3d_t2tma, two leapfrog steps per pass",
-                   3: "k_step3d_t3tma, three leapfrog steps per pass"}
+                   3: "k_march3d, three leapfrog steps per pass"}
 
 
 def kernel_sources_sha(names=STEP_KERNEL_SOURCES[2]) -> str:
@@ -305,7 +304,7 @@ def traffic_record(workload: str, tblock: int):
 
 class OwnedRun:
     """A run whose fields the library allocates (prs_create without prs_bind): after an odd number of
-    two-step passes its two dphi buffers swap roles, so every call keeps all its pairs."""
+    multi-step passes its two dphi buffers swap roles, so every call keeps all its passes."""
 
     def __init__(self, prs, shape, stream, **kw):
         self.prs = prs
@@ -319,13 +318,9 @@ class OwnedRun:
 
 
 def interval_calls(interval: int, tb: int, tmax: int = 0):
-    """An output interval as (pure, tail, tail_launches) after prs_step_measure(1), which takes the
-    diagnostics of the start state inside a one-step pass: prs_step(pure) is passes of the step
-    kernel only (with two steps per pass an even number of steps), prs_step(tail) the rest.  With two
-    steps per pass the remainder of an even interval is one single step, or, where the box takes
-    three-step passes (tmax >= 3) and the library picks the passes (tblock = 0), one pair and that
-    step as one three-step pass.  The run's buffers are library-owned, so every call keeps its
-    multi-step passes."""
+    """The steps of an interval after its first as (pure, tail, tail_launches): prs_step(pure) is
+    passes of tb steps only, prs_step(tail) the rest: single steps, or with tb = 2 on a box that takes
+    three-step passes (tmax >= 3), the odd step and a pair as one three-step pass."""
     rest = interval - 1
     tail = rest % tb
     if tb == 2 and tail == 1 and tmax >= 3 and rest >= 3:
@@ -346,12 +341,13 @@ def run_gpu(args, world, rank, local):
     stream = torch.cuda.Stream(dev)
     run = OwnedRun(prs, shape, stream, seed=1000 + rank, tblock=args.tblock)
     prs.prs_init(run.handle)
-    tb = args.tblock if args.tblock > 0 else lib_default_tblock(prs, shape)
-    # one bench step = one output interval: the diagnostics of its start state fused into its
-    # first step (prs_step_measure(1)), then the other steps: prs_step(pure), passes of the step
-    # kernel only (bracketed by events on the run's stream), and prs_step(tail)
-    tmax = prs.prs_max_tblock(run.params) if args.tblock == 0 else tb
-    pure, tail, tail_launches = interval_calls(args.interval, tb, tmax)
+    # one bench step = one output interval: the diagnostics of its start state, then its steps:
+    # prs_step(pure), passes of the step kernel only (bracketed by events on the run's stream), and
+    # prs_step(tail), the pass of the steps that remain.  Without a tblock the library steps these
+    # boxes in passes of three (3D) and five (2D) steps.
+    tb = min(args.tblock, prs.prs_max_tblock(run.params)) if args.tblock > 0 else (3 if len(shape) == 3 else 5)
+    pure, tail, _ = interval_calls(args.interval + 1, tb)
+    tail_launches = 1 if tail else 0
     pure_launches = pure // tb
     step_launches = pure_launches + tail_launches
 
@@ -359,7 +355,7 @@ def run_gpu(args, world, rank, local):
         e = [torch.cuda.Event(enable_timing=True) for _ in range(4)] if events is not None else [None] * 4
         rec = (lambda ev: ev.record(stream)) if events is not None else (lambda ev: None)
         rec(e[0])
-        d = prs.prs_step_measure(run.handle, 1)
+        d = prs.prs_measure_ex(run.handle)
         rec(e[1])
         if pure:
             prs.prs_step(run.handle, pure)
@@ -387,9 +383,9 @@ def run_gpu(args, world, rank, local):
     barrier(world)
     ms = start.elapsed_time(stop)
     ms_max = allreduce_max(ms, world, dev)
-    # the second bracket holds only launches of the step kernel (for interval = 20 and two
-    # steps per pass: nine two-step passes), so its mean launch duration is total / launches
-    fused_ms = sum(e[0].elapsed_time(e[1]) for e in events) / len(events)
+    # the second bracket holds only launches of the step kernel (for interval = 20 and three
+    # steps per pass: six passes), so its mean launch duration is total / launches
+    diag_ms = sum(e[0].elapsed_time(e[1]) for e in events) / len(events)
     pure_ms = sum(e[1].elapsed_time(e[2]) for e in events) / len(events)
     tail_ms = sum(e[2].elapsed_time(e[3]) for e in events) / len(events)
     launch_avg_ms = pure_ms / pure_launches if pure_launches else tail_ms / max(step_launches, 1)
@@ -425,9 +421,8 @@ def run_gpu(args, world, rank, local):
                 "effective_gbs": effective, "effective_frac": effective / peak,
                 "launch_ms": launch_avg_ms, "peak_source": f"{peak_kind} hbm_gbs (copy)",
                 "nominal_peak": NOMINAL_HBM_GBS, "frac_of_nominal": achieved / NOMINAL_HBM_GBS,
-                "fused_step_and_diagnostics_ms": fused_ms, "tail_passes_ms": tail_ms, "tail_steps": tail,
-                "tail_pass": ("one three-step pass (k_step3d_t3tma)" if tail == 3 and tail_launches == 1 else
-                              f"{tail} single step(s)" if tb == 2 or tb == 1 else f"{tail} step(s)")}
+                "diagnostics_ms": diag_ms, "tail_passes_ms": tail_ms, "tail_steps": tail,
+                "tail_pass": f"one pass of {tail} step(s)" if tail else "none"}
     if rec:
         roofline["dram_frac"] = rec["dram_bytes_per_launch"] / (launch_avg_ms / 1e3) / 1e9 / peak
 
@@ -443,14 +438,14 @@ def run_gpu(args, world, rank, local):
         "repeats": repeats,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": desc, "shape": list(shape), "interval": args.interval,
-                   "diagnostics": "of the state at the start of each interval, fused into its first step",
+                   "diagnostics": "of the state at the start of each interval (one pass)",
                    "fused_steps_per_pass": tb,
                    "l2": (f"inputs larger than L2 (state {state_gb:.1f} GB: phi, phi', dphi"
                           + (" and the second dphi buffer of multi-step passes)" if tb >= 2 else ")"))
                    if sites >= 512 ** 3 else "state comparable to L2; not flushed", "parallelism": f"replicas x{world}",
                    "last_output": {"area_per_volume": d.area_per_volume, "gamma_v": d.gamma_v, "step": d.step}},
         "roofline": roofline, "e2e": e2e, "clocks": clocks,
-        "gpu_launches": args.steps * (step_launches + 1),  # one fused step+diagnostics launch per interval
+        "gpu_launches": args.steps * (step_launches + 1),  # one launch of the diagnostics per interval
     }
     run.close()
     if rank == 0 and not args.no_2d and args.workload != "2d4096":
@@ -468,11 +463,6 @@ def run_gpu(args, world, rank, local):
     if rank == 0:
         print(json.dumps(line), flush=True)
     return 0
-
-
-def lib_default_tblock(prs, shape) -> int:
-    """Steps the library fuses per pass by default for this box (FP32)."""
-    return prs.prs_default_tblock(prs.make_params(shape))
 
 
 def run_e2e(args, prs, sim, shape, stream, dev, world) -> dict:
@@ -543,7 +533,7 @@ def ensemble_runs(scale: float = 1.0):
 
 
 def run_batch_figure(prs, stream, dev, scale: float) -> dict:
-    """Batched persistent launch vs one prs_step loop per run, on the same ensemble and outputs."""
+    """The ensemble calls vs one prs_step_measure loop per run, on the same ensemble and outputs."""
     import torch
 
     runs = ensemble_runs(scale)
@@ -566,7 +556,7 @@ def run_batch_figure(prs, stream, dev, scale: float) -> dict:
     budget = prs.prs_batch_tuning(b, 0)[1]
     prs.prs_batch_destroy(b)
     # one run at a time, with the library's fastest single-run path: each output interval is one
-    # prs_step_measure (the diagnostics of its start state fused into its first pass), and the
+    # prs_step_measure (the diagnostics of its start state, then its steps), and the
     # state after the last interval is measured by prs_measure_ex when it falls on an output
     a.record(stream)
     for (s, m, sd, n) in runs:
@@ -589,9 +579,8 @@ def run_batch_figure(prs, stream, dev, scale: float) -> dict:
             "site_updates": total, "batched_s": ms_batch / 1e3, "one_at_a_time_s": ms_seq / 1e3,
             "batched_value": total / (ms_batch / 1e3), "one_at_a_time_value": total / (ms_seq / 1e3),
             "unit": "site-updates/s", "speedup": ms_seq / ms_batch, "create_s": t_create,
-            "tuned_tile_len": tl, "tile_len_0": "a class of boxes stepped alone after the persistent launch of the others, "
-            "each pass launched once for up to 16 runs of the box (boxes of 2^22 sites and more, or 2D "
-            "classes of 8+ runs with 1024-column rows; multi-step passes)", "tuned_group_bytes": budget,
+            "tuned_tile_len": tl, "tile_len_0": "a box whose groups fill the GPU by themselves; "
+            "otherwise the most runs a launch groups", "tuned_group_bytes": budget,
             "first_output_run0": list(out[0, 0])}
 
 
@@ -652,8 +641,8 @@ def run_2d_figure(prs, stream, dev, interval: int) -> dict:
     sim = prs.Sim(shape, stream=stream, device=dev, seed=3)
     sim.init()
     for _ in range(5):
-        prs.prs_step_measure(sim.handle, 1)
-        prs.prs_step(sim.handle, interval - 1)
+        prs.prs_measure_ex(sim.handle)
+        prs.prs_step(sim.handle, interval)
     a, z = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     b0, b1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     k = 100
@@ -661,9 +650,9 @@ def run_2d_figure(prs, stream, dev, interval: int) -> dict:
     torch.cuda.synchronize(dev)
     a.record(stream)
     for _ in range(k):
-        prs.prs_step_measure(sim.handle, 1)
+        prs.prs_measure_ex(sim.handle)
         b0.record(stream)
-        prs.prs_step(sim.handle, interval - 1)
+        prs.prs_step(sim.handle, interval)
         b1.record(stream)
         b1.synchronize()
         step_ms += b0.elapsed_time(b1)
@@ -672,15 +661,15 @@ def run_2d_figure(prs, stream, dev, interval: int) -> dict:
     ms = a.elapsed_time(z)
     sim.close()
     peak, kind = peaks()
-    per_step = step_ms / (k * (interval - 1))  # the plain steps of an interval, in multi-step passes
-    tb = lib_default_tblock(prs, shape)
+    per_step = step_ms / (k * interval)  # the steps of an interval, in multi-step passes
+    tb = 5  # the library's plan of this box
     return {"workload": "2D 4096^2 FP32 PRS step (5-point), radiation era, 20 steps + FP64 wall diagnostics "
                         "(state 192 MB: L2-sized, not flushed)",
             "value": sites * interval * k / (ms / 1e3), "unit": "site-updates/s", "ms_per_step": ms / k,
             "fused_steps_per_pass": tb, "ms_per_leapfrog_step": per_step,
             "effective_frac_of_copy_bw": 16.0 * sites / (per_step / 1e3) / 1e9 / peak,
-            "note": "effective = 16 B per site-update over the time per step; with two or three steps per "
-                    "pass the DRAM traffic is a half or a third of that"}
+            "note": "effective = 16 B per site-update over the time per step; with five steps per "
+                    "pass the DRAM traffic is a fifth of that"}
 
 
 def run_precision_figure(prs, stream, dev) -> dict:
@@ -717,20 +706,21 @@ def run_precision_figure(prs, stream, dev) -> dict:
     del ga, gb
     torch.cuda.empty_cache()
     fp64_tflops = 2 * 4096 ** 3 / (best / 1e3) / 1e12
-    # the non-reproducible FP64 step issues 11 double instructions a site-update (5 adds of the
+    # a kick and drift in doubles takes 11 double instructions a site-update (5 adds of the
     # Laplacian's pairs, 2 multiplies, 4 fused multiply-adds), each one issue of the FP64 pipe
-    # that a DGEMM fills with fused multiply-adds (2 flops each)
+    # that a DGEMM fills with fused multiply-adds (2 flops each); the step evaluates the force in
+    # 64-bit integers instead, so it may pass this bound
     dp_inst = 11
     alu_bound = fp64_tflops * 1e12 / 2 / dp_inst
     value = sites / (ms / 1e3)
-    fp64 = {"workload": "3D 512^3 FP64 (generic kernel, folded kick, FMA)", "ms_per_step": ms,
+    fp64 = {"workload": "3D 512^3 FP64 (force in 64-bit fixed point, kick and drift in doubles)", "ms_per_step": ms,
             "value": value, "unit": "site-updates/s",
             "bound": "alu", "fp64_peak_tflops_measured": fp64_tflops,
             "fp64_peak_source": "cuBLAS DGEMM 4096^3 through torch on this GPU, best of 5",
             "dp_instructions_per_site_update": dp_inst, "alu_bound_value": alu_bound,
             "frac_of_alu_bound": value / alu_bound, "hbm_bound_value": peak * 1e9 / 32.0,
-            "note": "32 B per site-update in FP64 would allow the HBM-bound value; GB300 issues FP64 at a "
-                    "small fraction of its FP32 rate, so the FP64 pipe bounds the step"}
+            "note": "32 B per site-update in FP64 would allow the HBM-bound value; alu_bound_value is what the "
+                    "FP64 pipe allows a step done in doubles throughout"}
     # FP32 vs FP64 diagnostics of the same initial field, eta 1 -> 256 (2550 steps), every 10 steps
     # (FP32 with correctly rounded division and square root in the diagnostics: same fields)
     shape2 = (512, 512)

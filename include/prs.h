@@ -101,11 +101,10 @@ typedef struct {
     double phi0;       /* vacuum value (> 0)                                        */
     uint64_t seed;     /* seed of the random initial field (prs_init with NULL)     */
     uint32_t flags;    /* PRS_REPRO | PRS_FP32_CR | PRS_DEBUG, or 0                 */
-    int32_t tblock;    /* leapfrog steps per pass over HBM: 0 = library's choice (FP32
-                          3D: 1 below 2^24 sites, else 2 where the two-step tiles get at
-                          least 4 rows of y; FP32 2D: 3 on rows of 2048 or more and on
-                          boxes of at most 1024 rows, else 2 from 2^24 sites and 1
-                          below; otherwise 1; see prs_default_tblock); 2 = two-step passes for FP32 boxes with
+    int32_t tblock;    /* leapfrog steps per pass over HBM: 0 = library's choice (FP32: a
+                          mix of passes of 1 to 3 steps in 3D and 1 to 5 in 2D, whichever
+                          takes least time on this machine; FP64: 1); 1 = one step per pass;
+                          2 = two-step passes for FP32 boxes with
                           an x side that is a multiple of 128 (3D; z side >= 3) or a
                           multiple of 128 up to 4096 (2D), else 1; 3 = three-step
                           passes for FP32 3D boxes with an x side that is a multiple
@@ -156,23 +155,25 @@ int prs_init(prs_sim* sim, const void* h_phi, const void* h_dphi);
  * without waiting (the call never allocates, so it may be captured into a CUDA graph).
  * Step n uses delta_n, eta_n = eta0 + n deta.  Every step of the call must satisfy the
  * stability limit (checked at both ends, where the force prefactor a^beta is largest),
- * else PRS_EINVAL.  Passes of two or three steps (see prs_params.tblock) read dphi
+ * else PRS_EINVAL.  Passes of two and more steps (see prs_params.tblock) read dphi
  * across sites and write it out of place, into a second dphi buffer that prs_init,
- * prs_set_state or prs_set_state_device allocate when the run takes multi-step passes
- * (owned by the run, freed by prs_destroy; if that allocation fails, the steps run one
- * per pass).  A call of nsteps runs nsteps / T passes of T = tblock steps, then (T = 3)
- * one pair if two steps remain, then single steps; when the library chooses the steps per
- * pass (tblock = 0, T = 2) on a box that takes three-step passes, an odd count runs one
- * three-step pass instead of a pair and a single step.  Where dphi ends:
+ * prs_set_state or prs_set_state_device allocate when the run may take such passes (FP32
+ * with tblock = 0, or a tblock that fuses steps on its box;
+ * owned by the run, freed by prs_destroy; if that allocation fails, the steps run one
+ * per pass).  With tblock = 0 a call of nsteps runs the passes that its plan of the box
+ * gives the least time, the longest first, single steps last.  With T = tblock >= 2 it runs
+ * nsteps / T passes of T steps, then (T = 3) one pair if two steps remain, then single
+ * steps.  Where dphi ends:
  *   - library-owned buffers (no prs_bind, no PRS_DEBUG): after an odd number of
  *     multi-step passes the two dphi buffers swap roles; every step count keeps all its
  *     passes.  prs_device_state returns the current buffer.
  *   - bound buffers (prs_bind) or PRS_DEBUG: dphi ends in the run's own buffer after
  *     every call.  After an odd number of multi-step passes the first single step brings
- *     dphi home; with no single step to do it, the three-step pass of an odd T = 2 count
- *     runs as a pair and a single step, else the last pair as two single steps (T = 2:
- *     counts 2, 6, 10, ...; T = 3: counts 2, 8, 14, ...), else the last triple as a pair
- *     and a single step (T = 3: counts 3, 9, 15, ...). */
+ *     dphi home; plans without single steps then take an even number of passes where that
+ *     is possible, else the last pass as shorter ones (T = 2: the last pair of 2, 6, 10, ...
+ *     steps as two single steps; T = 3: the last pair of 2, 8, 14, ..., or the last triple
+ *     of 3, 9, 15, ... as a pair and a single step).
+ * FP32 passes of any length give the same bits as one step per pass. */
 int prs_step(prs_sim* sim, int64_t nsteps);
 
 /* Wall diagnostics of the current state (Eq. 7, Eq. 8), reduced on the device in
@@ -261,28 +262,20 @@ int prs_measure_noalloc(const prs_params* params, const void* d_phi, const void*
 int prs_destroy(prs_sim* sim);
 
 /* --------------------------------------------------------------- ensembles
- * Many independent runs (the paper's sets of realisations, Sec. III) advanced by
- * one persistent kernel: every run is cut into tiles and the work items
- * (run, tile, step) are taken in an order in which each item only waits, with a
- * bounded spin, for items already taken; diagnostics are fused into the steps
- * that read the same state.  Runs must be FP32 with an x side that is a multiple
- * of 128 dividing 4096 (3D: at most 1024) and 4096/x dividing the y side. */
+ * Many independent runs (the paper's sets of realisations, Sec. III).  Runs of one
+ * box are stepped together: each pass, and each output's diagnostics, is one launch over
+ * up to 16 of them, and the groups run concurrently.  Runs must be FP32 with an x side
+ * that is a multiple of 128 dividing 4096 (3D: at most 1024) and 4096/x dividing the y
+ * side. */
 
 /* Create an ensemble of nruns runs (each validated as by prs_create), allocate all
- * fields, pick a tile length for each geometry class of runs (4 to 32 planes or bands)
- * and the L2 grouping by timing short trials on them (the autotuner), then set every
- * run to its seeded random initial condition (step 0).  A run that the library steps
- * with multi-step passes (prs_default_tblock >= 2) and whose box has 2^22 sites or more
- * (it fills the GPU by itself), or, in 2D, 2^20 sites or more in rows of at least 1024
- * columns with at least 8 runs of that box in the ensemble (their passes are launched
- * together), is stepped alone, after the persistent launch of the others, as
- * prs_step_measure would step it (its fields and outputs are those of the same run
- * stepped alone; the run holds a second dphi buffer like a prs_sim).  stream may be
- * NULL (the ensemble then creates its own stream). */
+ * fields, then set every run to its seeded random initial condition (step 0).  A run's
+ * fields are those of the same run stepped alone, bit for bit; its diagnostic sums agree
+ * to FP64 rounding.  stream may be NULL (the ensemble then creates its own stream). */
 int prs_batch_create(const prs_params* runs, int nruns, void* stream, prs_batch** out);
 
-/* Advance run r by nsteps_per_run[r] (>= 0) steps: one persistent launch for the runs
- * it holds, then the runs stepped alone, all on the ensemble's stream.  With
+/* Advance run r by nsteps_per_run[r] (>= 0) steps, in grouped passes on streams forked
+ * from and joined to the ensemble's stream.  With
  * measure_every > 0, the diagnostics of run r at its steps n, n+m, ... (n its
  * step at the call, up to n + nsteps_per_run[r]) are written to
  *   out_series[(r*out_capacity + k)*4 + {0,1,2,3}] = {step, A/V, gamma v, n_links}
@@ -299,8 +292,10 @@ int prs_batch_get_state(prs_batch* batch, int run, void* h_phi, void* h_dphi, in
 /* Overwrite run `run`'s fields from host arrays and set its step index. */
 int prs_batch_set_state(prs_batch* batch, int run, const void* h_phi, const void* h_dphi, int64_t n);
 
-/* The autotuner's choice: tile length of `run` (bands of 4096/x rows in 2D,
- * z-planes in 3D; 0 for a run stepped alone) and the bytes of fields per L2 group. */
+/* How run `run` is scheduled: *tile_len is 0 for boxes whose groups fill the GPU by
+ * themselves (multi-step passes by default and 2^22 sites or more, or 2D classes of at least 8
+ * runs of 2^20 sites or more in rows of at least 1024 columns), else the most runs a
+ * launch groups; *group_bytes is the size of the fields of its box's runs. */
 int prs_batch_tuning(prs_batch* batch, int run, int* tile_len, double* group_bytes);
 
 /* Release the ensemble and everything it allocated. */
@@ -344,8 +339,9 @@ int prs_adjoint_timing(prs_sim* sim, double ms[3]);
  * out[4] = d delta_n / d alpha. */
 int prs_coefficients(const prs_params* params, int64_t n, double out[5]);
 
-/* Leapfrog steps the library fuses into one pass over HBM for these parameters
- * when params->tblock is 0 (>= 1), or a negative status for invalid parameters. */
+/* The fixed number of leapfrog steps per pass over HBM that suits these parameters (>= 1),
+ * or a negative status for invalid parameters.  (A run with params->tblock 0 mixes passes
+ * of several lengths; see prs_params.tblock.) */
 int prs_default_tblock(const prs_params* params);
 
 /* The most leapfrog steps one pass over HBM can fuse for these parameters (>= 1; a

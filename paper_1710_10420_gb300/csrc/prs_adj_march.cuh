@@ -2,10 +2,10 @@
 //
 // The staged sweep (k_adjoint3d_f32) takes boxes whose rows and y side fit its tiles, at the copy
 // bandwidth.  On other boxes one thread a site read lt and its neighbours, phi and its neighbours, dphi
-// and lphi one by one (250^3: 304 us a step; here 84.  128 x 104 x 200: 84 and 19).  Here a warp owns 64 columns (a pair a lane) of four rows and
-// marches along z as the forward march does (prs_march3d.cuh): lt's z neighbours wait in registers, its y
-// neighbours are the warp's other rows, x neighbours come by shuffle, and everything an iteration uses
-// comes in one slot of a ring each lane fills ahead for itself.  The dJ/dalpha term takes phi (L lt) for
+// and lphi one by one (250^3: 304 us a step; here 84.  128 x 104 x 200: 84 and 19).  Here a warp owns 64
+// columns (a pair a lane) of four rows and marches along z as the forward march does (prs_march3d.cuh):
+// lt's z neighbours wait in registers, its y neighbours are the warp's other rows, x neighbours come by
+// shuffle, and everything an iteration uses comes in one slot of a ring each lane fills ahead for itself.  The dJ/dalpha term takes phi (L lt) for
 // lt (L phi), as the staged sweep does, so phi is read at the site only.
 //
 // (Two steps a pass, 32 bytes a site instead of 48 with lt and lphi between them in registers, took 219

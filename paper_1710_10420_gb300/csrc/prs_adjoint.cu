@@ -20,8 +20,9 @@
 // (at the first step of the run it writes lv_n0 = c1 lt_n0 instead): 24 bytes per
 // site in FP32, one pass.  The L phi of dJ/dalpha becomes phi (L lt) in the sum over
 // sites (L is symmetric), so phi is never read across sites in the FP32 kernels,
-// which stage all four fields in shared memory with the TMA engine (prs_tile.cuh
-// does the same for the forward step); the generic kernel keeps the form above.
+// which stage all four fields in shared memory with the TMA engine, or on 3D boxes
+// without its alignment row by row (prs_adj_march.cuh); the generic kernel keeps the
+// form above.
 //
 // The forward states are either all kept (when they fit in device memory: GB300's
 // HBM holds e.g. 1271 states of a 256^3 FP32 run) or checkpointed every K steps

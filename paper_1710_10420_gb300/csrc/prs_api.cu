@@ -570,8 +570,8 @@ int prs::check_device_error(prs_sim* s)
     return PRS_ETIMEOUT;
 }
 
-// The staged FP32 diagnostic kernels (alone or fused into a step) serve this run;
-// PRS_FP32_CR asks for the generic kernel's correctly rounded division and sqrt.
+// The FP32 diagnostics may take the hardware's reciprocals and roots; PRS_FP32_CR asks for
+// correctly rounded division and sqrt, as do boxes off the staged tiles.
 static bool fast_diag_ok(const prs_sim* s)
 {
     return fast_step_ok(s->g, s->p.precision) && (s->p.flags & PRS_FP32_CR) == 0;

@@ -11,6 +11,10 @@
 // What bounds it: instruction issue.  The two outer rows of each level are computed twice (T = 2:
 // 1.25 updates an output and step, and 64/60 for the columns), which is what lets a warp run without
 // waiting for its neighbours at a barrier, on boxes whose rows have no alignment for tensor copies.
+//
+// Measured: 512^3, T = 3, 522 us a pass, 382 M warp instructions at 0.59 of the issue slots, 2.16 GB
+// of DRAM traffic for 2.15 GB of fields in and out; 1024^3 1.21 ms a step (pairs of staged tiles 1.37);
+// 450 x 421 x 380 128 us a step (one thread a site: 571); 128^3 6.7 us a step (staged, short chunks: 9.6).
 #pragma once
 
 #include "prs_march2d.cuh"

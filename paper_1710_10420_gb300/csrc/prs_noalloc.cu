@@ -114,9 +114,8 @@ extern "C" int prs_measure_noalloc(const prs_params* p, const void* d_phi, const
     double rcd[6] = {p->deta, 1.0 / (p->dx * p->dx), 1.0 / (p->phi0 * p->phi0), (double)(2 * p->dims),
                      pi * pi / (2.0 * p->W0 * p->W0), p->phi0};
     cudaStream_t st = (cudaStream_t)stream;
-    // one block per kNoAllocSitesPerBlock sites, striding over the rows along gridDim.y,
-    // whose limit (65535) is one below the 65536 partial slots: at the 2^30-site limit the
-    // blocks take a few more rows each
+    // one block per kNoAllocSitesPerBlock sites, below the 65536 partial slots: at the
+    // 2^30-site limit the blocks take a few more tiles each
     int64_t want = (S + kNoAllocSitesPerBlock - 1) / kNoAllocSitesPerBlock;
     const int grid = (int)(want < kMaxGridY ? want : kMaxGridY);
 

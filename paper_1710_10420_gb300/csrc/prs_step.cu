@@ -32,12 +32,10 @@ int max_fused_steps(const Geo& g, int precision, bool repro)
     return (g.dims == 3 ? t3_ok(g) : rows_ok(g)) ? 3 : 2;
 }
 
-// The library's default number of steps per pass (us per step, one / two / three steps per
-// pass).  FP32 3D: one below 2^24 sites, where a one-step pass cut into chunks of a few planes
-// occupies the GPU best (128^3 8.3 / 15.4 / 11.0, 256^2 x 128 18.1 / 21.6 / 20.5); from 2^24 two
-// wherever the two-step pass gets tiles of at least 4 rows (256^3 46.7 / 32.8 / 34.3; 1024^3
-// 2.53 / 1.37 / 1.43 ms).  FP32 2D: nominal; the register march has a plan of its own
-// (march_counts), as has FP32 3D without a tblock (march_counts_3d).  FP64 and other boxes: one.
+// The fixed number of steps per pass that suits a box, which prs_default_tblock reports.  A run without
+// a tblock is stepped by a plan of passes of several lengths instead (march_counts in 2D,
+// march_counts_3d), chosen by the time each length takes there.  What this decides still: how an
+// ensemble reports a box, and which 2D and 3D boxes take the packed arithmetic (march_packed).
 int default_fused_steps(const Geo& g, int precision, bool repro)
 {
     (void)repro;

@@ -1,5 +1,5 @@
 // prs_tmap.h -- TMA tensor maps of the FP32 3D fields and the tensor copy that reads them,
-// shared by the multi-step passes (prs_t2tma.cu, prs_t3tma.cu).
+// of the two-step pass (prs_t2tma.cu).
 //
 // A field is described to the TMA engine as a 3D array (x, y, z) of floats, x fastest, with
 // a box of bw x bh x 1 elements: one copy moves bh rows of bw columns of one plane.  The
