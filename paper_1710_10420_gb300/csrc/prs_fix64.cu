@@ -20,12 +20,13 @@
 // or more, and raised again when a plane needs it.  A warp that meets values at 2 phi0's S or beyond
 // (blow-ups) or not finite evaluates the double form.
 //
-// Measured (us a step; the double form): 256^3 163 (355), 512^3 1245 (2805), 128^3 29 (47), 2048^2 48
-// (74), 128^2 4.4 (4.2: the launch).  230 integer instructions a site at 0.6 of the issue slots now set
-// the pace.
+// Measured (us a step; the double form): 256^3 163 (355), 512^3 1245 (2805), 128^3 29 (47), 2048^2 39
+// (74), 128^2 4.2 (4.2: the launch).  230 integer instructions a site at 0.6
+// of the issue slots now set the pace.
 //
-// A warp owns 32 columns (30 outputs) of four rows (2D: one) and marches along z (2D: y): a value is
-// converted once where it enters, its z neighbours wait in registers, x neighbours come by shuffle.
+// A warp owns 32 columns (30 outputs) of four rows, in 2D 32 or 64 columns (one or two a lane) of one row,
+// and marches along z (2D: y): a value is converted once where it enters, its z neighbours wait in
+// registers, x neighbours come by shuffle.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -43,8 +44,10 @@ namespace {
 typedef long long i64;
 typedef unsigned long long u64;
 
-constexpr int kFxThreads = 128, kFxWarps = kFxThreads / 32, kFxU = 30;
-constexpr int fx_blocks(int dims) { return dims == 3 ? 4 : 8; }  // CTAs an SM (registers)
+constexpr int kFxThreads = 128, kFxWarps = kFxThreads / 32;
+// By dimensions and columns a lane (3D: 1): output columns of a warp, CTAs an SM (registers).
+constexpr int fx_width(int cols) { return 32 * cols - 2; }
+constexpr int fx_blocks(int dims, int cols) { return dims == 3 ? 4 : (cols == 1 ? 8 : 5); }
 
 // The force's constants: k1, k2 S^2 and g scaled by 2^(62-ek), 2^(66-ek), 2^(65-ek); e_base: what a
 // value's exponent field is subtracted from for its shift; e_out: exponent field of an A of 2^63.
@@ -115,35 +118,40 @@ __device__ __forceinline__ double force(i64 c, i64 s2, const Fix64& f, u64 k2, i
     return from_fixed(u + l, e_out);
 }
 
-template <int D>
-__global__ void __launch_bounds__(kFxThreads, fx_blocks(D)) k_step_fix64(const __grid_constant__ FixArgs a)
+template <int D, int C>
+__global__ void __launch_bounds__(kFxThreads, fx_blocks(D, C)) k_step_fix64(const __grid_constant__ FixArgs a)
 {
-    constexpr int R = D == 3 ? 4 : 1, N = D == 3 ? R + 2 : 1, H = D == 3 ? 1 : 0;  // output and stored rows; halo
+    // a lane's outputs (3D: rows, 2D: columns) and values, their halo, outputs of a warp across x
+    constexpr int R = D == 3 ? 4 : C, N = D == 3 ? R + 2 : R, H = D == 3 ? 1 : 0, U = fx_width(C);
     chain_enter();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nx = a.g.nx, ny = D == 3 ? a.g.ny : 1, nz = D == 3 ? a.g.nz : a.g.ny;
     int x0, y0, z0;
     if (D == 3) {
         int b = blockIdx.x;
-        x0 = b % a.nstrips * kFxU;
+        x0 = b % a.nstrips * U;
         b /= a.nstrips;
         y0 = (b % a.ygroups * kFxWarps + wid) * R;
         z0 = b / a.ygroups * a.cz;
         if (y0 >= ny) return;
     } else {
         const int w = blockIdx.x * kFxWarps + wid;
-        x0 = w % a.nstrips * kFxU;
+        x0 = w % a.nstrips * U;
         y0 = 0;
         z0 = w / a.nstrips * a.cz;
         if (z0 >= nz) return;
     }
-    const int planes = min(a.cz, nz - z0), rows = min(R, ny - y0);
-    int x = (x0 - 1 + lane) % nx;
+    const int planes = min(a.cz, nz - z0), rows = D == 3 ? min(R, ny - y0) : R;
+    int x = (x0 - 1 + C * lane) % nx;
     if (x < 0) x += nx;
-    const bool out = lane >= 1 && lane <= min(kFxU, nx - x0);
-    unsigned row[N];  // element offsets of the stored rows in a plane, periodic
+    const int first = C * lane - 1, last = min(U, nx - x0);  // the lane's first column of the strip's 0 .. last-1
+    unsigned row[N];  // element offsets of the lane's values in a plane, periodic
 #pragma unroll
     for (int r = 0; r < N; ++r) {
+        if (D == 2) {
+            row[r] = (unsigned)(x + r >= nx ? x + r - nx : x + r);
+            continue;
+        }
         int y = (y0 - H + r) % ny;
         if (y < 0) y += ny;
         row[r] = (unsigned)y * (unsigned)nx + (unsigned)x;
@@ -216,8 +224,9 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D)) k_step_fix64(const _
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     const i64 cc = c[r + H];
-                    i64 s2 = (__shfl_up_sync(0xffffffffu, cc, 1) + __shfl_down_sync(0xffffffffu, cc, 1)) +
-                             (m[r] + p[r + H]);
+                    const i64 left = D == 2 && r > 0 ? c[r - 1] : __shfl_up_sync(0xffffffffu, c[D == 2 ? R - 1 : r + H], 1);
+                    const i64 right = D == 2 && r < R - 1 ? c[r + 1] : __shfl_down_sync(0xffffffffu, c[D == 2 ? 0 : r + H], 1);
+                    i64 s2 = (left + right) + (m[r] + p[r + H]);
                     if (D == 3) s2 += c[r] + c[r + 2 * H];
                     v[r] = fma(a.k.c1, v[r], force(cc, s2, a.f, k2, a.f.e_out - down));
                     pn[r] = fma(a.deta, v[r], d[r]);
@@ -229,12 +238,12 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D)) k_step_fix64(const _
                 const double* qm = a.phi_in + (int64_t)zm * plane;
 #pragma unroll 1
                 for (int r = 0; r < rows; ++r) {
-                    const int y = y0 + r;
-                    const int64_t o = (int64_t)y * nx, up = (int64_t)(y + 1 == ny ? 0 : y + 1) * nx + x;
-                    const int64_t dn2 = (int64_t)(y == 0 ? ny - 1 : y - 1) * nx + x;
-                    const double xp = q[o + (x + 1 == nx ? 0 : x + 1)], xm = q[o + (x == 0 ? nx - 1 : x - 1)];
-                    const double cc = q[o + x], yp = D == 3 ? q[up] : qp[o + x], ym = D == 3 ? q[dn2] : qm[o + x];
-                    const double zpv = D == 3 ? qp[o + x] : 0.0, zmv = D == 3 ? qm[o + x] : 0.0;
+                    const int y = D == 3 ? y0 + r : 0, x1 = D == 3 ? x : (x + r >= nx ? x + r - nx : x + r);
+                    const int64_t o = (int64_t)y * nx, up = (int64_t)(y + 1 == ny ? 0 : y + 1) * nx + x1;
+                    const int64_t dn2 = (int64_t)(y == 0 ? ny - 1 : y - 1) * nx + x1;
+                    const double xp = q[o + (x1 + 1 == nx ? 0 : x1 + 1)], xm = q[o + (x1 == 0 ? nx - 1 : x1 - 1)];
+                    const double cc = q[o + x1], yp = D == 3 ? q[up] : qp[o + x1], ym = D == 3 ? q[dn2] : qm[o + x1];
+                    const double zpv = D == 3 ? qp[o + x1] : 0.0, zmv = D == 3 ? qm[o + x1] : 0.0;
                     double vv, pp;
 #pragma unroll
                     for (int u = 0; u < R; ++u) vv = u == r ? v[u] : vv;
@@ -246,7 +255,7 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D)) k_step_fix64(const _
             }
 #pragma unroll
             for (int r = 0; r < R; ++r)
-                if (out && r < rows) {
+                if (first + (D == 2 ? r : 0) >= 0 && first + (D == 2 ? r : 0) < last && r < rows) {
                     pout[row[r + H]] = pn[r];
                     vout[row[r + H]] = v[r];
                 }
@@ -297,13 +306,16 @@ cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const
     a.k = k;
     a.deta = deta;
     a.g = g;
-    a.nstrips = (g.nx + kFxU - 1) / kFxU;
+    // 2D: two columns a lane share a row's bookkeeping, one makes twice the warps (us a step, two and one:
+    // 256^2 4.0 3.4, 400^2 4.6 4.3, 512^2 5.2 5.5, 1024^2 11.9 13.2, 2048^2 39 44)
+    const int cols = g.dims == 3 || g.S < ((int64_t)1 << 18) ? 1 : 2, width = fx_width(cols);
+    a.nstrips = (g.nx + width - 1) / width;
     const int len = g.dims == 3 ? g.nz : g.ny;
     a.ygroups = g.dims == 3 ? (g.ny + 4 * kFxWarps - 1) / (4 * kFxWarps) : 1;
     // warps (2D) or blocks of them (3D) against the two planes a chunk re-reads and the iteration
     // that fills it
     const double tiles = (double)a.nstrips * a.ygroups / (g.dims == 3 ? 1 : kFxWarps);
-    const double slots = (double)fx_blocks(g.dims) * sm_count_current();
+    const double slots = (double)fx_blocks(g.dims, cols) * sm_count_current();
     double least = 1e300;
     a.cz = len;
     for (int nc = 1; nc <= len && nc <= 4096; nc += nc < 32 ? 1 : nc / 16) {
@@ -316,7 +328,8 @@ cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const
     const int64_t blocks = g.dims == 3 ? (int64_t)a.nstrips * a.ygroups * n
                                        : ((int64_t)a.nstrips * n + kFxWarps - 1) / kFxWarps;
     if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
-    return launch_chained(g.dims == 3 ? k_step_fix64<3> : k_step_fix64<2>, dim3((unsigned)blocks), kFxThreads, 0, st, a);
+    void (*kernel)(const FixArgs) = g.dims == 3 ? k_step_fix64<3, 1> : (cols == 1 ? k_step_fix64<2, 1> : k_step_fix64<2, 2>);
+    return launch_chained(kernel, dim3((unsigned)blocks), kFxThreads, 0, st, a);
 }
 
 }  // namespace prs

@@ -16,8 +16,8 @@ import paper_1710_10420_gb300 as prs
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [(3, 3), (29, 5), (30, 7), (31, 40), (61, 33), (128, 130), (3, 3, 3), (30, 16, 4), (31, 17, 5), (59, 15, 9),
-          (90, 33, 3), (64, 20, 21)]
+SHAPES = [(3, 3), (29, 5), (30, 7), (31, 40), (61, 33), (128, 130), (4030, 66), (4031, 66), (4097, 64), (5, 52429),
+          (3, 3, 3), (30, 16, 4), (31, 17, 5), (59, 15, 9), (90, 33, 3), (64, 20, 21)]
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -70,7 +70,7 @@ def test_one_step_against_the_oracle(shape, phi0, dx, kind):
     assert np.array_equal(na, -a) and np.array_equal(nb, -b)
 
 
-@pytest.mark.parametrize("shape", [(61, 33), (31, 17, 5)])
+@pytest.mark.parametrize("shape", [(61, 33), (517, 509), (31, 17, 5)])
 def test_a_non_finite_value_reaches_its_neighbours_only(shape):
     phi, v = _field(shape, "full", 1.0)
     phi.reshape(-1)[phi.size // 2] = math.inf
