@@ -102,7 +102,7 @@ typedef struct {
     uint64_t seed;     /* seed of the random initial field (prs_init with NULL)     */
     uint32_t flags;    /* PRS_REPRO | PRS_FP32_CR | PRS_DEBUG, or 0                 */
     int32_t tblock;    /* leapfrog steps per pass over HBM: 0 = library's choice (FP32: a
-                          mix of passes of 1 to 3 steps in 3D and 1 to 5 in 2D, whichever
+                          mix of passes of 1 to 3 steps in 3D and 1 to 6 in 2D, whichever
                           takes least time on this machine; FP64: 1); 1 = one step per pass;
                           2 = two-step passes for FP32 boxes with
                           an x side that is a multiple of 128 (3D; z side >= 3) or a

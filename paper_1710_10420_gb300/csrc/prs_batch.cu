@@ -3,7 +3,7 @@
 // The paper motivates large sets of production runs (Sec. I, Sec. IV: calibrating the one-scale model
 // needs many realisations); it runs them one at a time.  A small box leaves most of the GPU idle, and
 // its passes cost little more than their launches.  Here the runs of one box are stepped together, up to
-// 16 to a launch: each of their passes (the register marches, five steps a pass in 2D and three in 3D)
+// 16 to a launch: each of their passes (the register marches, up to six steps a pass in 2D and three in 3D)
 // and each output's diagnostics is one launch over all of them, its shape chosen for the group.  Groups
 // are independent, so each runs on a stream of its own between a fork and a join on the ensemble's
 // stream, and the latencies of one group's passes hide behind another's.
