@@ -17,7 +17,9 @@
 //
 // The integers hold their precision absolutely, doubles relatively.  So each warp scales by an S of its
 // own, S 2^-down: it is lowered when the three planes of an iteration hold no value of a sixteenth of it
-// or more, and raised again when a plane needs it.  A warp that meets values at 2 phi0's S or beyond
+// or more, and raised again when a plane needs it.  The planes already held are then converted again
+// from memory: an integer carried to a smaller S keeps the absolute error of the larger one, and one
+// rounded up to its S 2 no longer fits the products.  A warp that meets values at 2 phi0's S or beyond
 // (blow-ups) or not finite evaluates the double form.
 //
 // Measured (us a step; the double form): 256^3 163 (355), 512^3 1245 (2805), 128^3 29 (47), 2048^2 39
@@ -84,14 +86,6 @@ __device__ __forceinline__ i64 to_fixed(double d, int e_base, int& shift)
 
 // a times sign (0 or -1): its negation where sign is -1.
 __device__ __forceinline__ i64 with_sign(u64 a, i64 sign) { return (i64)(a ^ (u64)sign) - sign; }
-
-// a times 2^by, towards zero.
-__device__ __forceinline__ i64 rescaled(i64 a, int by)
-{
-    const i64 s = a >> 63;
-    const u64 m = (u64)with_sign((u64)a, s);
-    return with_sign(by >= 0 ? (by > 63 ? 0ull : m << by) : (by < -63 ? 0ull : m >> -by), s);
-}
 
 __device__ __forceinline__ double from_fixed(i64 a, int e_out)
 {
@@ -193,19 +187,26 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D, C)) k_step_fix64(cons
         }
         sp = __reduce_min_sync(0xffffffffu, sp);
         const int least = min(min(sm, sc), sp);  // the shift of the largest value
-        if ((least < 3 || least > 7) && least < 1100) {  // (planes of zeros keep the scale)
+        if ((least < 3 || least > 7) && least < 1100) {
             const int by = max(min(least - 3, most - down), -down);
-            if (by != 0) {
+            if (by != 0) {  // (planes of zeros lower the scale to its limit)
                 down += by;
                 k2 = down > 31 ? 0ull : a.f.k2 >> 2 * down;
                 sm -= by, sc -= by, sp -= by;
+                // planes z0 + i - 1 and z0 + i - 2, periodic (the first two iterations hold none there yet)
+                const int zc = z0 + i - 1 < 0 ? nz - 1 : z0 + i - 1, zm = zc == 0 ? nz - 1 : zc - 1;
+                const double* qc = a.phi_in + (int64_t)zc * plane;
+                const double* qm = a.phi_in + (int64_t)zm * plane;
+                int s;
 #pragma unroll
-                for (int r = 0; r < R; ++r) m[r] = rescaled(m[r], by);
+                for (int r = 0; r < N; ++r) p[r] = to_fixed(next[r], a.f.e_base - down, s);
+                if (i >= 0) {
 #pragma unroll
-                for (int r = 0; r < N; ++r) {
-                    int s;
-                    c[r] = rescaled(c[r], by);
-                    p[r] = to_fixed(next[r], a.f.e_base - down, s);
+                    for (int r = 0; r < N; ++r) c[r] = to_fixed(qc[row[r]], a.f.e_base - down, s);
+                }
+                if (i >= 1) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) m[r] = to_fixed(qm[row[r + H]], a.f.e_base - down, s);
                 }
             }
         }
