@@ -49,7 +49,11 @@ extern "C" {
 
 /* ---------------------------------------------------------------- precision */
 #define PRS_FP32 0 /* float storage and arithmetic; FP64 diagnostic sums           */
-#define PRS_FP64 1 /* double storage and arithmetic                                 */
+/* double storage; without PRS_REPRO the force of a step is evaluated in 64-bit fixed point wherever a
+ * site or one of its neighbours is large enough, beside the values around it, for that to be at least as
+ * accurate as doubles, else in doubles.  Which it is depends on the site's place among its neighbours in the
+ * box, so a field moved along the lattice gives the moved result to rounding, not bit for bit. */
+#define PRS_FP64 1
 
 /* ---------------------------------------------------------------- flags */
 /* FP64 only: evaluate each site in the canonical order with no fused multiply-add,

@@ -8,23 +8,26 @@
 // double operations (one fused multiply-add each).
 //
 // With S the power of two at or above phi0, a value |phi| < 2 S becomes the integer phi/S 2^59,
-// whose neighbour sum is exact; three high-half products evaluate the cubic and one the
-// neighbour term, with the constants scaled so that A, times 2^(60 - ek) / S, fits 63 bits (ek: the
-// exponent that bounds the constants); A is then rounded to double once.  Its error is a few 2^-60 of
-// S 2^ek, where the double evaluation rounds each of its terms (6 g phi and its like) to 2^-54: the
-// step's error against 64-bit references is not larger (tests/test_gpu_fix64.py).  Products take the
-// magnitudes, so the step of a negated field is the negated step, bit for bit.
+// whose neighbour sum is exact; high-half products evaluate k1 - k2 phi^2, and its product with phi and
+// the neighbour term, whose constants are scaled alike (2^(60-ek) / S; ek: the exponent that bounds the
+// constants), are added in 128 bits.  A is rounded to 2^(ek-61) S, then to double.  Products are whole or
+// of magnitudes, so the step of a negated field is the negated step, bit for bit.
 //
-// The integers hold their precision absolutely, doubles relatively.  So each warp scales by an S of its
-// own, S 2^-down: it is lowered when the three planes of an iteration hold no value of a sixteenth of it
-// or more, and raised again when a plane needs it.  The planes already held are then converted again
-// from memory: an integer carried to a smaller S keeps the absolute error of the larger one, and one
-// rounded up to its S 2 no longer fits the products.  A warp that meets values at 2 phi0's S or beyond
-// (blow-ups) or not finite evaluates the double form.
+// The integers hold their precision absolutely, doubles relatively: a value of S/128 or more converts
+// exactly, a smaller one to 2^-60 S.  So the integers serve a site only where it or one of its neighbours
+// is at least S/16, larger where the neighbours' constant g is below 2^ek/32 (wide lattices, strong
+// potentials; make_fix64): over random stencils whose largest value lies between that and twice that, with
+// W0 from 1.2 to infinity and dx from 0.5 to 10, the force's rms error is 0.02 to 0.79 of the double form's,
+// and at most 0.85 where one neighbour holds that value and all the others are 1e-6 of it.  A warp takes the
+// integers where they serve all its sites and no value is at 2 S or beyond (blow-ups) or not finite; else
+// it evaluates the double form.  So that this holds for fields of any size, each warp scales by an S of its
+// own, S 2^-down: it is lowered when the three planes of an iteration hold no value of a quarter of it or
+// more, and raised again when a plane needs it; the planes already held are then converted again.
 //
-// Measured (us a step; the double form): 256^3 163 (355), 512^3 1245 (2805), 128^3 29 (47), 2048^2 39
-// (74), 128^2 4.2 (4.2: the launch).  230 integer instructions a site at 0.6
-// of the issue slots now set the pace.
+// Measured (us a step of a network of walls ten sites wide; the double form): 256^3 194 (356), 512^3 1476
+// (2805), 128^3 32 (52), 2048^2 44 (74), 128^2 3.4 (4.3: the launch).  Wide walls have more sites without a
+// large neighbour: 40 sites wide, 256^3 takes 277.  Before the precision of small values was kept (128-bit
+// sums, the vote): 161 at 256^3, 39 at 2048^2.
 //
 // A warp owns 32 columns (30 outputs) of four rows, in 2D 32 or 64 columns (one or two a lane) of one row,
 // and marches along z (2D: y): a value is converted once where it enters, its z neighbours wait in
@@ -52,11 +55,12 @@ constexpr int fx_width(int cols) { return 32 * cols - 2; }
 constexpr int fx_blocks(int dims, int cols) { return dims == 3 ? 4 : (cols == 1 ? 8 : 5); }
 
 // The force's constants: k1, k2 S^2 and g scaled by 2^(62-ek), 2^(66-ek), 2^(65-ek); e_base: what a
-// value's exponent field is subtracted from for its shift; e_out: exponent field of an A of 2^63.
+// value's exponent field is subtracted from for its shift; e_out: exponent field of an A of 2^63; served:
+// the shift of the smallest values that serve their site and its neighbours (2: none do).
 struct Fix64 {
     i64 k1;
     u64 k2, g;
-    int e_base, e_out;
+    int e_base, e_out, served;
 };
 
 struct FixArgs {
@@ -87,29 +91,23 @@ __device__ __forceinline__ i64 to_fixed(double d, int e_base, int& shift)
 // a times sign (0 or -1): its negation where sign is -1.
 __device__ __forceinline__ i64 with_sign(u64 a, i64 sign) { return (i64)(a ^ (u64)sign) - sign; }
 
-__device__ __forceinline__ double from_fixed(i64 a, int e_out)
-{
-    const i64 s = a >> 63;
-    const u64 m = (u64)with_sign((u64)a, s);
-    const int lz = __clzll((i64)m);
-    const u64 n = m << (lz & 63);
-    // 53 bits and the next as rounding, added onto the exponent: a carry bumps it
-    const u64 bits = (n >> 11) + ((n >> 10) & 1ull) + ((u64)(unsigned)(e_out - lz - 1) << 52);
-    const double r = __longlong_as_double((i64)(bits | ((u64)s & 0x8000000000000000ull)));
-    return m ? r : 0.0;
-}
-
 // A of one site: c its value, s2 the sum of its neighbours.
 // k2, e_out: f's for the warp's scale.
 __device__ __forceinline__ double force(i64 c, i64 s2, const Fix64& f, u64 k2, int e_out)
 {
-    const i64 sc = c >> 63, ss = s2 >> 63;
-    const u64 b = (u64)with_sign((u64)c, sc) << 3;              // |x| 2^62
+    const i64 x = c << 3;                                       // x 2^62
+    const u64 b = (u64)with_sign((u64)x, x >> 63);
     const u64 t = __umul64hi(b, b);                             // x^2 2^60
     const i64 k = f.k1 - (i64)__umul64hi(t, k2);                // (k1 - k2 phi^2) 2^(62-ek)
-    const i64 u = with_sign((u64)__mul64hi((i64)b, k), sc);     // x (k1 - k2 phi^2) 2^(60-ek)
-    const i64 l = with_sign(__umul64hi((u64)with_sign((u64)s2, ss), f.g), ss);
-    return from_fixed(u + l, e_out);
+    const __int128 a = (__int128)x * k + (__int128)s2 * (i64)f.g;  // A 2^(124-ek), below 2^126
+    const i64 sa = (i64)(a >> 64) >> 63;
+    const unsigned __int128 w = (unsigned __int128)(sa ? -a : a);
+    const u64 m = ((u64)(w >> 62) + 1) >> 1;                    // |A| 2^(61-ek)
+    const int lz = __clzll((i64)m);
+    const u64 n = m << (lz & 63);
+    // 53 bits and the next as rounding, added onto the exponent: a carry bumps it
+    const u64 bits = (n >> 11) + ((n >> 10) & 1ull) + ((u64)(unsigned)(e_out - lz - 2) << 52);
+    return m ? __longlong_as_double((i64)(bits | ((u64)sa & 0x8000000000000000ull))) : 0.0;
 }
 
 template <int D, int C>
@@ -168,6 +166,11 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D, C)) k_step_fix64(cons
     i64 m[R], c[N], p[N];
     double d[R], v[R];
     int sm = 4096, sc = 4096, sp, down = 0;
+    // bit r: output r; value r of planes z-1 and z serves its site; one of plane z next to value r or it does
+    unsigned outputs = 0, bm = 0, bc = 0, wc = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (first + (D == 2 ? r : 0) >= 0 && first + (D == 2 ? r : 0) < last && r < rows) outputs |= 1u << (r + H);
     const int most = a.f.e_out - 192;  // exponents of A stay in range
     u64 k2 = a.f.k2;
     fetch();
@@ -175,51 +178,50 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D, C)) k_step_fix64(cons
     for (int r = 0; r < R; ++r) m[r] = 0, vnext[r] = 0.0, d[r] = 0.0;
 #pragma unroll
     for (int r = 0; r < N; ++r) c[r] = 0;
-    for (int i = -1; i <= planes; ++i) {  // plane z0 + i arrives, plane z0 + i - 1 is updated
+    // Plane z0 + i arrives, plane z0 + i - 1 is updated.  A warp that changes its scale goes back to the
+    // planes it holds (those before `live` have been updated).
+    for (int i = -1, live = -1; i <= planes; ++i) {
         sp = 4096;
         double dn[R];
+        unsigned bp = 0;  // bit r: value r serves its site and its neighbours
 #pragma unroll
         for (int r = 0; r < N; ++r) {
             int s;
             p[r] = to_fixed(next[r], a.f.e_base - down, s);
+            if (s <= a.f.served) bp |= 1u << r;
             sp = min(sp, s);
             if (r >= H && r < R + H) dn[r - H] = next[r];
         }
+        const bool served = __all_sync(0xffffffffu, ((wc | bm | bp) & outputs) == outputs);
         sp = __reduce_min_sync(0xffffffffu, sp);
         const int least = min(min(sm, sc), sp);  // the shift of the largest value
-        if ((least < 3 || least > 7) && least < 1100) {
+        if ((least < 3 || least > 5) && least < 1100 && i >= live) {
             const int by = max(min(least - 3, most - down), -down);
             if (by != 0) {  // (planes of zeros lower the scale to its limit)
                 down += by;
                 k2 = down > 31 ? 0ull : a.f.k2 >> 2 * down;
-                sm -= by, sc -= by, sp -= by;
-                // planes z0 + i - 1 and z0 + i - 2, periodic (the first two iterations hold none there yet)
-                const int zc = z0 + i - 1 < 0 ? nz - 1 : z0 + i - 1, zm = zc == 0 ? nz - 1 : zc - 1;
-                const double* qc = a.phi_in + (int64_t)zc * plane;
-                const double* qm = a.phi_in + (int64_t)zm * plane;
-                int s;
-#pragma unroll
-                for (int r = 0; r < N; ++r) p[r] = to_fixed(next[r], a.f.e_base - down, s);
-                if (i >= 0) {
-#pragma unroll
-                    for (int r = 0; r < N; ++r) c[r] = to_fixed(qc[row[r]], a.f.e_base - down, s);
-                }
-                if (i >= 1) {
-#pragma unroll
-                    for (int r = 0; r < R; ++r) m[r] = to_fixed(qm[row[r + H]], a.f.e_base - down, s);
-                }
+                sm = sc = 4096;
+                live = i;
+                i = i < 1 ? -1 : i - 2;
+                z = z0 + i < 0 ? nz - 1 : z0 + i;
+                pin = a.phi_in + (int64_t)z * plane;
+                fetch();
+                --i;
+                continue;
             }
         }
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = vnext[r];
         if (i < planes) fetch();
-        if (i >= 0 && i < planes) {
+        if (i >= live) {
 #pragma unroll
-            for (int r = 0; r < R; ++r) vnext[r] = r < rows ? vin[row[r + H]] : 0.0;
-            vin += plane;
+            for (int r = 0; r < R; ++r) v[r] = vnext[r];
+            if (i >= 0 && i < planes) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) vnext[r] = r < rows ? vin[row[r + H]] : 0.0;
+                vin += plane;
+            }
         }
-        if (i >= 1) {
-            const bool fixed = min(min(sm, sc), sp) >= 3;
+        if (i >= 1 && i >= live) {
+            const bool fixed = min(min(sm, sc), sp) >= 3 && served;
             double pn[R];
             if (fixed) {
 #pragma unroll
@@ -256,15 +258,17 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D, C)) k_step_fix64(cons
             }
 #pragma unroll
             for (int r = 0; r < R; ++r)
-                if (first + (D == 2 ? r : 0) >= 0 && first + (D == 2 ? r : 0) < last && r < rows) {
+                if (outputs >> (r + H) & 1u) {
                     pout[row[r + H]] = pn[r];
                     vout[row[r + H]] = v[r];
                 }
             pout += plane;
             vout += plane;
         }
-        sm = sc;
-        sc = sp;
+        sm = sc, sc = sp;
+        const unsigned bl = __shfl_up_sync(0xffffffffu, bp, 1), br = __shfl_down_sync(0xffffffffu, bp, 1);
+        wc = bp | bp << 1 | bp >> 1 | (D == 3 ? bl | br : bl >> (R - 1) | br << (R - 1));
+        bm = bc, bc = bp;
 #pragma unroll
         for (int r = 0; r < R; ++r) m[r] = c[r + H], d[r] = dn[r];
 #pragma unroll
@@ -291,6 +295,8 @@ static bool make_fix64(const KickD& k, double phi0, Fix64* f)
     f->g = (u64)llrint(ldexp(k.g, 65 - ek));
     f->e_base = 1026 + es;
     f->e_out = 1023 + 63 + ek - 60 + es;
+    f->served = 7;
+    for (double least = ldexp(1.0, ek - 5); k.g < least && f->served > 2; least *= 0.5) --f->served;
     return true;
 }
 

@@ -50,7 +50,7 @@ def _check(shape, phi, v, **kw):
 
 
 # values just below a power of two round up to it in fewer bits
-DROPS = [np.nextafter(2.0 ** -10, 0.0), 2.0 ** -40 * (1.0 - 2.0 ** -30), 3e-7, 1e-30]
+DROPS = [np.nextafter(2.0 ** -10, 0.0), 2.0 ** -40 * (1.0 - 2.0 ** -30), 3e-7, 1e-30, 1e-290]
 
 
 @pytest.mark.parametrize("drop", DROPS)
@@ -64,3 +64,39 @@ def test_planes_behind_a_drop_in_size(shape, drop):
     sign = np.where(np.arange(n) % 5 == 0, -1.0, 1.0)
     phi *= sign.reshape([-1] + [1] * (phi.ndim - 1))
     _check(shape, phi, np.zeros_like(phi))
+
+
+def _smooth_noise(rng, fshape, amplitude):
+    phi = rng.uniform(-1.0, 1.0, fshape)
+    for axis in range(phi.ndim):
+        phi = phi + np.roll(phi, 1, axis) + np.roll(phi, -1, axis)
+    return amplitude * phi / np.max(np.abs(phi))
+
+
+def _varied(kind, fshape):
+    rng = np.random.Generator(np.random.PCG64(sum(fshape) * 10 + len(fshape)))
+    at = np.meshgrid(*[np.arange(n) - n // 3 for n in fshape], indexing="ij")
+    r2 = sum(x.astype(np.float64) ** 2 for x in at)
+    if kind == "bump":  # a localised perturbation of the symmetric state
+        return 0.7 * np.exp(-r2 / 8.0) + _smooth_noise(rng, fshape, 1e-9)
+    if kind == "bump on zeros":
+        return 0.7 * np.exp(-r2 / 8.0) * (r2 < 60.0)
+    if kind == "columns":  # every power of two in the columns of one warp
+        return 1.2 * 2.0 ** -(np.abs(at[-1]) % 50).astype(np.float64) * rng.choice([-1.0, 1.0], fshape)
+    if kind == "blocks":  # sizes that change from block to block, along every axis
+        exps = rng.uniform(-14.0, 0.0, [n // 7 + 1 for n in fshape])
+        for axis, n in enumerate(fshape):
+            exps = np.repeat(exps, 7, axis).take(range(n), axis)
+        return 10.0 ** exps * rng.uniform(-1.0, 1.0, fshape)
+    walls = np.tanh(np.sin(2.0 * np.pi * at[0] / fshape[0]) + 0.7 * np.sin(2.0 * np.pi * at[-1] / fshape[-1]))
+    return walls * 1e-6 if kind == "linear growth" else walls
+
+
+@pytest.mark.parametrize("kind", ["bump", "bump on zeros", "columns", "blocks", "walls", "linear growth"])
+@pytest.mark.parametrize("phi0,dx", [(1.0, 1.0), (1.3, 0.7), (1.0, 6.0)])
+@pytest.mark.parametrize("shape", [(64, 60), (700, 400), (31, 17, 20), (64, 33, 40)])
+def test_small_values_beside_large_ones(shape, phi0, dx, kind):
+    fshape = tuple(reversed(shape))
+    rng = np.random.Generator(np.random.PCG64(7))
+    phi = phi0 * _varied(kind, fshape)
+    _check(shape, phi, 1e-3 * phi * rng.standard_normal(fshape), phi0=phi0, dx=dx, W0=7.0)
