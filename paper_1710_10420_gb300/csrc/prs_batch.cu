@@ -249,16 +249,27 @@ extern "C" int prs_batch_run(prs_batch* b, const int64_t* nsteps_per_run, int64_
     return PRS_OK;
 }
 
+// A run's copies are queued on its group's stream: behind what the caller queued on the ensemble's (which
+// may still fill or read the host arrays).
+static int follow_caller(prs_batch* b, int run)
+{
+    cudaError_t e = cudaEventRecord(b->fork, b->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->sims[run]->stream, b->fork, 0);
+    return batch_cuda(e, "ensemble state");
+}
+
 extern "C" int prs_batch_get_state(prs_batch* b, int run, void* h_phi, void* h_dphi, int64_t* n)
 {
     if (!b || run < 0 || run >= (int)b->sims.size()) return PRS_EINVAL;
-    return prs_get_state(b->sims[run], h_phi, h_dphi, n);
+    const int rc = follow_caller(b, run);
+    return rc ? rc : prs_get_state(b->sims[run], h_phi, h_dphi, n);
 }
 
 extern "C" int prs_batch_set_state(prs_batch* b, int run, const void* h_phi, const void* h_dphi, int64_t n)
 {
     if (!b || run < 0 || run >= (int)b->sims.size() || !h_phi || !h_dphi || n < 0) return PRS_EINVAL;
-    return prs_set_state(b->sims[run], h_phi, h_dphi, n);
+    const int rc = follow_caller(b, run);
+    return rc ? rc : prs_set_state(b->sims[run], h_phi, h_dphi, n);
 }
 
 extern "C" int prs_batch_tuning(prs_batch* b, int run, int* tile_len, double* group_bytes)

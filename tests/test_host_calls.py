@@ -1,0 +1,84 @@
+"""What the library's host code asks of the CUDA runtime, on a runtime that is not there (tests/fake_cudart.cpp):
+the order of work between streams, what is left behind by a call that fails, and how often memory is
+allocated.  The library's own object files are linked with it; no kernel runs."""
+import ctypes
+import glob
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import paper_1710_10420_gb300 as prs
+from paper_1710_10420_gb300 import _build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    _build.build()
+    objs = [os.path.join(_build.OBJDIR, os.path.basename(s) + ".o") for s in _build.sources()]
+    if not all(os.path.exists(o) for o in objs):
+        _build.build(force=True)
+    cuda = os.path.join(os.path.dirname(os.path.dirname(_build.nvcc())), "include")
+    out = str(tmp_path_factory.mktemp("fake") / "libprs_fake.so")
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", cuda,
+                    os.path.join(HERE, "fake_cudart.cpp"), *objs, "-o", out], check=True)
+    fake = ctypes.CDLL(out)
+    for name, (res, args) in prs._SIGS.items():
+        fn = getattr(fake, name)
+        fn.restype, fn.argtypes = res, args
+    fake.fake_log.restype = ctypes.c_char_p
+    fake.fake_fail.argtypes = [ctypes.c_char_p, ctypes.c_int, ctypes.c_int]
+    fake.fake_limit.argtypes = [ctypes.c_size_t]
+    return fake
+
+
+@pytest.fixture(autouse=True)
+def _clean(lib):
+    lib.fake_reset()
+
+
+def _log(lib):
+    return [line.split() for line in lib.fake_log().decode().splitlines()]
+
+
+def _batch(lib, runs, stream):
+    arr = (prs.prs_params * len(runs))(*runs)
+    b = ctypes.c_void_p()
+    assert lib.prs_batch_create(arr, len(runs), stream, ctypes.byref(b)) == prs.PRS_OK
+    lib.fake_reset()
+    return b
+
+
+STREAM = 77  # the caller's
+
+
+def _ordered(log, first, second):
+    """Whether work on stream `second` at the end of the log comes after all work on stream `first`."""
+    if first == second:
+        return True
+    events = {line[2] for line in log if line[0] == "record" and line[1] == first}
+    return any(line[0] == "wait" and line[1] == second and line[2] in events for line in log)
+
+
+@pytest.mark.parametrize("write", [True, False])
+def test_ensemble_state_copies_follow_the_callers_stream(lib, write):
+    """The copies of prs_batch_set_state and prs_batch_get_state come after what the caller queued on the
+    stream given to prs_batch_create (the fill of a pinned buffer, a kernel that reads one)."""
+    b = _batch(lib, [prs.make_params((128, 128)), prs.make_params((256, 64))], STREAM)
+    for run, shape in ((0, (128, 128)), (1, (64, 256))):
+        phi, v = np.zeros(shape, np.float32), np.zeros(shape, np.float32)
+        lib.fake_reset()
+        if write:
+            assert lib.prs_batch_set_state(b, run, phi.ctypes.data, v.ctypes.data, 3) == prs.PRS_OK
+        else:
+            assert lib.prs_batch_get_state(b, run, phi.ctypes.data, v.ctypes.data, None) == prs.PRS_OK
+        log = _log(lib)
+        copies = [i for i, line in enumerate(log) if line[0] == "copy"]
+        assert len(copies) == 2
+        for i in copies:
+            assert _ordered(log[:i], str(STREAM), log[i][1]), log
+        assert any(line[0] == "sync" and line[1] == log[copies[-1]][1] for line in log[copies[-1]:])
+    assert lib.prs_batch_destroy(b) == prs.PRS_OK
