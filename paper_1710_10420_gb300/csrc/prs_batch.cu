@@ -184,6 +184,29 @@ static int group_queue(prs_batch* b, const Group& q, const int64_t* nsteps, int6
     }
 }
 
+// Queue a call's work, each group on its stream between a fork and a join on the ensemble's, and wait for
+// its results.
+static int run_queue(prs_batch* b, const int64_t* nsteps, int64_t every, const size_t* slot, std::vector<DiagAcc>& res)
+{
+    cudaError_t e = cudaEventRecord(b->fork, b->stream);
+    for (Group& q : b->groups) {
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(q.stream, b->fork, 0);
+        if (e != cudaSuccess) return batch_cuda(e, "prs_batch_run");
+        const int rc = group_queue(b, q, nsteps, every, slot);
+        if (rc) return rc;
+        for (int r : q.runs)  // the error words of the runs' bounded waits
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(&b->sims[r]->h_status->error, &b->sims[r]->d_status->error, sizeof(unsigned),
+                                    cudaMemcpyDeviceToHost, q.stream);
+        if (e == cudaSuccess) e = cudaEventRecord(q.done, q.stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, q.done, 0);
+    }
+    if (e == cudaSuccess && !res.empty())
+        e = cudaMemcpyAsync(res.data(), b->results, res.size() * sizeof(DiagAcc), cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    return batch_cuda(e, "prs_batch_run");
+}
+
 extern "C" int prs_batch_run(prs_batch* b, const int64_t* nsteps_per_run, int64_t measure_every, double* out_series,
                              int64_t out_capacity)
 {
@@ -213,25 +236,14 @@ extern "C" int prs_batch_run(prs_batch* b, const int64_t* nsteps_per_run, int64_
         }
         b->result_slots = slots;
     }
-    if ((rc = batch_cuda(cudaEventRecord(b->fork, b->stream), "prs_batch_run"))) return rc;
-    int failed = PRS_OK;
-    for (Group& q : b->groups) {
-        if ((rc = batch_cuda(cudaStreamWaitEvent(q.stream, b->fork, 0), "prs_batch_run"))) return rc;
-        if (!failed) failed = group_queue(b, q, nsteps_per_run, measure_every, slot.data());
-        for (int r : q.runs)  // the error words of the runs' bounded waits
-            if ((rc = batch_cuda(cudaMemcpyAsync(&b->sims[r]->h_status->error, &b->sims[r]->d_status->error,
-                                                 sizeof(unsigned), cudaMemcpyDeviceToHost, q.stream),
-                                 "prs_batch_run")))
-                return rc;
-        if ((rc = batch_cuda(cudaEventRecord(q.done, q.stream), "prs_batch_run"))) return rc;
-        if ((rc = batch_cuda(cudaStreamWaitEvent(b->stream, q.done, 0), "prs_batch_run"))) return rc;
-    }
     std::vector<DiagAcc> res(slots);
-    if (slots && (rc = batch_cuda(cudaMemcpyAsync(res.data(), b->results, slots * sizeof(DiagAcc),
-                                                  cudaMemcpyDeviceToHost, b->stream), "prs_batch_run")))
+    if ((rc = run_queue(b, nsteps_per_run, measure_every, slot.data(), res))) {
+        // groups may be forked and not joined: nothing stays in flight behind an error
+        for (Group& q : b->groups) cudaStreamSynchronize(q.stream);
+        cudaStreamSynchronize(b->stream);
+        cudaGetLastError();
         return rc;
-    if ((rc = batch_cuda(cudaStreamSynchronize(b->stream), "prs_batch_run"))) return rc;
-    if (failed) return failed;
+    }
     for (prs_sim* s : b->sims)
         if ((rc = check_device_error(s))) return rc;
     for (int r = 0; r < R; ++r) {

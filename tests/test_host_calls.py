@@ -82,3 +82,23 @@ def test_ensemble_state_copies_follow_the_callers_stream(lib, write):
             assert _ordered(log[:i], str(STREAM), log[i][1]), log
         assert any(line[0] == "sync" and line[1] == log[copies[-1]][1] for line in log[copies[-1]:])
     assert lib.prs_batch_destroy(b) == prs.PRS_OK
+
+
+@pytest.mark.parametrize("call,nth", [("record", 1), ("wait", 1), ("wait", 2), ("wait", 3), ("launch", 2), ("launch", 5),
+                                      ("copy", 1), ("copy", 2), ("copy", 3), ("record", 2), ("record", 3), ("sync", 1)])
+def test_nothing_is_in_flight_behind_an_ensemble_error(lib, call, nth):
+    """When a CUDA call fails in the middle of prs_batch_run, every stream that was given work is waited
+    for before the error is returned (the caller may free its memory, and the groups are not joined)."""
+    b = _batch(lib, [prs.make_params((128, 128)), prs.make_params((256, 64))], STREAM)
+    ns = (ctypes.c_int64 * 2)(12, 12)
+    out = np.zeros((2, 4, 4))
+    lib.fake_fail(call.encode(), nth, 719)
+    assert lib.prs_batch_run(b, ns, 4, out.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), 4) == prs.PRS_ECUDA
+    log = _log(lib)
+    at = log.index(["FAIL", call])
+    for stream in {line[1] for line in log[:at] if line[0] in ("launch", "copy", "memset")}:
+        assert ["sync", stream] in log[at:], stream
+    assert not np.any(out)
+    lib.fake_reset()
+    assert lib.prs_batch_run(b, ns, 4, out.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), 4) == prs.PRS_OK
+    assert lib.prs_batch_destroy(b) == prs.PRS_OK
