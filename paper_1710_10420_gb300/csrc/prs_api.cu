@@ -498,7 +498,7 @@ static void step_plan(const prs_sim* s, const MarchPlan* march, int64_t nsteps, 
 }
 
 // Queue one pass of t steps from step n: phi[cur] -> phi[1 - cur], dphi from v_in to v_out (equal only
-// for t = 1).  Flips cur.
+// for t = 1).  Flips cur when the launch succeeds.
 static cudaError_t queue_pass(prs_sim* s, int t, int64_t n, const void* v_in, void* v_out)
 {
     const bool repro = (s->p.flags & PRS_REPRO) != 0;
@@ -524,7 +524,7 @@ static cudaError_t queue_pass(prs_sim* s, int t, int64_t n, const void* v_in, vo
         e = launch_step_io(s->g, s->p.precision, repro, in, out, v_in, v_out, &c[0][0], &c[0][1], &c[0][2], 1, s->rc,
                            err, s->stream);
     }
-    s->cur = 1 - s->cur;
+    if (e == cudaSuccess) s->cur = 1 - s->cur;
     return e;
 }
 

@@ -102,3 +102,30 @@ def test_nothing_is_in_flight_behind_an_ensemble_error(lib, call, nth):
     lib.fake_reset()
     assert lib.prs_batch_run(b, ns, 4, out.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), 4) == prs.PRS_OK
     assert lib.prs_batch_destroy(b) == prs.PRS_OK
+
+
+def _run(lib, shape, **kw):
+    h = ctypes.c_void_p()
+    assert lib.prs_create(ctypes.byref(prs.make_params(shape, **kw)), STREAM, ctypes.byref(h)) == prs.PRS_OK
+    return h
+
+
+def _state(lib, h):
+    p, v, n = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_int64()
+    assert lib.prs_device_state(h, ctypes.byref(p), ctypes.byref(v), ctypes.byref(n)) == prs.PRS_OK
+    return p.value, v.value, n.value
+
+
+@pytest.mark.parametrize("shape,kw", [((128, 128), {}), ((50, 40), dict(precision=prs.PRS_FP64)),
+                                      ((50, 40), dict(precision=prs.PRS_FP64, flags=prs.PRS_REPRO)),
+                                      ((128, 64, 64), {}), ((21, 20, 19), dict(tblock=1))])
+def test_a_launch_that_fails_leaves_the_state_where_it_is(lib, shape, kw):
+    h = _run(lib, shape, **kw)
+    assert lib.prs_init(h, None, None) == prs.PRS_OK
+    before = _state(lib, h)
+    lib.fake_fail(b"launch", 1, 9)  # an invalid configuration: the context stays usable
+    assert lib.prs_step(h, 1) == prs.PRS_ECUDA
+    assert _state(lib, h) == before
+    assert lib.prs_step(h, 1) == prs.PRS_OK
+    assert _state(lib, h)[0] != before[0] and _state(lib, h)[2] == 1
+    assert lib.prs_destroy(h) == prs.PRS_OK
