@@ -25,7 +25,9 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int block, size_t sm
     cfg.stream = st;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // the runtime keeps it, and a later plain launch would report it
+    return e;
 }
 
 }  // namespace prs

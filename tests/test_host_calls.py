@@ -129,3 +129,14 @@ def test_a_launch_that_fails_leaves_the_state_where_it_is(lib, shape, kw):
     assert lib.prs_step(h, 1) == prs.PRS_OK
     assert _state(lib, h)[0] != before[0] and _state(lib, h)[2] == 1
     assert lib.prs_destroy(h) == prs.PRS_OK
+
+
+@pytest.mark.parametrize("shape,kw", [((128, 128), {}), ((50, 40), dict(precision=prs.PRS_FP64)), ((128, 64, 64), {})])
+def test_a_launch_that_fails_is_reported_once(lib, shape, kw):
+    h = _run(lib, shape, **kw)
+    assert lib.prs_init(h, None, None) == prs.PRS_OK
+    lib.fake_fail(b"launch", 1, 9)
+    assert lib.prs_step(h, 1) == prs.PRS_ECUDA
+    J = ctypes.c_double()
+    assert lib.prs_observable(h, 0, 0.1, ctypes.byref(J)) == prs.PRS_OK
+    assert lib.prs_destroy(h) == prs.PRS_OK
