@@ -898,6 +898,7 @@ static int prs_adjoint_impl(prs_sim* s, int64_t nsteps, int observable, double e
         s->adj_timed = true;
     }
 #undef PRS_TRY
+    s->waits = false;
     int rc = check_device_error(s);
     if (rc) return rc;
     double da = 0.0;

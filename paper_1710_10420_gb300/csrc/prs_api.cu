@@ -513,6 +513,7 @@ static cudaError_t queue_pass(prs_sim* s, int t, int64_t n, const void* v_in, vo
                                   (float)s->rc[3], (float)s->rc[4], (float)s->rc[5]};
         e = launch_step_t2(s->g, (const float*)in, (float*)out, (const float*)v_in, (float*)v_out,
                            kick_f32(c[0], s->rc), kick_f32(c[1], s->rc), rcf, err, s->stream);
+        if (e == cudaSuccess) s->waits = true;
     }
     if (e == cudaErrorNotSupported && march_run(s) && (t > 1 || s->march.shape[1].cols)) {
         MarchRun r{in, out, v_in, v_out, {}, s->rc};
@@ -523,6 +524,7 @@ static cudaError_t queue_pass(prs_sim* s, int t, int64_t n, const void* v_in, vo
     } else if (e == cudaErrorNotSupported) {
         e = launch_step_io(s->g, s->p.precision, repro, in, out, v_in, v_out, &c[0][0], &c[0][1], &c[0][2], 1, s->rc,
                            err, s->stream);
+        if (fast_step_ok(s->g, s->p.precision)) s->waits = true;
     }
     if (e == cudaSuccess) s->cur = 1 - s->cur;
     return e;
@@ -616,6 +618,13 @@ static int prs_step_measure_impl(prs_sim* s, int64_t nsteps, prs_diag* out)
     scr.error = &s->d_status->error;
     const cudaError_t e = queue_measure(s, scr);
     if (e != cudaSuccess) return cuda_fail(e, "prs_measure launch");
+    const bool ask = nsteps > 0 && s->waits && !fast_diag_ok(s);
+    s->waits = false;  // the diagnostics bring the error word of the passes before them
+    if (ask) {
+        PRS_CUDA(cudaStreamSynchronize(s->stream));
+        const int err = check_device_error(s);
+        if (err) return err;
+    }
     if (nsteps > 0) {
         const int rs = prs_step(s, nsteps);
         if (rs) return rs;

@@ -22,6 +22,7 @@ struct prs_sim {
     bool have_buffers;
     bool initialised;
     int64_t n;           // step index of the state
+    bool waits;          // passes with bounded waits were queued since the error word was last read
     double rc[6];        // deta, 1/dx^2, 1/phi0^2, 2D, V0, phi0
     prs::DiagScratch scr;
     prs::MarchPlan march;     // FP32: the passes' shapes and times, for this run or a group it leads

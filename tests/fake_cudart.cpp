@@ -114,7 +114,7 @@ static cudaError_t get(const char* call, void** p, size_t n)
     *p = aligned_alloc(4096, (n + 4095) / 4096 * 4096);
     if (!*p) return g_last = cudaErrorMemoryAllocation;
     memset(*p, 0, n);
-    say("%s %zu", call, n);
+    say("%s %zu %zu", call, n, id(*p));
     return cudaSuccess;
 }
 cudaError_t cudaMalloc(void** p, size_t n) { return get("malloc", p, n); }

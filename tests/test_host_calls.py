@@ -140,3 +140,21 @@ def test_a_launch_that_fails_is_reported_once(lib, shape, kw):
     J = ctypes.c_double()
     assert lib.prs_observable(h, 0, 0.1, ctypes.byref(J)) == prs.PRS_OK
     assert lib.prs_destroy(h) == prs.PRS_OK
+
+
+def test_a_wait_that_gave_up_is_reported_before_the_state_is_stepped(lib):
+    """Correctly rounded diagnostics on a box of the staged passes: prs_step_measure returns the timeout of an
+    earlier pass (the test writes the error word the diagnostics would bring) and queues no step."""
+    h = _run(lib, (512, 512, 64), flags=prs.PRS_FP32_CR)
+    status = next(int(line[2]) for line in _log(lib) if line[0] == "mallochost")  # result (48 bytes), counter, error
+    assert lib.prs_init(h, None, None) == prs.PRS_OK
+    assert lib.prs_step(h, 1) == prs.PRS_OK
+    before = _state(lib, h)
+    ctypes.c_uint.from_address(status + 52).value = 1
+    lib.fake_reset()
+    d = prs.prs_diag()
+    assert lib.prs_step_measure(h, 3, ctypes.byref(d)) == prs.PRS_ETIMEOUT
+    assert len([line for line in _log(lib) if line[0] == "launch"]) == 1  # the diagnostics
+    assert _state(lib, h) == before
+    assert lib.prs_step_measure(h, 3, ctypes.byref(d)) == prs.PRS_OK and _state(lib, h)[2] == 4
+    assert lib.prs_destroy(h) == prs.PRS_OK
