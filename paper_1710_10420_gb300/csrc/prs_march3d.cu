@@ -107,8 +107,9 @@ int march3d_planes(const Geo& g, int t, int nruns, double* us)
 // The staged passes stay where they are the faster: one step on the boxes they take (1024^3: 2.54 ms,
 // HBM; the march 2.8), two steps on large boxes where the 256 x 8 tensor-copy tiles fit (us: 0.154 a
 // MB of the state crossing HBM twice and a start of up to 93, that is 2740 at 1024^3, 424 at 512^3 and
-// 65 at 256^3; the march 3100, 395 and 60).  Three steps are the march's: 3620, 510 and 80, which is the least
-// time a step from 1024^3 down to 100^3.
+// 65 at 256^3; the march 3100, 395 and 60; below 2^24 sites their few long tiles take 25 us whatever the box,
+// the march 6 to 16: 20 steps of 256 x 64 x 64 254 and 81 us).  Three steps are the march's: 3620, 510 and
+// 80, which is the least time a step from 1024^3 down to 100^3.
 void march_plan_3d(const Geo& g, int nruns, MarchPlan* p)
 {
     p->nruns = nruns;
@@ -121,7 +122,7 @@ void march_plan_3d(const Geo& g, int nruns, MarchPlan* p)
     const double mb = 16e-6 * (double)g.S;
     const double one = 3.5 + std::max(6.5, mb * 0.15), two = 3.5 + 0.154 * mb + std::min(93.0, 0.09 * mb);
     if (fast_step_ok(g, PRS_FP32) || !march3d_ok(g)) p->shape[1].cols = 0, p->us[1] = one;
-    if (t2tma_ok(g) && two < p->us[2]) p->shape[2].cols = 0, p->us[2] = two;
+    if (t2tma_ok(g) && g.S >= (int64_t)1 << 24 && two < p->us[2]) p->shape[2].cols = 0, p->us[2] = two;
 }
 
 void march_counts_3d(const MarchPlan& p, int64_t n, bool home, int64_t cnt[kMarchMaxT + 1])

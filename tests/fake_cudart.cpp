@@ -187,10 +187,14 @@ cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { return *
 // -------------------------------------------------------------- others
 cudaError_t cudaGetDevice(int* d) { return *d = 0, cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
-cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** f, unsigned, unsigned long long,
+static int encode_nothing() { return 0; }  // the tensor-map encoder
+cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** f, unsigned, unsigned long long,
                                              cudaDriverEntryPointQueryResult* q)
 {
-    return *f = nullptr, *q = cudaDriverEntryPointSymbolNotFound, cudaSuccess;
+    const bool have = !strcmp(name, "cuTensorMapEncodeTiled");
+    *f = have ? (void*)encode_nothing : nullptr;
+    *q = have ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
+    return cudaSuccess;
 }
 cudaError_t cudaGetLastError()
 {

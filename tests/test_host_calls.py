@@ -158,3 +158,17 @@ def test_a_wait_that_gave_up_is_reported_before_the_state_is_stepped(lib):
     assert _state(lib, h) == before
     assert lib.prs_step_measure(h, 3, ctypes.byref(d)) == prs.PRS_OK and _state(lib, h)[2] == 4
     assert lib.prs_destroy(h) == prs.PRS_OK
+
+
+@pytest.mark.parametrize("shape", [(256, 32, 32), (256, 64, 64), (1024, 32, 32), (256, 256, 32), (768, 128, 32),
+                                   (256, 512, 32)])
+@pytest.mark.parametrize("steps", [20, 13, 2])
+def test_small_boxes_take_no_staged_pairs(lib, shape, steps):
+    """The staged two-step tiles take 25 us on a box of few of them, several times the march's passes."""
+    h = _run(lib, shape)
+    assert lib.prs_init(h, None, None) == prs.PRS_OK
+    lib.fake_reset()
+    assert lib.prs_step(h, steps) == prs.PRS_OK
+    names = [line[2] for line in _log(lib) if line[0] == "launch"]
+    assert names and not any("step3d_t2" in name for name in names)
+    assert lib.prs_destroy(h) == prs.PRS_OK
