@@ -135,9 +135,10 @@ typedef struct {
 /* ------------------------------------------------------------ single runs */
 
 /* Create a run.  Validates the parameters, including the leapfrog stability
- * limit deta^2 (4 D/dx^2 + max|V''|) < 4 (Eqs. 3-5), and allocates the small
- * device scratch used by the diagnostics.  Field buffers are allocated on the
- * first prs_init/prs_set_state unless prs_bind supplies them.
+ * limit deta^2 (4 D/dx^2 + max|V''|) < 4 (Eqs. 3-5).  Device memory (the fields unless
+ * prs_bind supplies them, the diagnostics' scratch and, for runs that take passes of
+ * several steps, one more field; see prs_step) is allocated in one piece, by prs_bind
+ * or else by the first prs_init/prs_set_state.
  * stream: a cudaStream_t, or NULL.  *out receives the handle. */
 int prs_create(const prs_params* params, void* stream, prs_sim** out);
 
@@ -145,7 +146,9 @@ int prs_create(const prs_params* params, void* stream, prs_sim** out);
  * d_phi_a and d_phi_b each hold one field (the leapfrog writes phi^{n+1} into the
  * buffer that does not hold phi^n); d_dphi holds dphi and is updated in place.
  * Each must be 16-byte aligned and hold sites * element-size bytes; they stay
- * owned by the caller and must outlive the run.  Must precede prs_init. */
+ * owned by the caller and must outlive the run.  Must precede prs_init.  Allocates the
+ * run's own device memory (see prs_create), so that no later call of the run but
+ * prs_observable and prs_adjoint has to: PRS_ENOMEM if the scratch does not fit. */
 int prs_bind(prs_sim* sim, void* d_phi_a, void* d_phi_b, void* d_dphi);
 
 /* Set the initial state (step 0).  h_phi == NULL: phi_s is drawn on the device
@@ -160,12 +163,12 @@ int prs_init(prs_sim* sim, const void* h_phi, const void* h_dphi);
  * Step n uses delta_n, eta_n = eta0 + n deta.  Every step of the call must satisfy the
  * stability limit (checked at both ends, where the force prefactor a^beta is largest),
  * else PRS_EINVAL.  Passes of two and more steps (see prs_params.tblock) read dphi
- * across sites and write it out of place, into a second dphi buffer that prs_init,
- * prs_set_state or prs_set_state_device allocate when the run may take such passes (FP32
- * with tblock = 0, or a tblock that fuses steps on its box;
- * owned by the run, freed by prs_destroy; if that allocation fails, the steps run one
- * per pass).  With tblock = 0 a call of nsteps runs the passes that its plan of the box
- * gives the least time, the longest first, single steps last.  With T = tblock >= 2 it runs
+ * across sites and write it out of place, into a second dphi buffer that is part of the
+ * run's device memory when the run may take such passes (FP32 with tblock = 0, or a tblock
+ * that fuses steps on its box; owned by the run, freed by prs_destroy; if it does not fit,
+ * every prs_init and prs_set_state* tries again, and until then the steps run one per
+ * pass).  With tblock = 0 a call of nsteps runs the passes that its plan of the box gives
+ * the least time, the longest first, single steps last.  With T = tblock >= 2 it runs
  * nsteps / T passes of T steps, then (T = 3) one pair if two steps remain, then single
  * steps.  Where dphi ends:
  *   - library-owned buffers (no prs_bind, no PRS_DEBUG): after an odd number of

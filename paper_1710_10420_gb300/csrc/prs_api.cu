@@ -185,22 +185,9 @@ extern "C" int prs_create(const prs_params* params, void* stream, prs_sim** out)
     s->rc[5] = params->phi0;
     s->scr.max_blocks = kMeasureBlocks;
     if (march_run(s)) make_plan(s, 1);
-    void* blob = nullptr;
-    size_t bytes = sizeof(DiagAcc) * kMeasureBlocks + sizeof(DevStatus);
-    if (cudaMalloc(&blob, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        delete s;
-        return PRS_ENOMEM;
-    }
-    s->scr.partials = (DiagAcc*)blob;
-    s->d_status = (DevStatus*)(s->scr.partials + kMeasureBlocks);
-    s->scr.result = &s->d_status->result;
-    s->scr.counter = &s->d_status->counter;
-    if (cudaMemsetAsync(blob, 0, bytes, s->stream) != cudaSuccess ||
-        cudaMallocHost((void**)&s->h_status, sizeof(DevStatus)) != cudaSuccess ||
+    if (cudaMallocHost((void**)&s->h_status, sizeof(DevStatus)) != cudaSuccess ||
         ((params->flags & PRS_DEBUG) && cudaMalloc((void**)&s->d_dbg, sizeof(DebugCheck)) != cudaSuccess)) {
         int r = cuda_fail(cudaGetLastError(), "prs_create");
-        cudaFree(blob);
         cudaFreeHost(s->h_status);
         delete s;
         return r;
@@ -209,11 +196,64 @@ extern "C" int prs_create(const prs_params* params, void* stream, prs_sim** out)
     return PRS_OK;
 }
 
+// Steps per pass this run takes (params.tblock, or the library's choice, clamped).
+static int run_tblock(const prs_sim* s)
+{
+    const bool repro = (s->p.flags & PRS_REPRO) != 0;
+    int tmax = max_fused_steps(s->g, s->p.precision, repro);
+    int tb = s->p.tblock > 0 ? s->p.tblock : default_fused_steps(s->g, s->p.precision, repro);
+    if (tb > tmax) tb = tmax;
+    return tb < 1 ? 1 : tb;
+}
+
+// Whether the run takes passes of several steps, which need a second dphi buffer.
+static bool wants_alt(const prs_sim* s) { return run_tblock(s) >= 2 || march_plans(s); }
+
+// One allocation of `fields` fields, the second dphi buffer and the diagnostics' scratch; without the
+// buffer where it does not fit.  (Beyond 2 MB an allocation takes 30 to 100 us, and as long to free: a run of
+// 128^3 with its own fields 493 us from creation to release, with an allocation each 812; bound 498 and 630.)
+static int alloc_run(prs_sim* s, int fields)
+{
+    const size_t fs = ((size_t)s->g.S * s->elem + 511) & ~(size_t)511;
+    const size_t scratch = sizeof(DiagAcc) * kMeasureBlocks + sizeof(DevStatus);
+    void* m = nullptr;
+    bool alt = wants_alt(s);
+    if (cudaMalloc(&m, fs * (size_t)(fields + (alt ? 1 : 0)) + scratch) != cudaSuccess) {
+        cudaGetLastError();
+        if (!alt) return PRS_ENOMEM;
+        alt = false;
+        if (cudaMalloc(&m, fs * (size_t)fields + scratch) != cudaSuccess) {
+            cudaGetLastError();
+            return PRS_ENOMEM;
+        }
+    }
+    char* c = (char*)m + fs * (size_t)(fields + (alt ? 1 : 0));
+    const cudaError_t e = cudaMemsetAsync(c, 0, scratch, s->stream);
+    if (e != cudaSuccess) {
+        cudaFree(m);
+        return cuda_fail(e, "scratch of the diagnostics");
+    }
+    s->mem = m;
+    s->scr.partials = (DiagAcc*)c;
+    s->d_status = (DevStatus*)(s->scr.partials + kMeasureBlocks);
+    s->scr.result = &s->d_status->result;
+    s->scr.counter = &s->d_status->counter;
+    if (alt) s->dphi_alt = (char*)m + fs * (size_t)fields;
+    if (fields) {
+        s->phi[0] = m;
+        s->phi[1] = (char*)m + fs;
+        s->dphi = (char*)m + 2 * fs;
+    }
+    return PRS_OK;
+}
+
 extern "C" int prs_bind(prs_sim* s, void* d_phi_a, void* d_phi_b, void* d_dphi)
 {
     if (!s || !d_phi_a || !d_phi_b || !d_dphi || d_phi_a == d_phi_b) return PRS_EINVAL;
     if (((uintptr_t)d_phi_a | (uintptr_t)d_phi_b | (uintptr_t)d_dphi) & 15u) return PRS_EINVAL;
     if (s->have_buffers) return PRS_ESTATE;
+    const int rc = alloc_run(s, 0);
+    if (rc) return rc;
     s->phi[0] = d_phi_a;
     s->phi[1] = d_phi_b;
     s->dphi = d_dphi;
@@ -226,36 +266,23 @@ extern "C" int prs_bind(prs_sim* s, void* d_phi_a, void* d_phi_b, void* d_dphi)
 int prs::ensure_buffers(prs_sim* s)
 {
     if (s->have_buffers) return PRS_OK;
-    size_t bytes = (size_t)s->g.S * s->elem;
     if (s->p.flags & PRS_DEBUG) {
+        const size_t bytes = (size_t)s->g.S * s->elem;
         void* f[3] = {nullptr, nullptr, nullptr};
-        for (int i = 0; i < 3; ++i) {
-            int rc = debug_alloc_field(bytes, &s->guard_base[i], &f[i]);
-            if (rc) {
-                for (int k = 0; k < i; ++k) cudaFree(s->guard_base[k]), s->guard_base[k] = nullptr;
-                return rc;
-            }
+        int rc = PRS_OK;
+        for (int i = 0; i < 3 && !rc; ++i) rc = debug_alloc_field(bytes, &s->guard_base[i], &f[i]);
+        if (!rc) rc = alloc_run(s, 0);
+        if (rc) {
+            for (int k = 0; k < 3; ++k) cudaFree(s->guard_base[k]), s->guard_base[k] = nullptr;
+            return rc;
         }
         s->phi[0] = f[0];
         s->phi[1] = f[1];
         s->dphi = f[2];
-        s->cur = 0;
-        s->owned = true;
-        s->have_buffers = true;
-        return PRS_OK;
+    } else {
+        const int rc = alloc_run(s, 3);
+        if (rc) return rc;
     }
-    void *a = nullptr, *b = nullptr, *v = nullptr;
-    if (cudaMalloc(&a, bytes) != cudaSuccess || cudaMalloc(&b, bytes) != cudaSuccess ||
-        cudaMalloc(&v, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(a);
-        cudaFree(b);
-        cudaFree(v);
-        return PRS_ENOMEM;
-    }
-    s->phi[0] = a;
-    s->phi[1] = b;
-    s->dphi = v;
     s->cur = 0;
     s->owned = true;
     s->have_buffers = true;
@@ -266,16 +293,10 @@ extern "C" int prs_destroy(prs_sim* s)
 {
     if (!s) return PRS_EINVAL;
     cudaStreamSynchronize(s->stream);
-    if (s->owned && (s->p.flags & PRS_DEBUG)) {
-        for (int i = 0; i < 3; ++i) cudaFree(s->guard_base[i]);
-    } else if (s->owned) {
-        cudaFree(s->phi[0]);
-        cudaFree(s->phi[1]);
-        cudaFree(s->dphi);
-    }
+    for (int i = 0; i < 3; ++i) cudaFree(s->guard_base[i]);
+    cudaFree(s->mem);
+    cudaFree(s->alt_mem);
     cudaFree(s->d_dbg);
-    cudaFree(s->scr.partials);
-    cudaFree(s->dphi_alt);
     cudaFree(s->adj_ws);
     for (cudaEvent_t e : s->adj_ev) cudaEventDestroy(e);
     cudaFreeHost(s->h_status);
@@ -285,28 +306,17 @@ extern "C" int prs_destroy(prs_sim* s)
 
 // ------------------------------------------------------------------ state
 
-// Steps per pass this run takes (params.tblock, or the library's choice, clamped).
-static int run_tblock(const prs_sim* s)
-{
-    const bool repro = (s->p.flags & PRS_REPRO) != 0;
-    int tmax = max_fused_steps(s->g, s->p.precision, repro);
-    int tb = s->p.tblock > 0 ? s->p.tblock : default_fused_steps(s->g, s->p.precision, repro);
-    if (tb > tmax) tb = tmax;
-    return tb < 1 ? 1 : tb;
-}
-
-// The second dphi buffer of two-step passes, allocated with the fields (prs_init,
-// prs_set_state) so that prs_step itself never allocates; if there is no room the run
-// steps one step per pass.
+// The second dphi buffer where it did not fit beside the fields, tried again with every new state, so that
+// prs_step itself never allocates; while there is no room the run steps one step per pass.
 static void ensure_dphi_alt(prs_sim* s)
 {
-    if (s->dphi_alt || (run_tblock(s) < 2 && !march_plans(s))) return;
-    if (cudaMalloc(&s->dphi_alt, (size_t)s->g.S * s->elem) != cudaSuccess) {
+    if (s->dphi_alt || !wants_alt(s)) return;
+    if (cudaMalloc(&s->alt_mem, (size_t)s->g.S * s->elem) != cudaSuccess) {
         cudaGetLastError();
-        s->dphi_alt = nullptr;
+        s->alt_mem = nullptr;
     }
+    s->dphi_alt = s->alt_mem;
 }
-
 
 static int prs_init_impl(prs_sim* s, const void* h_phi, const void* h_dphi)
 {

@@ -122,8 +122,6 @@ static int batch_setup(prs_batch* b, const prs_params* runs, int nruns, void* st
         b->groups[k].runs.push_back(r);
         b->sims[r]->stream = b->groups[k].stream;
     }
-    // the runs' scratch was cleared on the ensemble's stream
-    if ((rc = batch_cuda(cudaStreamSynchronize(b->stream), "prs_batch_create"))) return rc;
     size_t off = 0;
     for (int r = 0; r < nruns; ++r) {
         prs_sim* s = b->sims[r];

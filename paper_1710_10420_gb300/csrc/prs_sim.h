@@ -24,11 +24,13 @@ struct prs_sim {
     int64_t n;           // step index of the state
     bool waits;          // passes with bounded waits were queued since the error word was last read
     double rc[6];        // deta, 1/dx^2, 1/phi0^2, 2D, V0, phi0
+    void* mem;           // library-owned fields (not with PRS_DEBUG), second dphi buffer, scratch
     prs::DiagScratch scr;
     prs::MarchPlan march;     // FP32: the passes' shapes and times, for this run or a group it leads
     prs::DevStatus* d_status; // device: result, counter, error word
     prs::DevStatus* h_status; // pinned host copy
-    void* dphi_alt;           // second dphi buffer for passes that read dphi across sites (library-owned)
+    void* dphi_alt;           // second dphi buffer for passes that read dphi across sites (in mem or alt_mem)
+    void* alt_mem;            // where it did not fit mem
     void* adj_ws;             // prs_adjoint working memory, kept for the next call
     size_t adj_ws_bytes;
     std::vector<cudaEvent_t> adj_ev; // prs_adjoint phase boundaries (created on demand)

@@ -172,3 +172,43 @@ def test_small_boxes_take_no_staged_pairs(lib, shape, steps):
     names = [line[2] for line in _log(lib) if line[0] == "launch"]
     assert names and not any("step3d_t2" in name for name in names)
     assert lib.prs_destroy(h) == prs.PRS_OK
+
+
+def _mallocs(lib):
+    return [int(line[1]) for line in _log(lib) if line[0] == "malloc"]
+
+
+@pytest.mark.parametrize("shape,kw", [((128, 128, 128), {}), ((250, 170), {}), ((256, 256), {}), ((45, 42, 38), {}),
+                                      ((64, 64), dict(precision=prs.PRS_FP64)), ((100, 90), dict(tblock=1))])
+@pytest.mark.parametrize("bound", [True, False])
+def test_a_run_allocates_once(lib, shape, kw, bound):
+    """Creation and the first state take one device allocation, and the first state of bound buffers none
+    (so it may be captured)."""
+    nbytes = int(np.prod(shape)) * (8 if kw.get("precision") else 4)
+    phi, v = np.zeros(nbytes, np.uint8), np.zeros(nbytes, np.uint8)
+    h = _run(lib, shape, **kw)
+    bufs = [np.zeros(nbytes + 64, np.uint8) for _ in range(3)]
+    if bound:
+        assert lib.prs_bind(h, *[b.ctypes.data + -b.ctypes.data % 16 for b in bufs]) == prs.PRS_OK
+        assert len(_mallocs(lib)) == 1
+    assert lib.prs_set_state_device(h, phi.ctypes.data, v.ctypes.data, 0) == prs.PRS_OK
+    assert lib.prs_step(h, 7) == prs.PRS_OK
+    assert len(_mallocs(lib)) == 1
+    assert lib.prs_destroy(h) == prs.PRS_OK
+    assert len([line for line in _log(lib) if line[0] == "free"]) == 1
+
+
+@pytest.mark.parametrize("fields", [4, 3])
+def test_a_run_without_room_for_the_second_dphi_buffer(lib, fields):
+    """Where four fields do not fit in one allocation the run takes three and asks for the fourth apart."""
+    n = 4 * 64 ** 3
+    h = _run(lib, (64, 64, 64))
+    lib.fake_limit(4 * n if fields == 4 else 3 * n)  # with the scratch, neither fits whole
+    assert lib.prs_init(h, None, None) == (prs.PRS_OK if fields == 4 else prs.PRS_ENOMEM)
+    if fields == 4:
+        assert len(_mallocs(lib)) == 2
+        assert lib.prs_step(h, 6) == prs.PRS_OK and _state(lib, h)[2] == 6
+    lib.fake_limit(0)
+    assert lib.prs_init(h, None, None) == prs.PRS_OK
+    assert lib.prs_destroy(h) == prs.PRS_OK
+    assert len([line for line in _log(lib) if line[0] == "free"]) == len(_mallocs(lib))
