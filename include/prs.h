@@ -273,7 +273,7 @@ int prs_destroy(prs_sim* sim);
  * box are stepped together: each pass, and each output's diagnostics, is one launch over
  * up to 16 of them, and the groups run concurrently.  Runs must be FP32 with an x side
  * that is a multiple of 128 dividing 4096 (3D: at most 1024) and 4096/x dividing the y
- * side. */
+ * side; their tblock is checked and then left aside (the steps of a pass are the group's). */
 
 /* Create an ensemble of nruns runs (each validated as by prs_create), allocate all
  * fields, then set every run to its seeded random initial condition (step 0).  A run's

@@ -212,3 +212,16 @@ def test_a_run_without_room_for_the_second_dphi_buffer(lib, fields):
     assert lib.prs_init(h, None, None) == prs.PRS_OK
     assert lib.prs_destroy(h) == prs.PRS_OK
     assert len([line for line in _log(lib) if line[0] == "free"]) == len(_mallocs(lib))
+
+
+@pytest.mark.parametrize("tblocks", [[0, 0, 1, 0], [1, 1, 1, 1], [3, 2, 0, 1]])
+@pytest.mark.parametrize("shape", [(256, 64), (128, 32, 16)])
+def test_runs_of_an_ensemble_share_their_launches_whatever_their_tblock(lib, shape, tblocks):
+    counts = []
+    for tbs in (tblocks, [0] * len(tblocks)):
+        b = _batch(lib, [prs.make_params(shape, tblock=t) for t in tbs], STREAM)
+        ns = (ctypes.c_int64 * len(tbs))(*[20] * len(tbs))
+        assert lib.prs_batch_run(b, ns, 0, None, 0) == prs.PRS_OK
+        counts.append([line[2] for line in _log(lib) if line[0] == "launch"])
+        assert lib.prs_batch_destroy(b) == prs.PRS_OK
+    assert counts[0] == counts[1] and len(counts[1]) <= 20
