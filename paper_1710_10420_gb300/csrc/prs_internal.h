@@ -151,7 +151,7 @@ struct MeasureRun {
     DiagScratch scr;
 };
 // fast (FP32): hardware reciprocal square root and division, else IEEE operations.  err: the run's
-// error word.
+// error word, or null for staging without bounded waits.
 cudaError_t launch_measure(const Geo& g, int precision, bool fast, const MeasureRun& run, unsigned int* err,
                            cudaStream_t st);
 // Up to kMeasureMaxRuns FP32 runs of one box in one launch, as launch_measure with fast.
@@ -179,9 +179,6 @@ cudaError_t launch_step_t2_tma(const Geo& g, const float* phi_in, float* phi_out
 
 // Store a message for prs_last_error() on this thread.
 void record_error(const char* msg);
-
-// The diagnostic kernel (IEEE operations) on at most `grid` blocks (1 <= grid <= scr.max_blocks).
-cudaError_t launch_measure_on_grid(const Geo& g, int precision, const MeasureRun& run, int grid, cudaStream_t st);
 
 // Host-side setup shared by the launchers.  Calls on different prs_sim handles may
 // run concurrently from several host threads, so neither keeps unsynchronised state.

@@ -533,7 +533,7 @@ bool phi_map(CUtensorMap* m, const R* phi, const Geo& g, const MTiling& T)
 }
 
 template <typename R, int D, bool FAST, int NR>
-cudaError_t measure_t(const Geo& g, int nruns, const MeasureRun* q, unsigned int* err, int grid, cudaStream_t st)
+cudaError_t measure_t(const Geo& g, int nruns, const MeasureRun* q, unsigned int* err, cudaStream_t st)
 {
     static std::atomic<unsigned long long> attr{0};
     const int sms = sm_count_current();
@@ -544,11 +544,10 @@ cudaError_t measure_t(const Geo& g, int nruns, const MeasureRun* q, unsigned int
     cudaError_t e = smem_limit_once(attr, (const void*)k_measure<R, D, FAST, NR>,
                                     (int)(sizeof(R) == 4 ? measure_smem(D, 4, most) : 100 * 1024));
     if (e != cudaSuccess) return e;
-    if (grid <= 0) {  // the resident CTAs, shared by the runs; one partial slot each
-        const int all = ctas_per_sm(D, sizeof(R), T) * sms / nruns;
-        grid = T.ntiles < (unsigned)all ? (int)T.ntiles : (all > 0 ? all : 1);
-        if (grid > q[0].scr.max_blocks) grid = q[0].scr.max_blocks;
-    }
+    // the resident CTAs, shared by the runs; one partial slot each
+    const int all = ctas_per_sm(D, sizeof(R), T) * sms / nruns;
+    int grid = T.ntiles < (unsigned)all ? (int)T.ntiles : (all > 0 ? all : 1);
+    if (grid > q[0].scr.max_blocks) grid = q[0].scr.max_blocks;
     MRuns<R, NR> runs;
     uintptr_t bits = 0;
     for (int r = 0; r < nruns; ++r) {
@@ -561,16 +560,16 @@ cudaError_t measure_t(const Geo& g, int nruns, const MeasureRun* q, unsigned int
     }
     const bool vec = g.nx % MRow<R>::kOff == 0 && (bits & 15u) == 0;
     CUtensorMap map{};
-    if (NR > 1 || !vec || !phi_map(&map, (const R*)q[0].phi, g, T)) err = nullptr;
+    if (NR > 1 || !err || !vec || !phi_map(&map, (const R*)q[0].phi, g, T)) err = nullptr;
     return launch_chained(k_measure<R, D, FAST, NR>, dim3((unsigned)grid, (unsigned)nruns), kMThreads,
                           measure_smem(D, sizeof(R), T), st, map, runs, g, T, vec, err);
 }
 
 template <typename R, bool FAST, int NR>
-cudaError_t measure_d(const Geo& g, int nruns, const MeasureRun* q, unsigned int* err, int grid, cudaStream_t st)
+cudaError_t measure_d(const Geo& g, int nruns, const MeasureRun* q, unsigned int* err, cudaStream_t st)
 {
-    return g.dims == 3 ? measure_t<R, 3, FAST, NR>(g, nruns, q, err, grid, st)
-                       : measure_t<R, 2, FAST, NR>(g, nruns, q, err, grid, st);
+    return g.dims == 3 ? measure_t<R, 3, FAST, NR>(g, nruns, q, err, st)
+                       : measure_t<R, 2, FAST, NR>(g, nruns, q, err, st);
 }
 
 }  // namespace
@@ -578,23 +577,14 @@ cudaError_t measure_d(const Geo& g, int nruns, const MeasureRun* q, unsigned int
 cudaError_t launch_measure(const Geo& g, int precision, bool fast, const MeasureRun& run, unsigned int* err,
                            cudaStream_t st)
 {
-    if (precision != PRS_FP32) return measure_d<double, false, 1>(g, 1, &run, err, 0, st);
-    return fast ? measure_d<float, true, 1>(g, 1, &run, err, 0, st) : measure_d<float, false, 1>(g, 1, &run, err, 0, st);
+    if (precision != PRS_FP32) return measure_d<double, false, 1>(g, 1, &run, err, st);
+    return fast ? measure_d<float, true, 1>(g, 1, &run, err, st) : measure_d<float, false, 1>(g, 1, &run, err, st);
 }
 
 cudaError_t launch_measure_runs(const Geo& g, int nruns, const MeasureRun* runs, cudaStream_t st)
 {
     if (nruns < 1 || nruns > kMeasureMaxRuns) return cudaErrorInvalidValue;
-    return measure_d<float, true, kMeasureMaxRuns>(g, nruns, runs, nullptr, 0, st);
-}
-
-cudaError_t launch_measure_on_grid(const Geo& g, int precision, const MeasureRun& run, int grid, cudaStream_t st)
-{
-    if (grid < 1 || grid > run.scr.max_blocks) return cudaErrorInvalidValue;
-    const int most = 3 * sm_count_current();  // resident CTAs: more only add partials
-    if (grid > most) grid = most;
-    if (precision == PRS_FP32) return measure_d<float, false, 1>(g, 1, &run, nullptr, grid, st);
-    return measure_d<double, false, 1>(g, 1, &run, nullptr, grid, st);
+    return measure_d<float, true, kMeasureMaxRuns>(g, nruns, runs, nullptr, st);
 }
 
 }  // namespace prs

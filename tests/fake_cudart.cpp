@@ -42,10 +42,11 @@ cudaError_t done(const char* call)
 
 size_t id(const void* p) { return (size_t)p; }
 
-cudaError_t launch(const void* func, cudaStream_t st)
+cudaError_t launch(const void* func, dim3 grid, cudaStream_t st)
 {
     const cudaError_t e = done("launch");
-    if (e == cudaSuccess) say("launch %zu %s", id(st), g_names.count(func) ? g_names[func].c_str() : "?");
+    const char* name = g_names.count(func) ? g_names[func].c_str() : "?";
+    if (e == cudaSuccess) say("launch %zu %s %zu", id(st), name, (size_t)grid.x * grid.y * grid.z);
     return e;
 }
 
@@ -90,11 +91,14 @@ cudaError_t __cudaPopCallConfiguration(dim3* grid, dim3* block, size_t* smem, vo
     *grid = t_config.grid, *block = t_config.block, *smem = t_config.smem, *(cudaStream_t*)st = t_config.st;
     return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void**, size_t, cudaStream_t st)
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void**, size_t, cudaStream_t st)
 {
-    return launch((const void*)k, st);
+    return launch((const void*)k, grid, st);
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) { return launch(f, c->stream); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**)
+{
+    return launch(f, c->gridDim, c->stream);
+}
 cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* n, const void*, int, size_t)
 {
@@ -145,7 +149,11 @@ cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t st)
 }
 cudaError_t cudaMemset(void* d, int v, size_t n) { return memset(d, v, n), cudaSuccess; }
 cudaError_t cudaMemGetInfo(size_t* f, size_t* t) { return *f = *t = (size_t)1 << 38, cudaSuccess; }
-cudaError_t cudaGetSymbolAddress(void**, const void*) { return g_last = cudaErrorInvalidSymbol; }
+cudaError_t cudaGetSymbolAddress(void** p, const void*)
+{
+    static char array[4 << 20];
+    return *p = array, cudaSuccess;
+}
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes*, const void*) { return g_last = cudaErrorInvalidValue; }
 
 // -------------------------------------------------- streams and events

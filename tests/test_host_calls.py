@@ -84,8 +84,8 @@ def test_ensemble_state_copies_follow_the_callers_stream(lib, write):
     assert lib.prs_batch_destroy(b) == prs.PRS_OK
 
 
-@pytest.mark.parametrize("call,nth", [("record", 1), ("wait", 1), ("wait", 2), ("wait", 3), ("launch", 2), ("launch", 5),
-                                      ("copy", 1), ("copy", 2), ("copy", 3), ("record", 2), ("record", 3), ("sync", 1)])
+@pytest.mark.parametrize("call,nth", [("record", 1), ("wait", 1), ("wait", 2), ("wait", 3), ("launch", 2),
+                                      ("launch", 5), ("copy", 1), ("copy", 2), ("copy", 3), ("record", 2), ("record", 3), ("sync", 1)])
 def test_nothing_is_in_flight_behind_an_ensemble_error(lib, call, nth):
     """When a CUDA call fails in the middle of prs_batch_run, every stream that was given work is waited
     for before the error is returned (the caller may free its memory, and the groups are not joined)."""
@@ -225,3 +225,13 @@ def test_runs_of_an_ensemble_share_their_launches_whatever_their_tblock(lib, sha
         counts.append([line[2] for line in _log(lib) if line[0] == "launch"])
         assert lib.prs_batch_destroy(b) == prs.PRS_OK
     assert counts[0] == counts[1] and len(counts[1]) <= 20
+
+
+@pytest.mark.parametrize("shape,tiles", [((4096, 3), 32), ((256, 256), 16), ((64, 64, 64), 32)])
+def test_noalloc_diagnostics_fill_the_gpu(lib, shape, tiles):
+    phi = np.zeros(tuple(reversed(shape)), np.float32)
+    d = prs.prs_diag()
+    p, at = ctypes.byref(prs.make_params(shape)), phi.ctypes.data
+    assert lib.prs_measure_noalloc(p, at, at, STREAM, ctypes.byref(d)) == prs.PRS_OK
+    assert [int(line[3]) >= tiles for line in _log(lib) if line[0] == "launch"] == [True]
+    assert not _mallocs(lib)
