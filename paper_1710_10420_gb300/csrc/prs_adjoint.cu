@@ -816,8 +816,8 @@ static int prs_adjoint_impl(prs_sim* s, int64_t nsteps, int observable, double e
             } else {
                 char* x = slot(k);
                 char* y = slot(k + 1);
-                e = launch_step_io(s->g, s->p.precision, repro, x, y, x + fs, y + fs, &c0[0], &c0[1], &c0[2], 1,
-                                   s->rc, err, st);
+                e = launch_step_io(s->g, s->p.precision, repro, x, y, x + fs, y + fs, c0, s->rc,
+                                   s->march.shape[1], err, st);
                 k += 1;
             }
             if (e != cudaSuccess) return e;

@@ -155,13 +155,15 @@ extern "C" int prs_max_tblock(const prs_params* params)
 static const int kMeasureBlocks = 8192;  // partial slots: the fast kernels use one per tile
 
 // FP32 runs step by the register marches (prs_march2d.cuh, prs_march3d.cuh; in 3D beside the staged
-// passes); without a tblock their plan also sets the steps of the passes.
+// passes); without a tblock their plan also sets the steps of the passes.  An FP64 run's plan is the shape of
+// its one-step passes.  (Planned with every launch it took 1.5 us of 12 for a step of 64^2.)
 static bool march_run(const prs_sim* s) { return s->p.precision == PRS_FP32; }
 static bool march_plans(const prs_sim* s) { return march_run(s) && s->p.tblock == 0; }
 static void make_plan(prs_sim* s, int nruns)
 {
     if (s->march.nruns == nruns) return;
-    if (s->g.dims == 2) march_plan(s->g, nruns, &s->march);
+    if (!march_run(s)) s->march.nruns = nruns, s->march.shape[1] = fix64_shape(s->g);
+    else if (s->g.dims == 2) march_plan(s->g, nruns, &s->march);
     else march_plan_3d(s->g, nruns, &s->march);
 }
 
@@ -184,7 +186,7 @@ extern "C" int prs_create(const prs_params* params, void* stream, prs_sim** out)
     s->rc[4] = potential_height(*params);
     s->rc[5] = params->phi0;
     s->scr.max_blocks = kMeasureBlocks;
-    if (march_run(s)) make_plan(s, 1);
+    make_plan(s, 1);
     if (cudaMallocHost((void**)&s->h_status, sizeof(DevStatus)) != cudaSuccess ||
         ((params->flags & PRS_DEBUG) && cudaMalloc((void**)&s->d_dbg, sizeof(DebugCheck)) != cudaSuccess)) {
         int r = cuda_fail(cudaGetLastError(), "prs_create");
@@ -532,8 +534,8 @@ static cudaError_t queue_pass(prs_sim* s, int t, int64_t n, const void* v_in, vo
         e = s->g.dims == 2 ? launch_march2d(s->g, t, s->march.shape[t], 1, &r, s->stream)
                            : launch_march3d(s->g, t, s->march.shape[t].cy, 1, &r, s->stream);
     } else if (e == cudaErrorNotSupported) {
-        e = launch_step_io(s->g, s->p.precision, repro, in, out, v_in, v_out, &c[0][0], &c[0][1], &c[0][2], 1, s->rc,
-                           err, s->stream);
+        e = launch_step_io(s->g, s->p.precision, repro, in, out, v_in, v_out, c[0], s->rc, s->march.shape[1], err,
+                           s->stream);
         if (fast_step_ok(s->g, s->p.precision)) s->waits = true;
     }
     if (e == cudaSuccess) s->cur = 1 - s->cur;
@@ -546,7 +548,7 @@ static int prs_step_impl(prs_sim* s, int64_t nsteps)
     if (!s->initialised) return PRS_ESTATE;
     if (nsteps == 0) return PRS_OK;
     if (!cfl_ok_over(s->p, s->n, nsteps)) return PRS_EINVAL;
-    if (march_run(s)) make_plan(s, 1);
+    make_plan(s, 1);
     int64_t cnt[kMarchMaxT + 1];
     step_plan(s, &s->march, nsteps, cnt);
     void* vbuf[2] = {s->dphi, s->dphi_alt};

@@ -39,6 +39,7 @@
 
 #include "prs_chain.h"
 #include "prs_internal.h"
+#include "prs_march2d.h"
 #include "prs_ptx.cuh"
 #include "prs_site.cuh"
 
@@ -300,8 +301,31 @@ static bool make_fix64(const KickD& k, double phi0, Fix64* f)
     return true;
 }
 
+// Columns a lane owns and planes (2D: rows) a warp marches.
+MarchShape fix64_shape(const Geo& g)
+{
+    // 2D: two columns a lane share a row's bookkeeping, one makes twice the warps (us a step, two and one:
+    // 256^2 4.0 3.4, 400^2 4.6 4.3, 512^2 5.2 5.5, 1024^2 11.9 13.2, 2048^2 39 44)
+    const int cols = g.dims == 3 || g.S < ((int64_t)1 << 18) ? 1 : 2, width = fx_width(cols);
+    const int nstrips = (g.nx + width - 1) / width, len = g.dims == 3 ? g.nz : g.ny;
+    const int ygroups = g.dims == 3 ? (g.ny + 4 * kFxWarps - 1) / (4 * kFxWarps) : 1;
+    // warps (2D) or blocks of them (3D) against the two planes a chunk re-reads and the iteration
+    // that fills it
+    const double tiles = (double)nstrips * ygroups / (g.dims == 3 ? 1 : kFxWarps);
+    const double slots = (double)fx_blocks(g.dims, cols) * sm_count_current();
+    double least = 1e300;
+    MarchShape best{cols, len};
+    for (int nc = 1; nc <= len && nc <= 4096; nc += nc < 32 ? 1 : nc / 16) {
+        const int c = (len + nc - 1) / nc, n = (len + c - 1) / c;
+        const double w = tiles * n / slots;
+        const double cost = (w <= 1.0 ? 0.7 + 0.3 * w : 0.5 * (ceil(w) + w + 0.35)) * (c + 2.0);
+        if (cost < least * 0.999) least = cost, best.cy = c;
+    }
+    return best;
+}
+
 cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const double* v, double* v_out,
-                              const KickD& k, double deta, double phi0, cudaStream_t st)
+                              const KickD& k, double deta, double phi0, const MarchShape& shape, cudaStream_t st)
 {
     FixArgs a;
     if (!make_fix64(k, phi0, &a.f)) return cudaErrorNotSupported;
@@ -313,30 +337,15 @@ cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const
     a.k = k;
     a.deta = deta;
     a.g = g;
-    // 2D: two columns a lane share a row's bookkeeping, one makes twice the warps (us a step, two and one:
-    // 256^2 4.0 3.4, 400^2 4.6 4.3, 512^2 5.2 5.5, 1024^2 11.9 13.2, 2048^2 39 44)
-    const int cols = g.dims == 3 || g.S < ((int64_t)1 << 18) ? 1 : 2, width = fx_width(cols);
-    a.nstrips = (g.nx + width - 1) / width;
-    const int len = g.dims == 3 ? g.nz : g.ny;
+    a.nstrips = (g.nx + fx_width(shape.cols) - 1) / fx_width(shape.cols);
     a.ygroups = g.dims == 3 ? (g.ny + 4 * kFxWarps - 1) / (4 * kFxWarps) : 1;
-    // warps (2D) or blocks of them (3D) against the two planes a chunk re-reads and the iteration
-    // that fills it
-    const double tiles = (double)a.nstrips * a.ygroups / (g.dims == 3 ? 1 : kFxWarps);
-    const double slots = (double)fx_blocks(g.dims, cols) * sm_count_current();
-    double least = 1e300;
-    a.cz = len;
-    for (int nc = 1; nc <= len && nc <= 4096; nc += nc < 32 ? 1 : nc / 16) {
-        const int c = (len + nc - 1) / nc, n = (len + c - 1) / c;
-        const double w = tiles * n / slots;
-        const double cost = (w <= 1.0 ? 0.7 + 0.3 * w : 0.5 * (ceil(w) + w + 0.35)) * (c + 2.0);
-        if (cost < least * 0.999) least = cost, a.cz = c;
-    }
-    const int64_t n = (len + a.cz - 1) / a.cz;
+    a.cz = shape.cy;
+    const int64_t n = ((g.dims == 3 ? g.nz : g.ny) + a.cz - 1) / a.cz;
     const int64_t blocks = g.dims == 3 ? (int64_t)a.nstrips * a.ygroups * n
                                        : ((int64_t)a.nstrips * n + kFxWarps - 1) / kFxWarps;
     if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
-    void (*kernel)(const FixArgs) = g.dims == 3 ? k_step_fix64<3, 1> : (cols == 1 ? k_step_fix64<2, 1> : k_step_fix64<2, 2>);
-    return launch_chained(kernel, dim3((unsigned)blocks), kFxThreads, 0, st, a);
+    void (*const flat)(const FixArgs) = shape.cols == 1 ? k_step_fix64<2, 1> : k_step_fix64<2, 2>;
+    return launch_chained(g.dims == 3 ? k_step_fix64<3, 1> : flat, dim3((unsigned)blocks), kFxThreads, 0, st, a);
 }
 
 }  // namespace prs

@@ -118,14 +118,13 @@ static RunConst<R> make_rc(const double rcd[6])
 }
 
 template <typename R, bool REPRO>
-static cudaError_t step_generic_t(const Geo& g, const void* in, void* out, const void* dphi, void* dphi_out, double c1,
-                                  double c2, double cV, const double rcd[6], cudaStream_t st)
+static cudaError_t step_generic_t(const Geo& g, const void* in, void* out, const void* dphi, void* dphi_out,
+                                  const double coef[3], const double rcd[6], cudaStream_t st)
 {
     const int block = 256;
     const dim3 grid = rows_grid(g, 152 * 16);
-    StepCoef<R> k{(R)c1, (R)c2, (R)cV};
+    StepCoef<R> k{(R)coef[0], (R)coef[1], (R)coef[2]};
     RunConst<R> rc = make_rc<R>(rcd);
-    const double coef[3] = {c1, c2, cV};
     const KickD kd = kick_f64(coef, rcd);
     void (*kernel)(const R*, R*, const R*, R*, Geo, StepCoef<R>, RunConst<R>, KickD) = k_step_generic<R, REPRO, 3>;
     if (g.dims == 2) {
@@ -136,15 +135,15 @@ static cudaError_t step_generic_t(const Geo& g, const void* in, void* out, const
 }
 
 cudaError_t launch_step_generic(const Geo& g, int precision, bool repro, const void* in, void* out, const void* dphi,
-                                void* dphi_out, double c1, double c2, double cV, const double rcd[6], cudaStream_t st)
+                                void* dphi_out, const double coef[3], const double rcd[6], const MarchShape& shape,
+                                cudaStream_t st)
 {
-    if (precision == PRS_FP32) return step_generic_t<float, false>(g, in, out, dphi, dphi_out, c1, c2, cV, rcd, st);
-    if (repro) return step_generic_t<double, true>(g, in, out, dphi, dphi_out, c1, c2, cV, rcd, st);
-    const double coef[3] = {c1, c2, cV};
+    if (precision == PRS_FP32) return step_generic_t<float, false>(g, in, out, dphi, dphi_out, coef, rcd, st);
+    if (repro) return step_generic_t<double, true>(g, in, out, dphi, dphi_out, coef, rcd, st);
     const cudaError_t e = launch_step_fix64(g, (const double*)in, (double*)out, (const double*)dphi, (double*)dphi_out,
-                                            kick_f64(coef, rcd), rcd[0], rcd[5], st);
+                                            kick_f64(coef, rcd), rcd[0], rcd[5], shape, st);
     if (e != cudaErrorNotSupported) return e;
-    return step_generic_t<double, false>(g, in, out, dphi, dphi_out, c1, c2, cV, rcd, st);
+    return step_generic_t<double, false>(g, in, out, dphi, dphi_out, coef, rcd, st);
 }
 
 // ---------------------------------------------------------- state copies

@@ -122,16 +122,18 @@ KickF kick_f32(const double coef[3], const double run_const[6]);
 cudaError_t launch_init_random(const Geo& g, int precision, uint64_t seed, void* phi, void* dphi, bool zero_dphi,
                                cudaStream_t st);
 
-// One leapfrog step (nsteps_in_pass is 1) from phi_in into phi_out, dphi from dphi_in into dphi_out
-// (may be equal).
+// One leapfrog step with coefficients c1, c2, cV from phi_in into phi_out, dphi from dphi_in into dphi_out
+// (may be equal).  shape: the run's plan of one-step passes (MarchPlan::shape[1]).
+struct MarchShape;
 cudaError_t launch_step_io(const Geo& g, int precision, bool repro, const void* phi_in, void* phi_out,
-                           const void* dphi_in, void* dphi_out, const double* c1, const double* c2, const double* cV,
-                           int nsteps_in_pass, const double run_const[6], unsigned int* err, cudaStream_t st);
+                           const void* dphi_in, void* dphi_out, const double coef[3], const double run_const[6],
+                           const MarchShape& shape, unsigned int* err, cudaStream_t st);
 
-// The FP64 step (folded kick) with its force in 64-bit fixed point (prs_fix64.cu);
-// cudaErrorNotSupported where its constants or the box do not fit.
+// The FP64 step (folded kick) with its force in 64-bit fixed point (prs_fix64.cu), cut as
+// fix64_shape plans; cudaErrorNotSupported where its constants or the box do not fit.
 cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const double* v, double* v_out,
-                              const KickD& k, double deta, double phi0, cudaStream_t st);
+                              const KickD& k, double deta, double phi0, const MarchShape& shape, cudaStream_t st);
+MarchShape fix64_shape(const Geo& g);
 
 // Copy a state's fields (device to device, `bytes` each; a field that is its own source stays).
 cudaError_t launch_copy_state(const void* phi, void* phi_out, const void* dphi, void* dphi_out, size_t bytes,

@@ -5,7 +5,8 @@
 namespace prs {
 
 cudaError_t launch_step_generic(const Geo& g, int precision, bool repro, const void* in, void* out, const void* dphi,
-                                void* dphi_out, double c1, double c2, double cV, const double rcd[6], cudaStream_t st);
+                                void* dphi_out, const double coef[3], const double rcd[6], const MarchShape& shape,
+                                cudaStream_t st);
 cudaError_t launch_step_fast(const Geo& g, const float* in, float* out, const float* v, float* v_out,
                              KickF k, RunConst<float> rc, unsigned int* err, cudaStream_t st);
 
@@ -49,30 +50,20 @@ int default_fused_steps(const Geo& g, int precision, bool repro)
 }
 
 cudaError_t launch_step_io(const Geo& g, int precision, bool repro, const void* phi_in, void* phi_out,
-                           const void* dphi_in, void* dphi_out, const double* c1, const double* c2, const double* cV,
-                           int nsteps_in_pass, const double run_const[6], unsigned int* err, cudaStream_t st)
+                           const void* dphi_in, void* dphi_out, const double coef[3], const double run_const[6],
+                           const MarchShape& shape, unsigned int* err, cudaStream_t st)
 {
-    if (nsteps_in_pass != 1) return cudaErrorInvalidValue;
-    if (g.dims == 2 && precision == PRS_FP32) {
-        MarchPlan p;
-        march_plan(g, 1, &p);
-        const MarchRun r{phi_in, phi_out, dphi_in, dphi_out, {{c1[0], c2[0], cV[0]}}, run_const};
-        return launch_march2d(g, 1, p.shape[1], 1, &r, st);
-    }
+    const MarchRun r{phi_in, phi_out, dphi_in, dphi_out, {{coef[0], coef[1], coef[2]}}, run_const};
+    if (g.dims == 2 && precision == PRS_FP32) return launch_march2d(g, 1, shape, 1, &r, st);
     if (fast_step_ok(g, precision)) {
-        const double coef[3] = {c1[0], c2[0], cV[0]};
         const KickF k = kick_f32(coef, run_const);
         RunConst<float> rc{(float)run_const[0], (float)run_const[1], (float)run_const[2], (float)run_const[3],
                            (float)run_const[4], (float)run_const[5]};
         return launch_step_fast(g, (const float*)phi_in, (float*)phi_out, (const float*)dphi_in, (float*)dphi_out, k,
                                 rc, err, st);
     }
-    if (precision == PRS_FP32 && march3d_ok(g)) {
-        const MarchRun r{phi_in, phi_out, dphi_in, dphi_out, {{c1[0], c2[0], cV[0]}}, run_const};
-        return launch_march3d(g, 1, march3d_planes(g, 1, 1, nullptr), 1, &r, st);
-    }
-    return launch_step_generic(g, precision, repro, phi_in, phi_out, dphi_in, dphi_out, c1[0], c2[0], cV[0], run_const,
-                               st);
+    if (precision == PRS_FP32 && march3d_ok(g)) return launch_march3d(g, 1, shape.cy, 1, &r, st);
+    return launch_step_generic(g, precision, repro, phi_in, phi_out, dphi_in, dphi_out, coef, run_const, shape, st);
 }
 
 }  // namespace prs
