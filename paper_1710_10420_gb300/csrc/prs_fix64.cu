@@ -57,7 +57,7 @@ constexpr int fx_blocks(int dims, int cols) { return dims == 3 ? 4 : (cols == 1 
 
 // The force's constants: k1, k2 S^2 and g scaled by 2^(62-ek), 2^(66-ek), 2^(65-ek); e_base: what a
 // value's exponent field is subtracted from for its shift; e_out: exponent field of an A of 2^63; served:
-// the shift of the smallest values that serve their site and its neighbours (2: none do).
+// the shift of the smallest values that serve their site and its neighbours.
 struct Fix64 {
     i64 k1;
     u64 k2, g;
@@ -163,9 +163,9 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D, C)) k_step_fix64(cons
         pin += z == nz ? plane * (1 - (int64_t)nz) : plane;
         if (z == nz) z = 0;
     };
-    // planes z-1 (output rows), z, z+1 as integers, plane z's values, the planes' smallest shifts
+    // planes z-1 (output rows), z, z+1 as integers, the values of planes z-1 (2D) and z, the planes' smallest shifts
     i64 m[R], c[N], p[N];
-    double d[R], v[R];
+    double dm[R], d[R], v[R];
     int sm = 4096, sc = 4096, sp, down = 0;
     // bit r: output r; value r of planes z-1 and z serves its site; one of plane z next to value r or it does
     unsigned outputs = 0, bm = 0, bc = 0, wc = 0;
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D, C)) k_step_fix64(cons
     u64 k2 = a.f.k2;
     fetch();
 #pragma unroll
-    for (int r = 0; r < R; ++r) m[r] = 0, vnext[r] = 0.0, d[r] = 0.0;
+    for (int r = 0; r < R; ++r) m[r] = 0, vnext[r] = dm[r] = d[r] = 0.0;
 #pragma unroll
     for (int r = 0; r < N; ++r) c[r] = 0;
     // Plane z0 + i arrives, plane z0 + i - 1 is updated.  A warp that changes its scale goes back to the
@@ -235,19 +235,25 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D, C)) k_step_fix64(cons
                     v[r] = fma(a.k.c1, v[r], force(cc, s2, a.f, k2, a.f.e_out - down));
                     pn[r] = fma(a.deta, v[r], d[r]);
                 }
-            } else {
+            } else if (D == 2) {  // the double form, from registers
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const double left = r > 0 ? d[r - 1] : __shfl_up_sync(0xffffffffu, d[R - 1], 1);
+                    const double right = r < R - 1 ? d[r + 1] : __shfl_down_sync(0xffffffffu, d[0], 1);
+                    site_update_folded<D>(d[r], right, left, dn[r], dm[r], 0.0, 0.0, v[r], pn[r], a.k, a.deta);
+                }
+            } else {  // from memory: the planes' doubles take more registers than four blocks an SM leave
                 const int zc = z0 + i - 1, zm = zc == 0 ? nz - 1 : zc - 1, zp = zc + 1 == nz ? 0 : zc + 1;
                 const double* q = a.phi_in + (int64_t)zc * plane;
                 const double* qp = a.phi_in + (int64_t)zp * plane;
                 const double* qm = a.phi_in + (int64_t)zm * plane;
 #pragma unroll 1
                 for (int r = 0; r < rows; ++r) {
-                    const int y = D == 3 ? y0 + r : 0, x1 = D == 3 ? x : (x + r >= nx ? x + r - nx : x + r);
-                    const int64_t o = (int64_t)y * nx, up = (int64_t)(y + 1 == ny ? 0 : y + 1) * nx + x1;
-                    const int64_t dn2 = (int64_t)(y == 0 ? ny - 1 : y - 1) * nx + x1;
-                    const double xp = q[o + (x1 + 1 == nx ? 0 : x1 + 1)], xm = q[o + (x1 == 0 ? nx - 1 : x1 - 1)];
-                    const double cc = q[o + x1], yp = D == 3 ? q[up] : qp[o + x1], ym = D == 3 ? q[dn2] : qm[o + x1];
-                    const double zpv = D == 3 ? qp[o + x1] : 0.0, zmv = D == 3 ? qm[o + x1] : 0.0;
+                    const int y = y0 + r;
+                    const int64_t o = (int64_t)y * nx + x, up = (int64_t)(y + 1 == ny ? 0 : y + 1) * nx + x;
+                    const int64_t dn2 = (int64_t)(y == 0 ? ny - 1 : y - 1) * nx + x, row0 = o - x;
+                    const double xp = q[row0 + (x + 1 == nx ? 0 : x + 1)], xm = q[row0 + (x == 0 ? nx - 1 : x - 1)];
+                    const double cc = q[o], yp = q[up], ym = q[dn2], zpv = qp[o], zmv = qm[o];
                     double vv, pp;
 #pragma unroll
                     for (int u = 0; u < R; ++u) vv = u == r ? v[u] : vv;
@@ -271,7 +277,7 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D, C)) k_step_fix64(cons
         wc = bp | bp << 1 | bp >> 1 | (D == 3 ? bl | br : bl >> (R - 1) | br << (R - 1));
         bm = bc, bc = bp;
 #pragma unroll
-        for (int r = 0; r < R; ++r) m[r] = c[r + H], d[r] = dn[r];
+        for (int r = 0; r < R; ++r) m[r] = c[r + H], dm[r] = d[r], d[r] = dn[r];
 #pragma unroll
         for (int r = 0; r < N; ++r) c[r] = p[r];
     }
@@ -279,7 +285,8 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D, C)) k_step_fix64(cons
 
 }  // namespace
 
-// The constants of a step, or false where they do not fit (the double form everywhere then).
+// The constants of a step, or false where they do not fit or no integers would serve (the double form
+// everywhere then).
 static bool make_fix64(const KickD& k, double phi0, Fix64* f)
 {
     int es;  // S = 2^es >= phi0
@@ -298,7 +305,7 @@ static bool make_fix64(const KickD& k, double phi0, Fix64* f)
     f->e_out = 1023 + 63 + ek - 60 + es;
     f->served = 7;
     for (double least = ldexp(1.0, ek - 5); k.g < least && f->served > 2; least *= 0.5) --f->served;
-    return true;
+    return f->served > 2;
 }
 
 // Columns a lane owns and planes (2D: rows) a warp marches.
@@ -329,6 +336,10 @@ cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const
 {
     FixArgs a;
     if (!make_fix64(k, phi0, &a.f)) return cudaErrorNotSupported;
+    // boxes of a few rows leave most of a block's warps without any (us a step, the integers and the double
+    // form: 2000 x 3 x 2000 316 and 280, 2000 x 5 x 2000 533 and 468, 2000 x 8 x 1000
+    // 292 and 375)
+    if (g.dims == 3 && g.ny < 6) return cudaErrorNotSupported;
     if (g.dims == 3 && (int64_t)g.nx * g.ny >= ((int64_t)1 << 32)) return cudaErrorNotSupported;
     a.phi_in = in;
     a.phi_out = out;

@@ -85,7 +85,8 @@ def test_ensemble_state_copies_follow_the_callers_stream(lib, write):
 
 
 @pytest.mark.parametrize("call,nth", [("record", 1), ("wait", 1), ("wait", 2), ("wait", 3), ("launch", 2),
-                                      ("launch", 5), ("copy", 1), ("copy", 2), ("copy", 3), ("record", 2), ("record", 3), ("sync", 1)])
+                                      ("launch", 5), ("copy", 1), ("copy", 2), ("copy", 3), ("record", 2),
+                                      ("record", 3), ("sync", 1)])
 def test_nothing_is_in_flight_behind_an_ensemble_error(lib, call, nth):
     """When a CUDA call fails in the middle of prs_batch_run, every stream that was given work is waited
     for before the error is returned (the caller may free its memory, and the groups are not joined)."""
@@ -235,3 +236,17 @@ def test_noalloc_diagnostics_fill_the_gpu(lib, shape, tiles):
     assert lib.prs_measure_noalloc(p, at, at, STREAM, ctypes.byref(d)) == prs.PRS_OK
     assert [int(line[3]) >= tiles for line in _log(lib) if line[0] == "launch"] == [True]
     assert not _mallocs(lib)
+
+
+@pytest.mark.parametrize("shape,kw,integers", [((40, 5, 40), {}, False), ((40, 3, 90), {}, False),
+                                               ((40, 6, 40), {}, True), ((40, 3), {}, True),
+                                               ((64, 64), dict(dx=10.0, W0=1.2), False),
+                                               ((64, 64), dict(flags=prs.PRS_REPRO), False)])
+def test_fp64_steps_take_the_integers_where_they_serve(lib, shape, kw, integers):
+    h = _run(lib, shape, precision=prs.PRS_FP64, **kw)
+    assert lib.prs_init(h, None, None) == prs.PRS_OK
+    lib.fake_reset()
+    assert lib.prs_step(h, 2) == prs.PRS_OK
+    names = [line[2] for line in _log(lib) if line[0] == "launch"]
+    assert len(names) == 2 and all(("step_fix64" if integers else "step_generic") in name for name in names)
+    assert lib.prs_destroy(h) == prs.PRS_OK
