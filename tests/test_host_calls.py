@@ -250,3 +250,13 @@ def test_fp64_steps_take_the_integers_where_they_serve(lib, shape, kw, integers)
     names = [line[2] for line in _log(lib) if line[0] == "launch"]
     assert len(names) == 2 and all(("step_fix64" if integers else "step_generic") in name for name in names)
     assert lib.prs_destroy(h) == prs.PRS_OK
+
+
+@pytest.mark.parametrize("shape", [(100000, 3), (60000, 5)])
+def test_a_step_of_a_few_long_rows_fills_the_gpu(lib, shape):
+    h = _run(lib, shape, precision=prs.PRS_FP64, flags=prs.PRS_REPRO)
+    assert lib.prs_init(h, None, None) == prs.PRS_OK
+    lib.fake_reset()
+    assert lib.prs_step(h, 1) == prs.PRS_OK
+    assert [int(line[3]) >= 152 for line in _log(lib) if line[0] == "launch"] == [True]
+    assert lib.prs_destroy(h) == prs.PRS_OK
