@@ -33,6 +33,7 @@
 #include <math.h>
 #include <stdio.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -583,10 +584,12 @@ cudaError_t launch_observable(const prs_sim* s, const void* phi, void* grad, voi
         const Geo& g = s->g;
         const int64_t tiles = g.dims == 3 ? (int64_t)((g.nx + 31) / 32) * ((g.ny + 7) / 8) : (g.nx + 255) / 256;
         const int len = g.dims == 3 ? g.nz : g.ny;
-        // about four blocks a CTA slot (eight an SM), chunks of at least 8 planes
-        const int64_t want = (int64_t)sm_count_current() * 32;
-        int cz = (int)((len * tiles + want - 1) / want);
-        cz = cz < 8 ? 8 : (cz > len ? len : cz);
+        // about four blocks a CTA slot (eight an SM), chunks of at least 8 planes where that leaves two blocks an
+        // SM, else as many as it takes (65 x 65: a gradient of no steps 85 us, 96 with 8 rows a block)
+        const int64_t sms = sm_count_current();
+        const int64_t cut = (len * tiles + 32 * sms - 1) / (32 * sms);
+        const int64_t few = len * tiles / (2 * sms) > 1 ? len * tiles / (2 * sms) : 1;
+        const int cz = (int)std::min<int64_t>(len, std::max<int64_t>(cut, std::min<int64_t>(8, few)));
         const int64_t blocks = tiles * ((len + cz - 1) / cz);
         const unsigned obs_grid = (unsigned)(blocks < scr.max_blocks ? blocks : scr.max_blocks);
         if (g.dims == 3)
@@ -705,8 +708,8 @@ static int prs_observable_impl(prs_sim* s, int observable, double eps_smooth, do
     if (observable != PRS_OBS_GRAD_ENERGY && observable != PRS_OBS_SMOOTH_AREA) return PRS_EINVAL;
     if (observable == PRS_OBS_SMOOTH_AREA && !(eps_smooth > 0)) return PRS_EINVAL;
     if (!s->initialised) return PRS_ESTATE;
-    Scratch mem;
-    void* grad = mem.get((size_t)s->g.S * s->elem);
+    Scratch mem;  // (the second dphi buffer holds nothing between calls: an allocation takes 100 us)
+    void* grad = s->dphi_alt ? s->dphi_alt : mem.get((size_t)s->g.S * s->elem);
     if (!grad) return PRS_ENOMEM;
     DiagScratch scr = s->scr;
     cudaError_t e = launch_observable(s, s->phi[s->cur], grad, nullptr, observable, eps_smooth, scr);

@@ -260,3 +260,14 @@ def test_a_step_of_a_few_long_rows_fills_the_gpu(lib, shape):
     assert lib.prs_step(h, 1) == prs.PRS_OK
     assert [int(line[3]) >= 152 for line in _log(lib) if line[0] == "launch"] == [True]
     assert lib.prs_destroy(h) == prs.PRS_OK
+
+
+def test_an_observable_of_a_small_box_has_a_block_for_every_row(lib):
+    h = _run(lib, (65, 65))
+    assert lib.prs_init(h, None, None) == prs.PRS_OK
+    J, before = ctypes.c_double(), len(_mallocs(lib))
+    lib.fake_reset()
+    assert lib.prs_observable(h, 1, 0.1, ctypes.byref(J)) == prs.PRS_OK
+    assert [int(line[3]) >= 65 for line in _log(lib) if line[0] == "launch"] == [True]
+    assert before == 1 and not _mallocs(lib)  # its gradient goes to the idle dphi buffer
+    assert lib.prs_destroy(h) == prs.PRS_OK
