@@ -1,5 +1,5 @@
-// prs_fast.cu -- the FP32 leapfrog step (Eqs. 3-6), one step per pass, for boxes whose x side is a multiple of 128 and at most 4096 (3D: 1024): the
-// path the benchmark times.  One kernel applies Eqs. 3-5 in a single pass over
+// prs_fast.cu -- the FP32 leapfrog step (Eqs. 3-6), one step per pass, for 3D boxes whose x side is a multiple
+// of 128 and at most 1024 (the single steps that the passes of several leave over).  One kernel applies Eqs. 3-5 in a single pass over
 // HBM (read phi and dphi once, write them once: 16 B per site-update), where the
 // paper's OpenCL code ran one kernel per equation.  The tile routines (bulk-async
 // plane staging, shuffles, bounded waits) live in prs_tile.cuh; this file sizes
@@ -33,7 +33,6 @@ __global__ void __launch_bounds__(kFastThreads, 2)
 static constexpr int kItems = 4;  // float4 per thread per plane: 4096 sites per plane tile
 
 static size_t smem3d(int nx, int ty) { return tile_smem3d(nx, ty); }
-static size_t smem2d(int nx, int rb) { return tile_smem2d(nx, rb); }
 
 static constexpr size_t kFastSmemMax = 100 * 1024;
 
@@ -41,9 +40,9 @@ bool fast_step_ok(const Geo& g, int precision)
 {
     if (precision != PRS_FP32) return false;
     if (g.nx % 128 != 0 || g.nx > kItems * 1024 || (kItems * 1024) % g.nx != 0) return false;
-    const int t = kItems * 1024 / g.nx;  // rows per plane tile (3D) or per band (2D)
+    const int t = kItems * 1024 / g.nx;  // rows per plane tile
     if (g.ny % t != 0) return false;
-    return (g.dims == 3 ? smem3d(g.nx, t) : smem2d(g.nx, t)) <= kFastSmemMax;
+    return g.dims == 2 || smem3d(g.nx, t) <= kFastSmemMax;
 }
 
 // Shortest chunks the planner considers: 4 planes.  A small box must be
@@ -78,24 +77,19 @@ static int pick_chunks(int tiles, int len, int min_len, int slots)
 cudaError_t launch_step_fast(const Geo& g, const float* in, float* out, const float* v, float* v_out,
                              KickF k, RunConst<float> rc, unsigned int* err, cudaStream_t st)
 {
-    static std::atomic<unsigned long long> attr3{0};
+    if (g.dims != 3 || !fast_step_ok(g, PRS_FP32)) return cudaErrorNotSupported;
+    static std::atomic<unsigned long long> attr{0};
     const int t = kItems * 1024 / g.nx;
     const int slots = 2 * sm_count_current();  // two resident CTAs per SM
-    if (g.dims == 3) {
-        const size_t sm = smem3d(g.nx, t);
-        {
-            const cudaError_t e = smem_limit_once(attr3, (const void*)k_step3d_f32<kItems>, (int)kFastSmemMax);
-            if (e != cudaSuccess) return e;
-        }
-        if (sm > kFastSmemMax) return cudaErrorInvalidValue;
-        const int ytiles = g.ny / t;
-        int nchunks = pick_chunks(ytiles, g.nz, kMinPlanes, slots);
-        const int cz = (g.nz + nchunks - 1) / nchunks;
-        nchunks = (g.nz + cz - 1) / cz;
-        return launch_chained(k_step3d_f32<kItems>, dim3((unsigned)(ytiles * nchunks)), kFastThreads, sm, st, in, out, v,
-                              v_out, g.nx, g.ny, g.nz, t, cz, k, rc, err);
-    }
-    return cudaErrorNotSupported;
+    const size_t sm = smem3d(g.nx, t);
+    const cudaError_t e = smem_limit_once(attr, (const void*)k_step3d_f32<kItems>, (int)kFastSmemMax);
+    if (e != cudaSuccess) return e;
+    const int ytiles = g.ny / t;
+    int nchunks = pick_chunks(ytiles, g.nz, kMinPlanes, slots);
+    const int cz = (g.nz + nchunks - 1) / nchunks;
+    nchunks = (g.nz + cz - 1) / cz;
+    return launch_chained(k_step3d_f32<kItems>, dim3((unsigned)(ytiles * nchunks)), kFastThreads, sm, st, in, out, v,
+                          v_out, g.nx, g.ny, g.nz, t, cz, k, rc, err);
 }
 
 }  // namespace prs

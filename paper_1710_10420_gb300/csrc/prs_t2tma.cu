@@ -206,7 +206,7 @@ __device__ __forceinline__ bool t2_iter(const T2Maps& m, const Lane2& t, int i, 
             const float hcen = Lj[t.hc];
             float vv = V[t.hv];
             L1[t.ho] = update1(hcen, Lj[t.hx >> 16], Lj[t.hx & 0xffffu], Lj[t.hc + 4], Lj[t.hc - 4], Ln[t.hc], q.hm,
-                               vv, kick_scalar(k0), deta_only(k0), true);
+                               vv, kick_scalar(k0), deta_only(k0));
             q.hm = hcen;
         }
     }

@@ -41,10 +41,10 @@ static __device__ __noinline__ void drain4(uint64_t* bar, int from, int issued, 
     for (int i = from; i <= issued; ++i) mbar_wait(&bar[i & 3], (unsigned)(i >> 2) & 1u, err);
 }
 
-// MID: also store the state between the two steps (phi^{n+1}, dphi^{n+1/2}: level 1 at
+// Also stores the state between the two steps (phi^{n+1}, dphi^{n+1/2}: level 1 at
 // the output sites) into phi_mid, v_mid.
 // The 128 x 8 tile (160 threads, 53 KB of shared memory) runs four CTAs per SM.
-template <int ITEMS, int XW, int TY, bool MID>
+template <int ITEMS, int XW, int TY>
 __global__ void __launch_bounds__(XW == 128 && TY == 8 ? 160 : kTbThreads, XW == 128 && TY == 8 ? 4 : 2)
     k_step3d_t2(const float* __restrict__ phi_in, float* __restrict__ phi_out, const float* __restrict__ v_in,
                 float* __restrict__ v_out, float* __restrict__ phi_mid, float* __restrict__ v_mid, int nx, int ny,
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(XW == 128 && TY == 8 ? 160 : kTbThreads, XW ==
                 if (lane == 31) right = c0[4];
                 float4 pn;
                 float4 vv = lds4(V + off[q]);
-                update4(c, left, right, lds4(c0 + W), lds4(c0 - W), f0p[q], f0m[q], vv, pn, k0, rc, true);
+                update4(c, left, right, lds4(c0 + W), lds4(c0 - W), f0p[q], f0m[q], vv, pn, k0, rc);
                 *reinterpret_cast<float4*>(L1 + off[q]) = pn;
                 if (whole) {  // the wrapped end columns of the row, for level 2's x neighbours
                     if (first[q]) L1[off[q] + xw] = pn.x;
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(XW == 128 && TY == 8 ? 160 : kTbThreads, XW ==
             if (hal) {
                 const float* c0 = Pj + hoff;
                 float vv = V[hoff];
-                L1[hoff] = update1(h0c, c0[1], c0[-1], c0[W], c0[-W], h0p, h0m, vv, k0, rc, true);
+                L1[hoff] = update1(h0c, c0[1], c0[-1], c0[W], c0[-W], h0p, h0m, vv, k0, rc);
             }
         }
         if (k >= 2 && k <= zn + 1) {
@@ -208,11 +208,9 @@ __global__ void __launch_bounds__(XW == 128 && TY == 8 ? 160 : kTbThreads, XW ==
                 if (lane == 31) right = c1p[4];
                 float4 pn;
                 float4 vv = w1[q];
-                if (MID) {
-                    stg4(phi_mid + zo + go[q], c);
-                    stg4(v_mid + zo + go[q], vv);
-                }
-                update4(c, left, right, lds4(c1p + W), lds4(c1p - W), f1p[q], f1m[q], vv, pn, k1, rc, true);
+                stg4(phi_mid + zo + go[q], c);
+                stg4(v_mid + zo + go[q], vv);
+                update4(c, left, right, lds4(c1p + W), lds4(c1p - W), f1p[q], f1m[q], vv, pn, k1, rc);
                 stg4(phi_out + zo + go[q], pn);
                 stg4(v_out + zo + go[q], vv);
             }
@@ -263,17 +261,16 @@ bool plan3(const Geo& g, Tile3* t)
     return t->smem <= kTbSmemMax && t->threads >= 3 * (2 * ty + 6);
 }
 
-template <bool MID>
 cudaError_t launch3(const Geo& g, const float* phi_in, float* phi_out, const float* v_in, float* v_out, float* phi_mid,
                     float* v_mid, KickF k0, KickF k1, RunConst<float> rc, unsigned int* err, cudaStream_t st)
 {
     Tile3 t;
     if (!plan3(g, &t)) return cudaErrorInvalidValue;
     // the common tiles (256 x 8, 128 x 8) have their own instantiations with every size known
-    const void* fn = t.xw == 256 ? (t.ty == 8 ? (const void*)k_step3d_t2<kTbItems, 256, 8, MID>
-                                              : (const void*)k_step3d_t2<kTbItems, 256, 0, MID>)
-                                 : (t.ty == 8 ? (const void*)k_step3d_t2<kTbItems, 128, 8, MID>
-                                              : (const void*)k_step3d_t2<kTbItems, 128, 0, MID>);
+    const void* fn = t.xw == 256 ? (t.ty == 8 ? (const void*)k_step3d_t2<kTbItems, 256, 8>
+                                              : (const void*)k_step3d_t2<kTbItems, 256, 0>)
+                                 : (t.ty == 8 ? (const void*)k_step3d_t2<kTbItems, 128, 8>
+                                              : (const void*)k_step3d_t2<kTbItems, 128, 0>);
     static std::atomic<unsigned long long> attr[4];
     {
         const int which = t.xw == 256 ? (t.ty == 8 ? 0 : 1) : (t.ty == 8 ? 3 : 2);
@@ -302,16 +299,16 @@ cudaError_t launch3(const Geo& g, const float* phi_in, float* phi_out, const flo
     const long long blocks = (long long)tiles * ((g.nz + cz - 1) / cz);
     if (blocks > 0x7fffffffll) return cudaErrorInvalidValue;
     if (t.xw == 256 && t.ty == 8)
-        k_step3d_t2<kTbItems, 256, 8, MID><<<(unsigned)blocks, t.threads, t.smem, st>>>(
+        k_step3d_t2<kTbItems, 256, 8><<<(unsigned)blocks, t.threads, t.smem, st>>>(
             phi_in, phi_out, v_in, v_out, phi_mid, v_mid, g.nx, g.ny, g.nz, t.ty, cz, k0, k1, rc, err);
     else if (t.xw == 256)
-        k_step3d_t2<kTbItems, 256, 0, MID><<<(unsigned)blocks, t.threads, t.smem, st>>>(
+        k_step3d_t2<kTbItems, 256, 0><<<(unsigned)blocks, t.threads, t.smem, st>>>(
             phi_in, phi_out, v_in, v_out, phi_mid, v_mid, g.nx, g.ny, g.nz, t.ty, cz, k0, k1, rc, err);
     else if (t.ty == 8)
-        k_step3d_t2<kTbItems, 128, 8, MID><<<(unsigned)blocks, t.threads, t.smem, st>>>(
+        k_step3d_t2<kTbItems, 128, 8><<<(unsigned)blocks, t.threads, t.smem, st>>>(
             phi_in, phi_out, v_in, v_out, phi_mid, v_mid, g.nx, g.ny, g.nz, t.ty, cz, k0, k1, rc, err);
     else
-        k_step3d_t2<kTbItems, 128, 0, MID><<<(unsigned)blocks, t.threads, t.smem, st>>>(
+        k_step3d_t2<kTbItems, 128, 0><<<(unsigned)blocks, t.threads, t.smem, st>>>(
             phi_in, phi_out, v_in, v_out, phi_mid, v_mid, g.nx, g.ny, g.nz, t.ty, cz, k0, k1, rc, err);
     return cudaGetLastError();
 }
@@ -344,7 +341,7 @@ cudaError_t launch_step_t2(const Geo& g, const float* phi_in, float* phi_out, co
         if (e != cudaErrorNotSupported) return e;
     }
     if (!phi_mid) return cudaErrorNotSupported;
-    return launch3<true>(g, phi_in, phi_out, v_in, v_out, phi_mid, v_mid, k0, k1, rc, err, st);
+    return launch3(g, phi_in, phi_out, v_in, v_out, phi_mid, v_mid, k0, k1, rc, err, st);
 }
 
 }  // namespace prs

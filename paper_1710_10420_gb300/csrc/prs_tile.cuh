@@ -30,17 +30,17 @@ __device__ __forceinline__ float4 ldg_stream4(const float* p) { return __ldcs(re
 __device__ __forceinline__ void stg4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 
 // Eqs. 3-5 at one site, FP32: x neighbours (xp, xm), y neighbours (a, b), z neighbours
-// (e, f; 3D only).  Returns phi^{n+1}; vv becomes dphi^{n+1/2}.  The kick is KickF's
+// (e, f).  Returns phi^{n+1}; vv becomes dphi^{n+1/2}.  The kick is KickF's
 // folded form, 11 operations a site (the FP64 path keeps the canonical order of Eqs. 3-5
 // as written); every term is odd in phi, so a negated field steps to the negated field
 // exactly.  Each operation is pinned (round-to-nearest intrinsics, the three fused
 // multiply-adds explicit), so update4's packed pairs give the same bits.
 __device__ __forceinline__ float update1(float cc, float xp, float xm, float a, float b, float e, float f, float& vv,
-                                         const KickF& k, const RunConst<float>& rc, bool three_d)
+                                         const KickF& k, const RunConst<float>& rc)
 {
     float s2 = __fadd_rn(xp, xm);
     s2 = __fadd_rn(s2, __fadd_rn(a, b));
-    if (three_d) s2 = __fadd_rn(s2, __fadd_rn(e, f));
+    s2 = __fadd_rn(s2, __fadd_rn(e, f));
     const float u = __fmul_rn(cc, __fmaf_rn(-k.k2, __fmul_rn(cc, cc), k.k1));
     const float vn = __fmaf_rn(k.c1, vv, __fmaf_rn(k.g, s2, u));
     vv = vn;
@@ -51,8 +51,7 @@ __device__ __forceinline__ float update1(float cc, float xp, float xm, float a, 
 // of sites (x, y) and (z, w), one f32x2 instruction per pair and operation, except the
 // x-neighbour sums, whose operands straddle the pairs.
 __device__ __forceinline__ void update4(float4 c, float left, float right, float4 yp, float4 ym, float4 zp, float4 zm,
-                                        float4& v, float4& pn, const KickF& k, const RunConst<float>& rc,
-                                        bool three_d)
+                                        float4& v, float4& pn, const KickF& k, const RunConst<float>& rc)
 {
     const f2 kc1 = pk2(k.c1, k.c1), kg = pk2(k.g, k.g), kk1 = pk2(k.k1, k.k1), nk2 = pk2(-k.k2, -k.k2);
     const f2 dt = pk2(rc.deta, rc.deta);
@@ -60,10 +59,8 @@ __device__ __forceinline__ void update4(float4 c, float left, float right, float
     f2 s1 = pk2(__fadd_rn(c.w, c.y), __fadd_rn(right, c.z));
     s0 = add2(s0, add2(pk2(yp.x, yp.y), pk2(ym.x, ym.y)));
     s1 = add2(s1, add2(pk2(yp.z, yp.w), pk2(ym.z, ym.w)));
-    if (three_d) {
-        s0 = add2(s0, add2(pk2(zp.x, zp.y), pk2(zm.x, zm.y)));
-        s1 = add2(s1, add2(pk2(zp.z, zp.w), pk2(zm.z, zm.w)));
-    }
+    s0 = add2(s0, add2(pk2(zp.x, zp.y), pk2(zm.x, zm.y)));
+    s1 = add2(s1, add2(pk2(zp.z, zp.w), pk2(zm.z, zm.w)));
     const f2 c0 = pk2(c.x, c.y), c1 = pk2(c.z, c.w);
     const f2 u0 = mul2(c0, fma2(nk2, mul2(c0, c0), kk1));
     const f2 u1 = mul2(c1, fma2(nk2, mul2(c1, c1), kk1));
@@ -76,8 +73,7 @@ __device__ __forceinline__ void update4(float4 c, float left, float right, float
 }
 
 // update4 with the constants already packed (KickP): the same operations in the same order,
-// so the same bits.  THREE_D = false: the 2D update (zp, zm unused).
-template <bool THREE_D = true>
+// so the same bits.
 __device__ __forceinline__ void update4p(float4 c, float left, float right, float4 yp, float4 ym, float4 zp,
                                          float4 zm, float4& v, float4& pn, const KickP& k)
 {
@@ -86,10 +82,8 @@ __device__ __forceinline__ void update4p(float4 c, float left, float right, floa
     f2 s1 = pk2(__fadd_rn(c.w, c.y), __fadd_rn(right, c.z));
     s0 = add2(s0, add2(pk2(yp.x, yp.y), pk2(ym.x, ym.y)));
     s1 = add2(s1, add2(pk2(yp.z, yp.w), pk2(ym.z, ym.w)));
-    if (THREE_D) {
-        s0 = add2(s0, add2(pk2(zp.x, zp.y), pk2(zm.x, zm.y)));
-        s1 = add2(s1, add2(pk2(zp.z, zp.w), pk2(zm.z, zm.w)));
-    }
+    s0 = add2(s0, add2(pk2(zp.x, zp.y), pk2(zm.x, zm.y)));
+    s1 = add2(s1, add2(pk2(zp.z, zp.w), pk2(zm.z, zm.w)));
     const f2 c0 = pk2(c.x, c.y), c1 = pk2(c.z, c.w);
     const f2 u0 = mul2(c0, fma2(nk2, mul2(c0, c0), kk1));
     const f2 u1 = mul2(c1, fma2(nk2, mul2(c1, c1), kk1));
@@ -182,7 +176,6 @@ struct Tile3D {
 };
 
 __host__ __device__ constexpr size_t tile_smem3d(int nx, int ty) { return 128 + 4 * (size_t)(ty + 2) * nx * sizeof(float); }
-__host__ __device__ constexpr size_t tile_smem2d(int nx, int rb) { return 128 + 4 * (size_t)rb * nx * sizeof(float); }
 
 // One 3D tile: Eqs. 3-5 (phi_in -> phi_out, v_in -> v_out).
 template <int ITEMS>
@@ -275,7 +268,7 @@ __device__ __forceinline__ bool tile3d(const Tile3D& T, const KickF& k, const Ru
             float left, right;
             x_halo(pc + r * nx, col[j], nq, nx, lane, c, left, right);
             float4 pn;
-            update4(c, left, right, yp, ym, zp, zm, vc[j], pn, k, rc, true);
+            update4(c, left, right, yp, ym, zp, zm, vc[j], pn, k, rc);
             stg4(po + off, pn);
             stg4(vo + off, vc[j]);
         }
