@@ -2,6 +2,7 @@
 // host's, copies happen at once, kernels do not run.  Every call that orders or changes work is written
 // to a log ("<call> <stream> ..."), and the n-th call of a name can be made to fail.
 #include <cuda_runtime_api.h>
+#include <sys/mman.h>
 
 #include <cstdarg>
 #include <cstdio>
@@ -14,6 +15,7 @@ namespace {
 
 std::string g_log;
 std::map<const void*, std::string> g_names;  // host stub -> kernel
+std::map<void*, size_t> g_sizes;              // allocations
 std::string g_fail_call;
 int g_fail_nth = 0;
 cudaError_t g_fail_code = cudaSuccess, g_last = cudaSuccess;
@@ -115,9 +117,10 @@ static cudaError_t get(const char* call, void** p, size_t n)
     const cudaError_t e = done(call);
     if (e != cudaSuccess) return e;
     if (g_limit && n > g_limit) return g_last = cudaErrorMemoryAllocation;
-    *p = aligned_alloc(4096, (n + 4095) / 4096 * 4096);
-    if (!*p) return g_last = cudaErrorMemoryAllocation;
-    memset(*p, 0, n);
+    // zeros, and no memory for what nothing touches (fields of production size)
+    *p = mmap(nullptr, n, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
+    if (*p == MAP_FAILED) return g_last = cudaErrorMemoryAllocation;
+    g_sizes[*p] = n;
     say("%s %zu %zu", call, n, id(*p));
     return cudaSuccess;
 }
@@ -126,10 +129,13 @@ cudaError_t cudaMallocHost(void** p, size_t n) { return get("mallochost", p, n);
 cudaError_t cudaFree(void* p)
 {
     if (p) say("free");
-    free(p);
+    return cudaFreeHost(p);
+}
+cudaError_t cudaFreeHost(void* p)
+{
+    if (p) munmap(p, g_sizes[p]), g_sizes.erase(p);
     return cudaSuccess;
 }
-cudaError_t cudaFreeHost(void* p) { return free(p), cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t st)
 {
     const cudaError_t e = done("copy");

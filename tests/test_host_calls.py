@@ -271,3 +271,22 @@ def test_an_observable_of_a_small_box_has_a_block_for_every_row(lib):
     assert [int(line[3]) >= 65 for line in _log(lib) if line[0] == "launch"] == [True]
     assert before == 1 and not _mallocs(lib)  # its gradient goes to the idle dphi buffer
     assert lib.prs_destroy(h) == prs.PRS_OK
+
+
+def test_the_benchmark_counts_the_passes_the_library_takes(lib):
+    """bench.py divides the time of an interval's steps by passes of three (3D) and five (2D) steps."""
+    import bench
+
+    for shape, calls in (((1024, 1024, 1024), [(18, 3, 6), (2, 2, 1)]), ((512, 512, 512), [(18, 3, 6), (2, 2, 1)]),
+                         ((4096, 4096), [(20, 5, 4)])):
+        h = _run(lib, shape)
+        assert lib.prs_init(h, None, None) == prs.PRS_OK  # memory that nothing touches
+        tb = 3 if len(shape) == 3 else 5
+        assert bench.interval_calls(21, tb)[:2] == (calls[0][0], calls[1][0] if len(calls) > 1 else 0)
+        for steps, t, passes in calls:
+            lib.fake_reset()
+            assert lib.prs_step(h, steps) == prs.PRS_OK
+            names = [line[2] for line in _log(lib) if line[0] == "launch"]
+            assert len(names) == passes, (shape, names)
+            assert all(f"Fold32ELi{t}E" in n or (t == 2 and "t2tma" in n) for n in names), names
+        assert lib.prs_destroy(h) == prs.PRS_OK
