@@ -5,8 +5,9 @@
 // and lphi one by one (250^3: 304 us a step; here 84.  128 x 104 x 200: 84 and 19).  Here a warp owns 64
 // columns (a pair a lane) of four rows and marches along z as the forward march does (prs_march3d.cuh):
 // lt's z neighbours wait in registers, its y neighbours are the warp's other rows, x neighbours come by
-// shuffle, and everything an iteration uses comes in one slot of a ring each lane fills ahead for itself.  The dJ/dalpha term takes phi (L lt) for
-// lt (L phi), as the staged sweep does, so phi is read at the site only.
+// shuffle, and everything an iteration uses comes in one slot of a ring each lane fills ahead for itself.
+// The dJ/dalpha term takes phi (L lt) for lt (L phi), as the staged sweep does, so phi is read at the
+// site only.
 //
 // (Two steps a pass, 32 bytes a site instead of 48 with lt and lphi between them in registers, took 219
 // us a pass at 256^3 against 128 for two staged steps: 32 rows staged for four, eight warps an SM.)

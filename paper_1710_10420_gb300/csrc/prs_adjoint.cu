@@ -582,6 +582,7 @@ cudaError_t launch_observable(const prs_sim* s, const void* phi, void* grad, voi
         const float gscale = area ? (float)(0.5 * area_scale / eps) : (float)s->rc[1];
         const float inv_eps = area ? (float)(1.0 / eps) : 0.0f;
         const Geo& g = s->g;
+        const float deta = (float)s->p.deta;
         const int64_t tiles = g.dims == 3 ? (int64_t)((g.nx + 31) / 32) * ((g.ny + 7) / 8) : (g.nx + 255) / 256;
         const int len = g.dims == 3 ? g.nz : g.ny;
         // about four blocks a CTA slot (eight an SM), chunks of at least 8 planes where that leaves two blocks an
@@ -594,10 +595,10 @@ cudaError_t launch_observable(const prs_sim* s, const void* phi, void* grad, voi
         const unsigned obs_grid = (unsigned)(blocks < scr.max_blocks ? blocks : scr.max_blocks);
         if (g.dims == 3)
             k_observable_f32<3><<<obs_grid, 256, 0, s->stream>>>((const float*)phi, (float*)grad, (float*)grad_deta, g,
-                                                                 obs, inv_eps, jscale, gscale, (float)s->p.deta, cz, scr);
+                                                                 obs, inv_eps, jscale, gscale, deta, cz, scr);
         else
             k_observable_f32<2><<<obs_grid, 256, 0, s->stream>>>((const float*)phi, (float*)grad, (float*)grad_deta, g,
-                                                                 obs, inv_eps, jscale, gscale, (float)s->p.deta, cz, scr);
+                                                                 obs, inv_eps, jscale, gscale, deta, cz, scr);
     } else {
         if (s->g.dims == 3) PRS_OBS_LAUNCH(double, 3); else PRS_OBS_LAUNCH(double, 2);
     }

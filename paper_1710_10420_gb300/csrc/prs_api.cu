@@ -475,12 +475,13 @@ static void step_plan(const prs_sim* s, const MarchPlan* march, int64_t nsteps, 
     // Multi-step passes read dphi across sites, so they write it to a second buffer.  A call runs its
     // passes the longest first, single steps last: FP32 without a tblock what march_counts plans; else
     // with T = tblock = 3, nsteps / 3 triples and a pair or a single step for the remainder; with T = 2,
-    // pairs, and for an odd count a single step.  After an odd number of multi-step passes dphi sits in the second buffer.  A run whose
-    // buffers the library owns (no PRS_DEBUG guard bands) then swaps the roles of its two dphi
-    // buffers.  A run with bound buffers keeps dphi in the bound buffer at the end of every call: the
-    // first single step after an odd number of multi-step passes reads dphi in the second buffer and
-    // writes the bound one; with no single step to do it, the last pair runs as two single steps, else
-    // the last triple as a pair and a single step.  Single steps otherwise update dphi in place.
+    // pairs, and for an odd count a single step.  After an odd number of multi-step passes dphi sits in the
+    // second buffer.  A run whose buffers the library owns (no PRS_DEBUG guard bands) then swaps the
+    // roles of its two dphi buffers.  A run with bound buffers keeps dphi in the bound buffer at the end
+    // of every call: the first single step after an odd number of multi-step passes reads dphi in the
+    // second buffer and writes the bound one; with no single step to do it, the last pair runs as two
+    // single steps, else the last triple as a pair and a single step.  Single steps otherwise update dphi
+    // in place.
     const bool swap_ok = s->owned && (s->p.flags & PRS_DEBUG) == 0;
     for (int t = 0; t <= kMarchMaxT; ++t) cnt[t] = 0;
     // no second buffer (no room at prs_init), or planes beyond the march's offsets
@@ -662,7 +663,8 @@ int prs::step_runs(prs_sim* const* runs, int nruns, int64_t nsteps)
         if (!cfl_ok_over(s->p, s->n, nsteps)) return PRS_EINVAL;
         const Geo &g = s->g, &g0 = runs[0]->g;
         together = together && march_plans(s) && g.dims == g0.dims && g.nx == g0.nx && g.ny == g0.ny &&
-                   g.nz == g0.nz && march_packed(g) && (g.dims == 2 || march3d_ok(g)) && s->stream == runs[0]->stream && s->dphi_alt && s->owned == runs[0]->owned &&
+                   g.nz == g0.nz && march_packed(g) && (g.dims == 2 || march3d_ok(g)) &&
+                   s->stream == runs[0]->stream && s->dphi_alt && s->owned == runs[0]->owned &&
                    (s->p.flags & PRS_DEBUG) == 0;
     }
     if (!together) {
@@ -784,7 +786,8 @@ extern "C" int prs_measure_ex(prs_sim* s, prs_diag* out)
     return debug_after(s, prs_measure_ex_impl(s, out), "prs_measure_ex", false);
 }
 
-extern "C" int prs_measure(prs_sim* s, double* area_per_volume, double* gamma_v, int64_t* n_links, int64_t* n_wall_sites)
+extern "C" int prs_measure(prs_sim* s, double* area_per_volume, double* gamma_v, int64_t* n_links,
+                           int64_t* n_wall_sites)
 {
     const int rc = prs_measure_impl(s, area_per_volume, gamma_v, n_links, n_wall_sites);
     return debug_after(s, rc, "prs_measure", false);

@@ -1,7 +1,7 @@
 // prs_fast.cu -- the FP32 leapfrog step (Eqs. 3-6), one step per pass, for 3D boxes whose x side is a multiple
-// of 128 and at most 1024 (the single steps that the passes of several leave over).  One kernel applies Eqs. 3-5 in a single pass over
-// HBM (read phi and dphi once, write them once: 16 B per site-update), where the
-// paper's OpenCL code ran one kernel per equation.  The tile routines (bulk-async
+// of 128 and at most 1024 (the single steps that the passes of several leave over).  One kernel
+// applies Eqs. 3-5 in a single pass over HBM (read phi and dphi once, write them once: 16 B per
+// site-update), where the paper's OpenCL code ran one kernel per equation.  The tile routines (bulk-async
 // plane staging, shuffles, bounded waits) live in prs_tile.cuh; this file sizes
 // the grids: one CTA per tile, two resident per SM.
 #include <cuda_runtime.h>

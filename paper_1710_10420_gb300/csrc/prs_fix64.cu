@@ -27,7 +27,8 @@
 // Measured (us a step of a network of walls ten sites wide; the double form): 256^3 194 (356), 512^3 1476
 // (2805), 128^3 32 (52), 2048^2 44 (74), 128^2 3.4 (4.3: the launch).  Wide walls have more sites without a
 // large neighbour: 40 sites wide, 256^3 takes 277.  Before the precision of small values was kept (128-bit
-// sums, the vote): 161 at 256^3, 39 at 2048^2.
+// sums, the vote): 161 at 256^3, 39 at 2048^2.  What sets the pace now: 250 warp instructions for 32 sites at
+// 0.59 of the issue slots, with the 16 warps an SM that 128 registers leave.
 //
 // A warp owns 32 columns (30 outputs) of four rows, in 2D 32 or 64 columns (one or two a lane) of one row,
 // and marches along z (2D: y): a value is converted once where it enters, its z neighbours wait in
@@ -228,8 +229,10 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D, C)) k_step_fix64(cons
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     const i64 cc = c[r + H];
-                    const i64 left = D == 2 && r > 0 ? c[r - 1] : __shfl_up_sync(0xffffffffu, c[D == 2 ? R - 1 : r + H], 1);
-                    const i64 right = D == 2 && r < R - 1 ? c[r + 1] : __shfl_down_sync(0xffffffffu, c[D == 2 ? 0 : r + H], 1);
+                    const i64 left =
+                        D == 2 && r > 0 ? c[r - 1] : __shfl_up_sync(0xffffffffu, c[D == 2 ? R - 1 : r + H], 1);
+                    const i64 right =
+                        D == 2 && r < R - 1 ? c[r + 1] : __shfl_down_sync(0xffffffffu, c[D == 2 ? 0 : r + H], 1);
                     i64 s2 = (left + right) + (m[r] + p[r + H]);
                     if (D == 3) s2 += c[r] + c[r + 2 * H];
                     v[r] = fma(a.k.c1, v[r], force(cc, s2, a.f, k2, a.f.e_out - down));

@@ -9,10 +9,11 @@
 // beyond the element's.  Each level loses a column and a
 // row on every side, so a strip yields 2 HX columns less than its width and a chunk re-reads 2T rows.
 //
-// What bounds it: instruction issue (6 to 8 instructions a site-update in FP32, against about 16
-// when each level's rows pass through shared memory) and, on boxes larger than L2, HBM at 16 B per
-// T site-updates.  Both sides of a row are recomputed instead of exchanged, which is what lets warps
-// run without waiting for one another.  phi and dphi are read across sites, so both go out of place.
+// What bounds it: the latency of an iteration's chain on small boxes, HBM at 16 B per T site-updates on
+// boxes larger than L2 and between the two instruction issue (6 to 8 instructions a site-update in
+// FP32, against about 16 when each level's rows pass through shared memory).  Both sides of a row are
+// recomputed instead of exchanged, which is what lets warps run without waiting for one another.  phi
+// and dphi are read across sites, so both go out of place.
 //
 // Measured (an output interval of 10 steps and the diagnostics, us; with the one- to three-step passes
 // over rows in shared memory, or one thread a site on ragged boxes, that this replaced): 256^2 42 (82),

@@ -8,8 +8,9 @@ namespace prs {
 constexpr int kMarchMaxT = 6;      // steps per pass
 constexpr int kMarchMaxRuns = 16;  // runs of one box per launch
 
-// Whether an FP32 box steps by the folded kick of the staged passes (the boxes they take), else by the
-// generic step's arithmetic, whose rounding errors are a little smaller.
+// Whether an FP32 box steps by the folded kick of the staged passes (the boxes of the one-step tiles, and
+// those of 2^24 sites and more, in 2D also smaller ones, of the two- and three-step passes), else by
+// the generic step's arithmetic, whose rounding errors are a little smaller.
 bool march_packed(const Geo& g);
 
 // The state of one FP32 run and the steps of a pass over it: coefficients (c1, c2, cV) of each

@@ -8,13 +8,15 @@
 // fills ahead for itself.  The warps of a block own neighbouring rows, so that the halo rows of one
 // are another's in L1.
 //
-// What bounds it: instruction issue.  The two outer rows of each level are computed twice (T = 2:
-// 1.25 updates an output and step, and 64/60 for the columns), which is what lets a warp run without
-// waiting for its neighbours at a barrier, on boxes whose rows have no alignment for tensor copies.
+// What bounds it: latency, with the 8 (T = 3) or 12 (T = 2) warps an SM that the registers leave, which keep
+// 0.4 to 0.6 of the issue slots busy.  The outer rows of each level are computed twice (T = 2: 1.25
+// updates an output and step and 64/60 for the columns; T = 3: 1.5 and 64/56), which is what lets a warp
+// run without waiting for its neighbours at a barrier, on boxes whose rows have no alignment for
+// tensor copies.
 //
-// Measured: 512^3, T = 3, 522 us a pass, 382 M warp instructions at 0.59 of the issue slots, 2.16 GB
+// Measured: 512^3, T = 3, 522 us a pass, 382 M warp instructions at 0.60 of the issue slots, 2.16 GB
 // of DRAM traffic for 2.15 GB of fields in and out; 1024^3 1.21 ms a step (pairs of staged tiles 1.37);
-// 450 x 421 x 380 128 us a step (one thread a site: 571); 128^3 6.7 us a step (staged, short chunks: 9.6).
+// 450 x 421 x 380 112 us a step (one thread a site: 571); 128^3 6.7 us a step (staged, short chunks: 9.6).
 #pragma once
 
 #include "prs_march2d.cuh"

@@ -40,8 +40,9 @@ __device__ __forceinline__ void acc_warp_reduce(DiagAcc& a)
 
 // Every thread of the block calls this once with its own sums: block bid of the nblocks
 // that reduce into scr; their total lands in *scr.result and the counter is reset for the
-// next launch.  sums: shared memory for blockDim.x pairs, free for use.  The last block reads the partials with all its threads (one warp reading 456
-// of them took about 8 us of a small box's diagnostics).
+// next launch.  sums: shared memory for blockDim.x pairs, free for use.  The last block reads the
+// partials with all its threads (one warp reading 456 of them took about 8 us of a small box's
+// diagnostics).
 __device__ __forceinline__ void block_reduce_and_finish_at(DiagAcc a, const DiagScratch& scr, unsigned int bid,
                                                            unsigned int nblocks, double2* sums)
 {

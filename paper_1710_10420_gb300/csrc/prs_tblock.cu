@@ -233,9 +233,9 @@ constexpr size_t kTbSmemMax = 160 * 1024;
 // Tile of a 3D two-step pass: xw columns (128 for x sides up to 256, four CTAs per SM;
 // else the widest 128-multiple up to 256 that divides nx, two CTAs per SM: several CTAs
 // per SM hide each other's barrier waits; measured 38.2 against 41.2 us per step at
-// 256^3 for 128-column tiles, 1.72 against 1.67 ms at 1024^3) by ty rows (the largest divisor of ny whose level-1 plane takes at most
-// kTbItems float4 per thread of a kTbThreads CTA; a sliced tile has one halo lane of
-// warp 0 per level-1 row and side).
+// 256^3 for 128-column tiles, 1.72 against 1.67 ms at 1024^3) by ty rows (the largest divisor of
+// ny whose level-1 plane takes at most kTbItems float4 per thread of a kTbThreads CTA; a sliced
+// tile has one halo lane of warp 0 per level-1 row and side).
 struct Tile3 {
     int xw, ty, threads;
     size_t smem;
