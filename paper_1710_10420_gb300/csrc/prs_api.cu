@@ -618,8 +618,10 @@ static void diag_from_status(const prs_sim* s, int64_t step, prs_diag* d)
 
 // The diagnostics of the current state, then nsteps steps queued behind them while the result
 // travels to the host.  (A one-step pass that also evaluated the diagnostics of the state it read
-// took 4.6 ms at 1024^3, against 3.5 ms for the diagnostics alone and 1.4 for the same step inside
-// a multi-step pass; on small and 2D boxes the two ways take the same time.)
+// took 4.6 ms at 1024^3, against 3.5 ms for the diagnostics alone and 1.4 for the same step inside a
+// multi-step pass: it paid for intervals of one or two steps on large aligned 3D boxes, by 3 to 12%.)
+// Runs whose diagnostics are the IEEE ones first hear of earlier passes whose bounded waits gave up: their
+// state is not stepped on.
 static int prs_step_measure_impl(prs_sim* s, int64_t nsteps, prs_diag* out)
 {
     if (!s || !out || nsteps < 0) return PRS_EINVAL;
