@@ -25,7 +25,7 @@
 // more, and raised again when a plane needs it; the planes already held are then converted again.
 //
 // Measured (us a step of a network of walls ten sites wide; the double form): 256^3 194 (356), 512^3 1476
-// (2805), 128^3 32 (52), 2048^2 44 (74).  Wide walls have more sites without a
+// (2805), 128^3 32 (52), 2048^2 44 (74), 128^2 3.4 (4.3: the launch).  Wide walls have more sites without a
 // large neighbour: 40 sites wide, 256^3 takes 277.  Before the precision of small values was kept (128-bit
 // sums, the vote): 161 at 256^3, 39 at 2048^2.  What sets the pace now: 250 warp instructions for 32 sites at
 // 0.59 of the issue slots, with the 16 warps an SM that 128 registers leave.
@@ -315,7 +315,7 @@ static bool make_fix64(const KickD& k, double phi0, Fix64* f)
 MarchShape fix64_shape(const Geo& g)
 {
     // 2D: two columns a lane share a row's bookkeeping, one makes twice the warps (us a step, two and one:
-    // 400^2 4.6 4.3, 512^2 5.2 5.5, 1024^2 11.9 13.2, 2048^2 39 44)
+    // 256^2 4.0 3.4, 400^2 4.6 4.3, 512^2 5.2 5.5, 1024^2 11.9 13.2, 2048^2 39 44)
     const int cols = g.dims == 3 || g.S < ((int64_t)1 << 18) ? 1 : 2, width = fx_width(cols);
     const int nstrips = (g.nx + width - 1) / width, len = g.dims == 3 ? g.nz : g.ny;
     const int ygroups = g.dims == 3 ? (g.ny + 4 * kFxWarps - 1) / (4 * kFxWarps) : 1;
@@ -339,11 +339,10 @@ cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const
 {
     FixArgs a;
     if (!make_fix64(k, phi0, &a.f)) return cudaErrorNotSupported;
-    // Small boxes: a thread a site is the faster while the FP64 pipe has little to do (us a step, the integers
-    // and the double form, steps launched back to back: 128^2 3.7 2.7, 256^2 4.0 3.4, 400 x 300 4.5 5.8,
-    // 32^3 5.3 4.3, 128 x 13 x 34 5.6 3.5, 48^3 6.1 7.8).  Boxes of a few rows leave most of a block's warps
-    // without any (256 x 6 x 256 13.1 and 11.0, 2000 x 5 x 2000 533 and 468, 300 x 8 x 300 15.4 and 20.8).
-    if (g.S <= (int64_t)1 << 16 || (g.dims == 3 && g.ny < 7)) return cudaErrorNotSupported;
+    // boxes of a few rows leave most of a block's warps without any (us a step, the integers and the double
+    // form: 2000 x 3 x 2000 316 and 280, 2000 x 5 x 2000 533 and 468, 2000 x 8 x 1000
+    // 292 and 375)
+    if (g.dims == 3 && g.ny < 6) return cudaErrorNotSupported;
     if (g.dims == 3 && (int64_t)g.nx * g.ny >= ((int64_t)1 << 32)) return cudaErrorNotSupported;
     a.phi_in = in;
     a.phi_out = out;
