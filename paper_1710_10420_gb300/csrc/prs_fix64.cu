@@ -290,8 +290,9 @@ __global__ void __launch_bounds__(kFxThreads, fx_blocks(D, C)) k_step_fix64(cons
 
 // The constants of a step, or false where they do not fit or no integers would serve (the double form
 // everywhere then).
-static bool make_fix64(const KickD& k, double phi0, Fix64* f)
+static bool make_fix64(const KickD& k, const double coef[3], const double run_const[6], Fix64* f)
 {
+    const double phi0 = run_const[5];
     int es;  // S = 2^es >= phi0
     const double fr = frexp(phi0, &es);
     if (fr == 0.5) --es;
@@ -301,7 +302,11 @@ static bool make_fix64(const KickD& k, double phi0, Fix64* f)
     int ek;
     frexp(bound, &ek);  // bound < 2^ek
     if (ek < -400 || ek > 400 || es < -400 || es > 400) return false;
-    f->k1 = (i64)llrint(ldexp(k.k1, 62 - ek));
+    // k1 = c2 cV - 2D c2/dx^2 from its unrounded parts: as a double it is off by up to 2^-55 (at sides of one),
+    // which every step would repeat, and which a 63-bit constant need not carry
+    const double h = coef[1] * coef[2], h_lo = fma(coef[1], coef[2], -h), g_lo = fma(coef[1], run_const[1], -k.g);
+    const auto fixed = [&](double x) { return (i64)llrint(ldexp(x, 62 - ek)); };
+    f->k1 = fixed(h) + fixed(h_lo) - (i64)run_const[3] * (fixed(k.g) + fixed(g_lo));
     f->k2 = (u64)llrint(ldexp(k2s, 65 - ek)) << 1;
     f->g = (u64)llrint(ldexp(k.g, 65 - ek));
     f->e_base = 1026 + es;
@@ -335,10 +340,12 @@ MarchShape fix64_shape(const Geo& g)
 }
 
 cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const double* v, double* v_out,
-                              const KickD& k, double deta, double phi0, const MarchShape& shape, cudaStream_t st)
+                              const double coef[3], const double run_const[6], const MarchShape& shape,
+                              cudaStream_t st)
 {
+    const KickD k = kick_f64(coef, run_const);
     FixArgs a;
-    if (!make_fix64(k, phi0, &a.f)) return cudaErrorNotSupported;
+    if (!make_fix64(k, coef, run_const, &a.f)) return cudaErrorNotSupported;
     // boxes of a few rows leave most of a block's warps without any (us a step, the integers and the double
     // form: 2000 x 3 x 2000 316 and 280, 2000 x 5 x 2000 533 and 468, 2000 x 8 x 1000
     // 292 and 375)
@@ -349,7 +356,7 @@ cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const
     a.v_in = v;
     a.v_out = v_out;
     a.k = k;
-    a.deta = deta;
+    a.deta = run_const[0];
     a.g = g;
     a.nstrips = (g.nx + fx_width(shape.cols) - 1) / fx_width(shape.cols);
     a.ygroups = g.dims == 3 ? (g.ny + 4 * kFxWarps - 1) / (4 * kFxWarps) : 1;

@@ -143,7 +143,7 @@ cudaError_t launch_step_generic(const Geo& g, int precision, bool repro, const v
     if (precision == PRS_FP32) return step_generic_t<float, false>(g, in, out, dphi, dphi_out, coef, rcd, st);
     if (repro) return step_generic_t<double, true>(g, in, out, dphi, dphi_out, coef, rcd, st);
     const cudaError_t e = launch_step_fix64(g, (const double*)in, (double*)out, (const double*)dphi, (double*)dphi_out,
-                                            kick_f64(coef, rcd), rcd[0], rcd[5], shape, st);
+                                            coef, rcd, shape, st);
     if (e != cudaErrorNotSupported) return e;
     return step_generic_t<double, false>(g, in, out, dphi, dphi_out, coef, rcd, st);
 }

@@ -132,7 +132,8 @@ cudaError_t launch_step_io(const Geo& g, int precision, bool repro, const void* 
 // The FP64 step (folded kick) with its force in 64-bit fixed point (prs_fix64.cu), cut as
 // fix64_shape plans; cudaErrorNotSupported where its constants or the box do not fit.
 cudaError_t launch_step_fix64(const Geo& g, const double* in, double* out, const double* v, double* v_out,
-                              const KickD& k, double deta, double phi0, const MarchShape& shape, cudaStream_t st);
+                              const double coef[3], const double run_const[6], const MarchShape& shape,
+                              cudaStream_t st);
 MarchShape fix64_shape(const Geo& g);
 
 // Copy a state's fields (device to device, `bytes` each; a field that is its own source stays).
