@@ -176,7 +176,7 @@ def test_small_boxes_take_no_staged_pairs(lib, shape, steps):
 
 
 def _mallocs(lib):
-    return [int(line[1]) for line in _log(lib) if line[0] == "malloc"]
+    return [int(line[1]) for line in _log(lib) if line[0] in ("malloc", "poolmalloc")]
 
 
 @pytest.mark.parametrize("shape,kw", [((128, 128, 128), {}), ((250, 170), {}), ((256, 256), {}), ((45, 42, 38), {}),
@@ -290,3 +290,24 @@ def test_the_benchmark_counts_the_passes_the_library_takes(lib):
             assert len(names) == passes, (shape, names)
             assert all(f"Fold32ELi{t}E" in n or (t == 2 and "t2tma" in n) for n in names), names
         assert lib.prs_destroy(h) == prs.PRS_OK
+
+
+def test_small_bound_runs_share_a_pool_that_the_last_one_gives_back(lib):
+    bufs = [np.zeros((64, 64), np.float32) for _ in range(3)]
+
+    def bind(shape, **kw):
+        h = _run(lib, shape, **kw)
+        assert lib.prs_bind(h, *[b.ctypes.data + -b.ctypes.data % 16 for b in bufs]) == prs.PRS_OK
+        return h
+
+    lone, a, b, large = bind((64, 60)), bind((64, 60)), bind((100, 90, 80)), bind((512, 512, 40))
+    assert [line[0] for line in _log(lib) if line[0] in ("malloc", "poolmalloc")] == \
+        ["malloc", "poolmalloc", "poolmalloc", "malloc"]  # alone, small, small, 42 MB
+    for h, trims in ((a, 0), (lone, 0), (large, 0), (b, 1)):
+        assert lib.prs_destroy(h) == prs.PRS_OK
+        assert len([line for line in _log(lib) if line[0] == "trim"]) == trims
+    lib.fake_reset()
+    lib.fake_fail(b"poolmalloc", 1, 2)  # no room in the pool: the driver's memory
+    for h in (bind((64, 60)), bind((64, 60))):
+        assert lib.prs_destroy(h) == prs.PRS_OK
+    assert [line[0] for line in _log(lib) if line[0] in ("malloc", "poolmalloc")] == ["malloc", "malloc"]
