@@ -265,15 +265,13 @@ static int run_tblock(const prs_sim* s)
 // Whether the run takes passes of several steps, which need a second dphi buffer.
 static bool wants_alt(const prs_sim* s) { return run_tblock(s) >= 2 || march_plans(s); }
 
-// One allocation of `fields` fields, the second dphi buffer and the diagnostics' scratch; without the
-// buffer where it does not fit.  (Beyond 2 MB an allocation takes 30 to 100 us, and as long to free: a run of
-// 128^3 with its own fields 493 us from creation to release, with an allocation each 812; bound 498 and 630.)
-static int alloc_run(prs_sim* s, int fields)
+// stream: the run's, or null while it is captured.
+static int alloc_run_on(prs_sim* s, int fields, const cudaStream_t* stream)
 {
     const size_t fs = ((size_t)s->g.S * s->elem + 511) & ~(size_t)511;
     const size_t scratch = sizeof(DiagAcc) * kMeasureBlocks + sizeof(DevStatus);
     bool alt = wants_alt(s);
-    void* m = fields ? nullptr : pool_alloc(fs * (alt ? 1 : 0) + scratch, s->stream);
+    void* m = fields || !stream ? nullptr : pool_alloc(fs * (alt ? 1 : 0) + scratch, *stream);
     s->pooled = m != nullptr;
     if (!m && cudaMalloc(&m, fs * (size_t)(fields + (alt ? 1 : 0)) + scratch) != cudaSuccess) {
         cudaGetLastError();
@@ -285,7 +283,8 @@ static int alloc_run(prs_sim* s, int fields)
         }
     }
     char* c = (char*)m + fs * (size_t)(fields + (alt ? 1 : 0));
-    const cudaError_t e = cudaMemsetAsync(c, 0, scratch, s->stream);
+    cudaError_t e = cudaMemsetAsync(c, 0, scratch, stream ? *stream : cudaStreamPerThread);
+    if (e == cudaSuccess && !stream) e = cudaStreamSynchronize(cudaStreamPerThread);
     s->mem = m;
     if (e != cudaSuccess) {
         free_run(s);
@@ -302,6 +301,22 @@ static int alloc_run(prs_sim* s, int fields)
         s->dphi = (char*)m + 2 * fs;
     }
     return PRS_OK;
+}
+
+// One allocation of `fields` fields, the second dphi buffer and the diagnostics' scratch; without the
+// buffer where it does not fit.  (Beyond 2 MB an allocation takes 30 to 100 us, and as long to free: a run of
+// 128^3 with its own fields 493 us from creation to release, with an allocation each 812; bound 498 and 630.)
+// Neither it nor the scratch's first contents become part of a graph that the run's stream is captured into.
+static int alloc_run(prs_sim* s, int fields)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s->stream, &status) != cudaSuccess) cudaGetLastError();
+    const bool capturing = status != cudaStreamCaptureStatusNone;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (capturing) cudaThreadExchangeStreamCaptureMode(&mode);
+    const int rc = alloc_run_on(s, fields, capturing ? nullptr : &s->stream);
+    if (capturing) cudaThreadExchangeStreamCaptureMode(&mode);
+    return rc;
 }
 
 extern "C" int prs_bind(prs_sim* s, void* d_phi_a, void* d_phi_b, void* d_dphi)

@@ -184,6 +184,11 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned)
     return e;
 }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s)
+{
+    return *s = cudaStreamCaptureStatusNone, cudaSuccess;
+}
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode*) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t st)
 {
     const cudaError_t e = done("sync");
