@@ -27,8 +27,8 @@
  *   - A handle must not be used from two host threads at once.  Calls on different
  *     handles may run concurrently from different host threads (each run has its
  *     own stream; the library keeps no other unsynchronised state), which lets one
- *     run's host transfers overlap another run's kernels.  (What they share is a pool of
- *     device memory for small runs, at most 64 MB of it kept while any run exists, safe
+ *     run's host transfers overlap another run's kernels.  (What they share: device
+ *     memory that small bound runs gave back, at most 64 MB while any run exists, safe
  *     with several threads, streams and devices.)
  */
 #ifndef PRS_H

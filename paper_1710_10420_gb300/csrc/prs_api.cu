@@ -7,7 +7,6 @@
 #include <stdlib.h>
 #include <string.h>
 
-#include <atomic>
 #include <mutex>
 #include <new>
 
@@ -169,55 +168,62 @@ static void make_plan(prs_sim* s, int nruns)
     else march_plan_3d(s->g, nruns, &s->march);
 }
 
-// Bound runs of small boxes take their device memory from a pool where they are not the only run.  It keeps at
-// most kPoolBytes of what such runs gave back while any run exists, and nothing afterwards: from the driver
-// 10 MB take 90 us to get and 60 to return, from the pool 1 and 1, beside a first interval of 190 us at 128^3.
-// (The pool maps larger pieces slower than cudaMalloc does, 290 MB 200 us against 90, and giving its memory
-// back after each run of a program that has one at a time would take 50.)
-static const size_t kPoolBytes = (size_t)64 << 20, kPoolMost = (size_t)32 << 20;
-static std::atomic<int> g_runs{0};  // runs that exist
-static std::mutex g_pool_mutex;
-static cudaMemPool_t g_pool[64];  // by device
+// Device memory that bound runs of small boxes gave back, for the next such run: from the driver 10 MB take 90 us
+// to get and 60 to return, beside a first interval of 190 us at 128^3.  At most kKeptBytes of it while any
+// run exists, none afterwards.  (A pool of the driver's serves as fast but takes 2.2 ms to make.)  A piece
+// comes here when the stream of its run has passed all its work, and no caller ever held its address.
+static const size_t kKeptBytes = (size_t)64 << 20, kKeptMost = (size_t)32 << 20;
+struct Kept {
+    void* p;
+    size_t bytes;
+    int dev;
+};
+static std::mutex g_kept_mutex;  // of the three below
+static Kept g_kept[16];
+static size_t g_kept_bytes;
+static int g_runs;  // runs that exist
 
-// Memory of the current device's pool, or null.
-static void* pool_alloc(size_t bytes, cudaStream_t st)
+static int current_device()
 {
-    int dev = 0;
-    void* p = nullptr;
-    if (g_runs < 2 || bytes > kPoolMost || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    std::lock_guard<std::mutex> lock(g_pool_mutex);
-    if (!g_pool[dev]) {
-        cudaMemPoolProps props{};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        unsigned long long keep = kPoolBytes;
-        if (cudaMemPoolCreate(&g_pool[dev], &props) != cudaSuccess ||
-            cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-    }
-    if (cudaMallocFromPoolAsync(&p, bytes, g_pool[dev], st) == cudaSuccess) return p;
-    cudaGetLastError();
-    return nullptr;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
+    return dev;
 }
 
-static void free_run(prs_sim* s)
+// A kept piece of at least `bytes` and not much more on the current device, and its size; or null.
+static void* take_kept(size_t bytes, size_t* size)
 {
-    if (s->pooled) cudaFreeAsync(s->mem, s->stream);
-    else cudaFree(s->mem);
-    s->mem = nullptr;
+    const int dev = current_device();
+    std::lock_guard<std::mutex> lock(g_kept_mutex);
+    Kept* best = nullptr;
+    for (Kept& k : g_kept)
+        if (k.p && k.dev == dev && k.bytes >= bytes && k.bytes / 2 <= bytes && (!best || k.bytes < best->bytes))
+            best = &k;
+    if (!best) return nullptr;
+    void* p = best->p;
+    *size = best->bytes;
+    g_kept_bytes -= best->bytes;
+    *best = Kept{};
+    return p;
 }
 
-// A run less: the last one gives the pools' memory back (what it freed has been passed by its stream).
-static void run_gone()
+// A run comes (1) or goes (-1), its bound device memory with it (or null).
+static void count_run(int change, void* mem = nullptr, size_t bytes = 0)
 {
-    if (--g_runs > 0) return;
-    std::lock_guard<std::mutex> lock(g_pool_mutex);
-    for (cudaMemPool_t pool : g_pool)
-        if (pool && g_runs == 0) cudaMemPoolTrimTo(pool, 0);
-    cudaGetLastError();
+    const int dev = mem ? current_device() : -1;
+    std::lock_guard<std::mutex> lock(g_kept_mutex);
+    g_runs += change;
+    if (g_runs > 0 && mem && bytes <= kKeptMost && g_kept_bytes + bytes <= kKeptBytes)
+        for (Kept& k : g_kept)
+            if (!k.p) {
+                k = Kept{mem, bytes, dev};
+                g_kept_bytes += bytes;
+                return;
+            }
+    cudaFree(mem);
+    for (Kept& k : g_kept)
+        if (g_runs == 0 && k.p) cudaFree(k.p), k = Kept{};
+    if (g_runs == 0) g_kept_bytes = 0;
 }
 
 extern "C" int prs_create(const prs_params* params, void* stream, prs_sim** out)
@@ -247,7 +253,7 @@ extern "C" int prs_create(const prs_params* params, void* stream, prs_sim** out)
         delete s;
         return r;
     }
-    ++g_runs;
+    count_run(1);
     *out = s;
     return PRS_OK;
 }
@@ -271,13 +277,14 @@ static int alloc_run_on(prs_sim* s, int fields, const cudaStream_t* stream)
     const size_t fs = ((size_t)s->g.S * s->elem + 511) & ~(size_t)511;
     const size_t scratch = sizeof(DiagAcc) * kMeasureBlocks + sizeof(DevStatus);
     bool alt = wants_alt(s);
-    void* m = fields || !stream ? nullptr : pool_alloc(fs * (alt ? 1 : 0) + scratch, *stream);
-    s->pooled = m != nullptr;
-    if (!m && cudaMalloc(&m, fs * (size_t)(fields + (alt ? 1 : 0)) + scratch) != cudaSuccess) {
+    size_t bytes = fs * (size_t)(fields + (alt ? 1 : 0)) + scratch, size = 0;
+    void* m = fields ? nullptr : take_kept(bytes, &size);
+    if (!m && cudaMalloc(&m, bytes) != cudaSuccess) {
         cudaGetLastError();
         if (!alt) return PRS_ENOMEM;
         alt = false;
-        if (cudaMalloc(&m, fs * (size_t)fields + scratch) != cudaSuccess) {
+        bytes = fs * (size_t)fields + scratch;
+        if (cudaMalloc(&m, bytes) != cudaSuccess) {
             cudaGetLastError();
             return PRS_ENOMEM;
         }
@@ -285,11 +292,12 @@ static int alloc_run_on(prs_sim* s, int fields, const cudaStream_t* stream)
     char* c = (char*)m + fs * (size_t)(fields + (alt ? 1 : 0));
     cudaError_t e = cudaMemsetAsync(c, 0, scratch, stream ? *stream : cudaStreamPerThread);
     if (e == cudaSuccess && !stream) e = cudaStreamSynchronize(cudaStreamPerThread);
-    s->mem = m;
     if (e != cudaSuccess) {
-        free_run(s);
+        cudaFree(m);
         return cuda_fail(e, "scratch of the diagnostics");
     }
+    s->mem = m;
+    s->mem_bytes = size ? size : bytes;
     s->scr.partials = (DiagAcc*)c;
     s->d_status = (DevStatus*)(s->scr.partials + kMeasureBlocks);
     s->scr.result = &s->d_status->result;
@@ -366,15 +374,14 @@ extern "C" int prs_destroy(prs_sim* s)
     if (!s) return PRS_EINVAL;
     cudaStreamSynchronize(s->stream);
     for (int i = 0; i < 3; ++i) cudaFree(s->guard_base[i]);
-    free_run(s);
     cudaFree(s->alt_mem);
     cudaFree(s->d_dbg);
     cudaFree(s->adj_ws);
     for (cudaEvent_t e : s->adj_ev) cudaEventDestroy(e);
     cudaFreeHost(s->h_status);
-    if (s->pooled) cudaStreamSynchronize(s->stream);
+    if (s->owned) cudaFree(s->mem), s->mem = nullptr;
+    count_run(-1, s->mem, s->mem_bytes);
     delete s;
-    run_gone();
     return PRS_OK;
 }
 

@@ -25,7 +25,7 @@ struct prs_sim {
     bool waits;          // passes with bounded waits were queued since the error word was last read
     double rc[6];        // deta, 1/dx^2, 1/phi0^2, 2D, V0, phi0
     void* mem;           // library-owned fields (not with PRS_DEBUG), second dphi buffer, scratch
-    bool pooled;         // mem is from the pool of small bound runs
+    size_t mem_bytes;
     prs::DiagScratch scr;
     prs::MarchPlan march;     // FP32: the passes' shapes and times, for this run or a group it leads
     prs::DevStatus* d_status; // device: result, counter, error word

@@ -126,25 +126,11 @@ static cudaError_t get(const char* call, void** p, size_t n)
 }
 cudaError_t cudaMalloc(void** p, size_t n) { return get("malloc", p, n); }
 cudaError_t cudaMallocHost(void** p, size_t n) { return get("mallochost", p, n); }
-cudaError_t cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps*)
-{
-    const cudaError_t e = done("pool");
-    if (e == cudaSuccess) *p = (cudaMemPool_t)(0x1000000 + g_next++);
-    return e;
-}
-cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
-cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t, cudaStream_t) { return get("poolmalloc", p, n); }
-cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t n)
-{
-    say("trim %zu", n);
-    return cudaSuccess;
-}
 cudaError_t cudaFree(void* p)
 {
     if (p) say("free");
     return cudaFreeHost(p);
 }
-cudaError_t cudaFreeAsync(void* p, cudaStream_t) { return cudaFree(p); }
 cudaError_t cudaFreeHost(void* p)
 {
     if (p) munmap(p, g_sizes[p]), g_sizes.erase(p);

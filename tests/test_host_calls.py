@@ -176,7 +176,7 @@ def test_small_boxes_take_no_staged_pairs(lib, shape, steps):
 
 
 def _mallocs(lib):
-    return [int(line[1]) for line in _log(lib) if line[0] in ("malloc", "poolmalloc")]
+    return [int(line[1]) for line in _log(lib) if line[0] == "malloc"]
 
 
 @pytest.mark.parametrize("shape,kw", [((128, 128, 128), {}), ((250, 170), {}), ((256, 256), {}), ((45, 42, 38), {}),
@@ -292,22 +292,38 @@ def test_the_benchmark_counts_the_passes_the_library_takes(lib):
         assert lib.prs_destroy(h) == prs.PRS_OK
 
 
-def test_small_bound_runs_share_a_pool_that_the_last_one_gives_back(lib):
+def test_bound_runs_reuse_small_memory_while_runs_exist(lib):
+    """What a small bound run gives back serves the next one; the last run gives everything back, and 64 MB
+    and 16 pieces are the most that is kept."""
     bufs = [np.zeros((64, 64), np.float32) for _ in range(3)]
 
-    def bind(shape, **kw):
-        h = _run(lib, shape, **kw)
+    def bind(shape):
+        h = _run(lib, shape)
         assert lib.prs_bind(h, *[b.ctypes.data + -b.ctypes.data % 16 for b in bufs]) == prs.PRS_OK
         return h
 
-    lone, a, b, large = bind((64, 60)), bind((64, 60)), bind((100, 90, 80)), bind((512, 512, 40))
-    assert [line[0] for line in _log(lib) if line[0] in ("malloc", "poolmalloc")] == \
-        ["malloc", "poolmalloc", "poolmalloc", "malloc"]  # alone, small, small, 42 MB
-    for h, trims in ((a, 0), (lone, 0), (large, 0), (b, 1)):
-        assert lib.prs_destroy(h) == prs.PRS_OK
-        assert len([line for line in _log(lib) if line[0] == "trim"]) == trims
-    lib.fake_reset()
-    lib.fake_fail(b"poolmalloc", 1, 2)  # no room in the pool: the driver's memory
-    for h in (bind((64, 60)), bind((64, 60))):
-        assert lib.prs_destroy(h) == prs.PRS_OK
-    assert [line[0] for line in _log(lib) if line[0] in ("malloc", "poolmalloc")] == ["malloc", "malloc"]
+    def done(*runs):
+        for h in runs:
+            assert lib.prs_destroy(h) == prs.PRS_OK
+
+    def held():
+        return len(_mallocs(lib)) - len([line for line in _log(lib) if line[0] == "free"])
+
+    first, a = bind((64, 60)), bind((100, 90, 80))
+    done(a)
+    assert len(_mallocs(lib)) == 2 and held() == 2  # kept
+    b = bind((100, 90, 79))
+    assert len(_mallocs(lib)) == 2  # taken again
+    c, large = bind((100, 90, 80)), bind((512, 512, 40))
+    assert len(_mallocs(lib)) == 4
+    done(large)
+    assert held() == 3  # 42 MB go back
+    done(*[bind((64, 64)) for _ in range(3)], b, c)
+    assert held() == 1 + 3 + 2  # the first's; kept: three of 64 x 64, b's and c's
+    runs = [bind((180, 160, 160)) for _ in range(8)]  # 19 MB each
+    done(*runs)
+    assert held() == 6 + 3  # 64 MB are 67.1e6 bytes, of which 7.7e6 were kept before
+    done(first)
+    assert held() == 0
+    done(bind((64, 60)))
+    assert held() == 0
