@@ -190,10 +190,9 @@ static int current_device()
     return dev;
 }
 
-// A kept piece of at least `bytes` and not much more on the current device, and its size; or null.
-static void* take_kept(size_t bytes, size_t* size)
+// A kept piece of at least `bytes` and not much more on device dev, and its size; or null.
+static void* take_kept(size_t bytes, int dev, size_t* size)
 {
-    const int dev = current_device();
     std::lock_guard<std::mutex> lock(g_kept_mutex);
     Kept* best = nullptr;
     for (Kept& k : g_kept)
@@ -207,10 +206,9 @@ static void* take_kept(size_t bytes, size_t* size)
     return p;
 }
 
-// A run comes (1) or goes (-1), its bound device memory with it (or null).
-static void count_run(int change, void* mem = nullptr, size_t bytes = 0)
+// A run comes (1) or goes (-1), its bound device memory on device dev with it (or null).
+static void count_run(int change, void* mem = nullptr, size_t bytes = 0, int dev = -1)
 {
-    const int dev = mem ? current_device() : -1;
     std::lock_guard<std::mutex> lock(g_kept_mutex);
     g_runs += change;
     if (g_runs > 0 && mem && bytes <= kKeptMost && g_kept_bytes + bytes <= kKeptBytes)
@@ -278,7 +276,8 @@ static int alloc_run_on(prs_sim* s, int fields, const cudaStream_t* stream)
     const size_t scratch = sizeof(DiagAcc) * kMeasureBlocks + sizeof(DevStatus);
     bool alt = wants_alt(s);
     size_t bytes = fs * (size_t)(fields + (alt ? 1 : 0)) + scratch, size = 0;
-    void* m = fields ? nullptr : take_kept(bytes, &size);
+    const int dev = current_device();
+    void* m = fields ? nullptr : take_kept(bytes, dev, &size);
     if (!m && cudaMalloc(&m, bytes) != cudaSuccess) {
         cudaGetLastError();
         if (!alt) return PRS_ENOMEM;
@@ -298,6 +297,7 @@ static int alloc_run_on(prs_sim* s, int fields, const cudaStream_t* stream)
     }
     s->mem = m;
     s->mem_bytes = size ? size : bytes;
+    s->mem_dev = dev;
     s->scr.partials = (DiagAcc*)c;
     s->d_status = (DevStatus*)(s->scr.partials + kMeasureBlocks);
     s->scr.result = &s->d_status->result;
@@ -380,7 +380,7 @@ extern "C" int prs_destroy(prs_sim* s)
     for (cudaEvent_t e : s->adj_ev) cudaEventDestroy(e);
     cudaFreeHost(s->h_status);
     if (s->owned) cudaFree(s->mem), s->mem = nullptr;
-    count_run(-1, s->mem, s->mem_bytes);
+    count_run(-1, s->mem, s->mem_bytes, s->mem_dev);
     delete s;
     return PRS_OK;
 }

@@ -26,6 +26,7 @@ struct prs_sim {
     double rc[6];        // deta, 1/dx^2, 1/phi0^2, 2D, V0, phi0
     void* mem;           // library-owned fields (not with PRS_DEBUG), second dphi buffer, scratch
     size_t mem_bytes;
+    int mem_dev;         // the device it is on
     prs::DiagScratch scr;
     prs::MarchPlan march;     // FP32: the passes' shapes and times, for this run or a group it leads
     prs::DevStatus* d_status; // device: result, counter, error word

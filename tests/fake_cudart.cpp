@@ -63,6 +63,8 @@ void fake_fail(const char* call, int nth, int code)
     g_fail_call = call, g_fail_nth = nth, g_fail_code = (cudaError_t)code;
 }
 void fake_limit(size_t bytes) { g_limit = bytes; }
+static int g_device = 0;
+void fake_device(int device) { g_device = device; }
 
 // ------------------------------------------------------------ kernels
 void** __cudaRegisterFatBinary(void*)
@@ -204,7 +206,7 @@ cudaError_t cudaStreamWaitEvent(cudaStream_t st, cudaEvent_t v, unsigned)
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { return *ms = 1.0f, cudaSuccess; }
 
 // -------------------------------------------------------------- others
-cudaError_t cudaGetDevice(int* d) { return *d = 0, cudaSuccess; }
+cudaError_t cudaGetDevice(int* d) { return *d = g_device, cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
 static int encode_nothing() { return 0; }  // the tensor-map encoder
 cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** f, unsigned, unsigned long long,

@@ -327,3 +327,26 @@ def test_bound_runs_reuse_small_memory_while_runs_exist(lib):
     assert held() == 0
     done(bind((64, 60)))
     assert held() == 0
+
+
+def test_kept_memory_stays_with_its_device(lib):
+    bufs = [np.zeros((64, 64), np.float32) for _ in range(3)]
+
+    def bind(device):
+        lib.fake_device(device)
+        h = _run(lib, (64, 60))
+        assert lib.prs_bind(h, *[b.ctypes.data + -b.ctypes.data % 16 for b in bufs]) == prs.PRS_OK
+        return h
+
+    try:
+        first, a = bind(0), bind(0)
+        lib.fake_device(1)
+        assert lib.prs_destroy(a) == prs.PRS_OK  # made on device 0, released with device 1 current
+        b = bind(1)
+        assert len(_mallocs(lib)) == 3
+        c = bind(0)
+        assert len(_mallocs(lib)) == 3
+        for h in (first, b, c):
+            assert lib.prs_destroy(h) == prs.PRS_OK
+    finally:
+        lib.fake_device(0)
